@@ -166,11 +166,14 @@ def _graph(case, seed):
         for _ in range(40):
             mid = 0.5 * (lo + hi)
             lo, hi = (mid, hi) if float(torch.clamp(w * mid, max=cap).mean()) < case["degree"] else (lo, mid)
-        cum = torch.cumsum(torch.clamp(w * hi, max=cap), 0)
+        # weights as whole numbers: a prefix sum of doubles on the GPU does not add in a fixed order,
+        # and the same seed has to give the same graph
+        cum = torch.cumsum((torch.clamp(w * hi, max=cap) * (1 << 20)).to(torch.int64), 0)
         count = int(n * case["degree"] / 2)
         ends = []
         for _ in range(2):
-            x = torch.rand(count, generator=gen, device=DEV, dtype=torch.float64) * cum[-1]
+            x = torch.rand(count, generator=gen, device=DEV, dtype=torch.float64) * cum[-1].double()
+            x = x.to(torch.int64)
             ends.append(torch.clamp(torch.searchsorted(cum, x, right=True), max=n - 1))
         perm = torch.randperm(n, generator=gen, device=DEV)
         src, dst = perm[ends[0]], perm[ends[1]]
