@@ -194,8 +194,9 @@ typedef struct {
     uint32_t warps_per_cta;  /* in: warps per bitmap-path block, 1..32 (0: 32); fewer are used
                                 when the block's shared memory would not fit */
     uint32_t flags;          /* in: CITRON_COUNT_* bits */
-    uint32_t compact_max;    /* in: candidate sets of the bitmap path with at most this many
-                                members are re-encoded as compact bitmaps: 0 or 128 mean 128,
+    uint32_t compact_max;    /* in: candidate sets of the bitmap path are re-encoded as compact
+                                bitmaps, and dense ones counted on their complement: 0 or 128 mean
+                                sets of at most 128 members by one warp and wider ones by several,
                                 1 means never */
     uint32_t max_blocks;     /* in: cap on the blocks of each counting launch, so that work on
                                 other streams keeps some SMs (0: no cap) */
@@ -204,8 +205,7 @@ typedef struct {
     float kernel_ms[3];      /* out: device ms of the warp-register, bitmap, sorted-list kernels */
     uint32_t split_min;      /* in: for k >= 6, bitmap-path roots of at least this out-degree
                                 share their work with idle blocks (heavy-edge splitting,
-                                Sec. VII-C): their edge tasks, and the sub-tasks (u, a_t, b) of
-                                rows above 128 members, are taken from a global cursor, which
+                                Sec. VII-C): their edge tasks are taken from global cursors, which
                                 blocks that find the root queue empty join after rebuilding the
                                 root's subgraph.  0: default (384); 1: never; else the threshold */
     float busy_ms[2];        /* out (CITRON_COUNT_BALANCE): bitmap kernel's span from the first

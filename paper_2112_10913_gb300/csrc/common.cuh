@@ -233,14 +233,15 @@ struct RootSink {
     __device__ __forceinline__ bool wants_root_total() const { return per_root || group_counts; }
 };
 
-// A heavy root whose units (edge tasks, or edge sub-tasks (u, a_t, b)) any block may take: the
-// block that took the root from the queue publishes it here; blocks that find the root queue
-// empty rebuild its local subgraph and take units from the same cursor.
+// A heavy root whose units (its edge tasks, i.e. the rows of its local subgraph) any block may
+// take: the block that took the root from the queue publishes it here; blocks that find the root
+// queue empty rebuild its local subgraph and take units from the same cursors.
 struct HeavySlot {
-    uint32_t u;       // the root
-    uint32_t units;   // size of its unit space
-    uint32_t cursor;  // next unit to take (may run past `units`)
-    uint32_t ready;   // 1 once u and units are published
+    uint32_t u;            // the root
+    uint32_t units;        // bit 31 once u is published; its rows by class: 10 bits of wide rows
+                           // for large groups, 10 of those for two warps, 11 of the others
+    uint32_t wide_cursor;  // next wide row to take of the first (low half) and second class, and ...
+    uint32_t cursor;       // ... next other row (all may run past the end)
 };
 
 struct HelpTable {

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "dense.cuh"
 
 namespace citron {
 
@@ -150,22 +151,17 @@ struct WarpCtx {
     uint32_t *lbuf;
     uint32_t *mv;    // compress masks: 5 per candidate word, then the member prefix per word
     uint32_t *mbuf;  // compact rows, 4 words each (16-byte aligned); aliases lbuf
-    uint32_t compact_max;  // largest candidate set re-encoded compactly (0 or 128)
-    uint32_t compact3_max; // same for the R = 3 level, which also takes packed 5- and 6-word rows
+    uint32_t compact_max;  // largest candidate set re-encoded compactly by one warp (0 or 128)
     uint32_t pair_cap;     // uint16 entries of elem
+    uint32_t *err;
 };
 
-// Carry-save accumulation of bit counts (a full adder per bit position): the bits of
-// ones + a + b are kept as a new `ones` word and a carry word of weight two (two LOP3s), so that
-// one POPC counts two words.  POPC and the bit scans share the narrow XU pipe, which bounds the
-// leaves; the LOP3s go to the wider ALU pipe.  The running total is s + popc(ones): every user
-// adds popc(ones) once at the end.
-__device__ __forceinline__ void csa_add(uint32_t &ones, uint32_t a, uint32_t b, uint32_t &s)
+// One lane's running count plus a set's total (the sum of the lanes is checked by warp_sum_u64).
+__device__ __forceinline__ void add_acc(unsigned long long &acc, unsigned long long n, uint32_t *err)
 {
-    const uint32_t u = ones ^ a;
-    const uint32_t carry = (ones & a) | (u & b);
-    ones = u ^ b;
-    s += 2u * (uint32_t)__popc(carry);
+    const unsigned long long t = acc + n;
+    if (t < acc) set_error(err, kDevOverflow);
+    acc = t;
 }
 
 // Number of DAG arcs inside the lane's own candidate set lb (words [lo, hi)): the penultimate
@@ -204,20 +200,19 @@ __device__ __forceinline__ uint32_t lane_arcs(const WarpCtx &x, const uint32_t *
 }
 
 // Writes the candidate set (lane word c) to cbuf and its member indices to elem; returns the
-// member count and the range [clo, chi) of its non-zero words.
+// member count and the range [clo, chi) of its non-zero words.  The members are listed one word at
+// a time, lane l taking bit l: a lane that lists its own word takes up to 32 steps.
 __device__ __forceinline__ uint32_t compact(const WarpCtx &x, uint32_t c, int lane, int &clo, int &chi)
 {
-    const uint32_t pc = __popc(c);
-    const uint32_t incl = warp_incl_scan(pc);
-    const uint32_t total = __shfl_sync(kFull, incl, 31);
-    uint32_t pos = incl - pc;
     if (lane < (int)x.W) x.cbuf[lane] = c;
-    uint32_t y = c;
-    while (y) {
-        x.elem[pos++] = (uint16_t)((lane << 5) + __ffs(y) - 1);
-        y &= y - 1;
-    }
     const uint32_t nz = __ballot_sync(kFull, c != 0);
+    uint32_t total = 0;
+    for (uint32_t r = nz; r; r &= r - 1) {
+        const int w = __ffs(r) - 1;
+        const uint32_t m = __shfl_sync(kFull, c, w);
+        if ((m >> lane) & 1u) x.elem[total + __popc(m & lanemask_lt())] = (uint16_t)((w << 5) + lane);
+        total += __popc(m);
+    }
     clo = nz ? __ffs(nz) - 1 : 0;
     chi = nz ? 32 - __clz(nz) : 0;
     __syncwarp();
@@ -257,109 +252,84 @@ __device__ __forceinline__ uint32_t tri_rounds(const WarpCtx &x, const uint32_t 
     return s + __popc(ones);
 }
 
-// ---- Compact re-encoding of a small candidate set ------------------------------------------
-// A candidate set with s <= 128 members (listed in elem) is re-encoded as the s x s adjacency of
-// its induced sub-DAG: row i = the members j that are out-neighbours of member i, packed into
-// CW = ceil(s/32) <= 4 words ("compact rows"; upper-triangular when the DAG is relabelled to its
-// order).  The remaining levels of the recursion then work on at most 4 words per set instead
-// of the root-wide span; a row is one 16-byte shared-memory load.  At R = 3, sets of 129..192
-// members take packed rows of 5 or 6 words (below); wider sets stay on the root-wide bitmap
-// (full 8-word rows for every level were measured slower on R-MAT 20).
+// ---- Compact re-encoding of a candidate set ------------------------------------------------
+// A candidate set with s members (listed in elem) is re-encoded as the s x s adjacency of its
+// induced subgraph: bit j of row i is member j, so that the remaining levels work on ceil(s/32)
+// words per set instead of the root-wide span.  What is stored is the COMPLEMENT, symmetric (the
+// members j that are not adjacent to member i): dense sets are counted on it (dense.cuh); a set
+// with more than half of its pairs missing is turned back into upper-triangular adjacency rows
+// and enumerated (cdfs below).  Sets of at most 128 members are handled by one warp (one 16-byte
+// load per row), wider ones by a group of warps (wide_row).
 //
-// Bits are gathered word by word with the parallel-suffix "compress" of H. S. Warren, Hacker's
-// Delight (2nd ed., Sec. 7-4): for a mask m the five move masks depend on m only, so they are
-// computed once per candidate word (lane-parallel) and shared by every row.
-__device__ __forceinline__ void compress_masks(uint32_t m, uint32_t mv[5])
+// Compress masks and member prefix of every candidate word (lane w: word w), for the builders.
+__device__ __forceinline__ void prepare_masks(const WarpCtx &x, int clo, int chi, int lane)
 {
-    uint32_t mk = ~m << 1;
+    const uint32_t m = (lane < chi && lane >= clo) ? x.cbuf[lane] : 0u;
+    uint32_t mv[5];
+    compress_masks(m, mv);
+    const uint32_t pc = __popc(m);
+    const uint32_t pre = warp_incl_scan(pc) - pc;
 #pragma unroll
-    for (int i = 0; i < 5; i++) {
-        uint32_t mp = mk ^ (mk << 1);
-        mp ^= mp << 2;
-        mp ^= mp << 4;
-        mp ^= mp << 8;
-        mp ^= mp << 16;
-        const uint32_t v = mp & m;
-        mv[i] = v;
-        m = (m ^ v) | (v >> (1 << i));
-        mk &= ~mp;
-    }
-}
-
-__device__ __forceinline__ uint32_t compress_with(uint32_t x, uint32_t m, const uint32_t *mv)
-{
-    x &= m;
-#pragma unroll
-    for (int i = 0; i < 5; i++) {
-        const uint32_t t = x & mv[i];
-        x = (x ^ t) | (t >> (1 << i));
-    }
-    return x;
-}
-
-// o[q] |= lo, o[q + 1] |= hi for a warp-uniform q (the member prefix of a candidate word is the
-// same on every lane): a uniform branch instead of a select per output word.
-template <int NW>
-__device__ __forceinline__ void place_piece(uint32_t (&o)[NW], uint32_t q, uint32_t lo, uint32_t hi)
-{
-#pragma unroll
-    for (int t = 0; t < NW; t++) {
-        if (q == (uint32_t)t) {
-            o[t] |= lo;
-            if (t + 1 < NW) o[t + 1] |= hi;
-        }
-    }
-}
-
-// Builds the compact rows of the s members of the candidate set (words in cbuf, members in
-// elem, non-zero words [clo, chi)).  NW = 4 output words per row (one uint4) is the width in
-// use; NW = 8 (two uint4 per row) is also supported.
-template <int NW>
-__device__ __forceinline__ void build_compact(const WarpCtx &x, uint32_t s, int clo, int chi, int lane)
-{
-    // per candidate word w (lane w): compress masks and the number of members before word w
-    {
-        const uint32_t m = (lane < chi && lane >= clo) ? x.cbuf[lane] : 0u;
-        uint32_t mv[5];
-        compress_masks(m, mv);
-        const uint32_t pc = __popc(m);
-        const uint32_t pre = warp_incl_scan(pc) - pc;
-#pragma unroll
-        for (int i = 0; i < 5; i++) x.mv[i * 32 + lane] = mv[i];
-        x.mv[160 + lane] = pre;
-    }
+    for (int i = 0; i < 5; i++) x.mv[i * 32 + lane] = mv[i];
+    x.mv[160 + lane] = pre;
     __syncwarp();
-    uint4 *out = reinterpret_cast<uint4 *>(x.mbuf);
-    for (uint32_t i0 = 0; i0 < s; i0 += 32) {
-        const uint32_t i = i0 + lane;
-        const bool act = i < s;
-        const uint32_t ei = act ? x.elem[i] : x.elem[i0];
-        const uint32_t *row = x.rows + ei * x.RS;
-        uint32_t o[NW];
+}
+
+// The bits of row word `bits` at the members of candidate word w (mask m), packed to the low end.
+__device__ __forceinline__ uint32_t member_bits(const WarpCtx &x, uint32_t bits, uint32_t m, int w)
+{
+    uint32_t mv[5];
 #pragma unroll
-        for (int t = 0; t < NW; t++) o[t] = 0;
-        // triangular rows hold bits above their own member only: start at the word of the
-        // round's first member
-        for (int w = x.tri ? (int)(x.elem[i0] >> 5) : clo; w < chi; w++) {
+    for (int t = 0; t < 5; t++) mv[t] = x.mv[t * 32 + w];
+    return compress_with(bits, m, mv);
+}
+
+// Complement rows of the s <= 128 members of the candidate set (words in cbuf, members in elem,
+// non-zero words [clo, chi); triangular layout) in mbuf, one uint4 per row.  Each round of 32
+// members streams its packed row words: the member prefix of a candidate word is the same on every
+// lane, so the words fill and leave at warp-uniform places.  Returns the complement's bits written
+// by this lane (in all, twice its edges).
+__device__ __forceinline__ uint32_t build_complement(const WarpCtx &x, uint32_t s, int clo, int chi, int lane)
+{
+    prepare_masks(x, clo, chi, lane);
+    const uint32_t nblk = (s + 31) >> 5;
+    uint32_t bits = 0;
+    for (uint32_t a = 0; a < nblk; a++) {
+        const uint32_t i0 = a << 5, i = i0 + lane;
+        const uint32_t *row = x.rows + (uint32_t)x.elem[i < s ? i : s - 1] * x.RS;
+        // rows hold bits above their own member only: start at the word of the first member
+        int w = (int)(x.elem[i0] >> 5);
+        uint32_t ow = x.mv[160 + w] >> 5, sh = x.mv[160 + w] & 31u, cur = 0;
+        for (; w < chi; w++) {
             const uint32_t m = x.cbuf[w];
             if (!m) continue;
-            uint32_t mv[5];
-#pragma unroll
-            for (int t = 0; t < 5; t++) mv[t] = x.mv[t * 32 + w];
-            const uint32_t pre = x.mv[160 + w];
-            const uint32_t piece = compress_with(row[w], m, mv);
-            const uint32_t q = pre >> 5, sh = pre & 31;
-            const uint32_t lo = piece << sh, hi = sh ? (piece >> (32 - sh)) : 0u;
-            place_piece<NW>(o, q, lo, hi);
-        }
-        if (act) {
-            if (NW == 4) {
-                out[i] = make_uint4(o[0], o[1], o[2], o[3]);
-            } else {
-                out[2 * i] = make_uint4(o[0], o[1], o[2], o[3]);
-                out[2 * i + 1] = make_uint4(o[4 % NW], o[5 % NW], o[6 % NW], o[7 % NW]);
+            const uint32_t piece = member_bits(x, row[w], m, w);
+            cur |= piece << sh;
+            const uint32_t end = sh + __popc(m);
+            if (end >= 32) {
+                if (ow >= a) bits += put_block(x.mbuf, 0, s, a, ow, cur, lane);
+                ow++;
+                cur = sh ? piece >> (32 - sh) : 0u;
             }
+            sh = end & 31u;
         }
+        if (sh && ow >= a) bits += put_block(x.mbuf, 0, s, a, ow, cur, lane);
+    }
+    __syncwarp();
+    return bits;
+}
+
+// mbuf from complement rows to upper-triangular adjacency rows of the s <= 128 members.
+__device__ __forceinline__ void complement_to_rows(const WarpCtx &x, uint32_t s, int lane)
+{
+    uint4 *M = reinterpret_cast<uint4 *>(x.mbuf);
+    for (uint32_t i = lane; i < s; i += 32) {
+        const uint4 h = M[i];
+        uint32_t g[4] = {~h.x, ~h.y, ~h.z, ~h.w};
+#pragma unroll
+        for (uint32_t t = 0; t < 4; t++)
+            g[t] &= word_mask(s, t) & (t > (i >> 5) ? kFull : (t == (i >> 5) ? above_bit(i & 31u) : 0u));
+        M[i] = make_uint4(g[0], g[1], g[2], g[3]);
     }
     __syncwarp();
 }
@@ -380,124 +350,6 @@ __device__ __forceinline__ void drop_top(uint32_t (&Y)[CW])
     }
 }
 
-// Packed triangular compact rows for R = 3 sets of 129..192 members (CW = 5 or 6 words): the row
-// of member i holds only its words q = i/32 .. CW-1 (the words below are zero in an
-// upper-triangular sub-DAG), so 192 rows take 672 words instead of 1152 and fit the warp's
-// scratch.  Rows of the members of word q start at packed_base(q) and are (CW - q) words long.
-template <int CW>
-__host__ __device__ constexpr uint32_t packed_base(int q)
-{
-    return q <= 0 ? 0u : packed_base<CW>(q - 1) + 32u * (uint32_t)(CW - (q - 1));
-}
-
-__host__ __device__ constexpr uint32_t packed_words(int cw) { return 16u * (uint32_t)(cw * (cw + 1)); }
-
-template <int CW>
-__device__ __forceinline__ void build_packed(const WarpCtx &x, uint32_t s, int clo, int chi, int lane)
-{
-    {
-        const uint32_t m = (lane < chi && lane >= clo) ? x.cbuf[lane] : 0u;
-        uint32_t mv[5];
-        compress_masks(m, mv);
-        const uint32_t pc = __popc(m);
-        const uint32_t pre = warp_incl_scan(pc) - pc;
-#pragma unroll
-        for (int i = 0; i < 5; i++) x.mv[i * 32 + lane] = mv[i];
-        x.mv[160 + lane] = pre;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int q = 0; q < CW; q++) {
-        const uint32_t i0 = (uint32_t)q * 32;
-        if (i0 >= s) break;
-        const uint32_t i = i0 + lane;
-        const bool act = i < s;
-        const uint32_t ei = act ? x.elem[i] : x.elem[i0];
-        const uint32_t *row = x.rows + ei * x.RS;
-        uint32_t o[CW];
-#pragma unroll
-        for (int t = 0; t < CW; t++) o[t] = 0;
-        for (int w = (int)(x.elem[i0] >> 5); w < chi; w++) {
-            const uint32_t m = x.cbuf[w];
-            if (!m) continue;
-            uint32_t mv[5];
-#pragma unroll
-            for (int t = 0; t < 5; t++) mv[t] = x.mv[t * 32 + w];
-            const uint32_t pre = x.mv[160 + w];
-            const uint32_t piece = compress_with(row[w], m, mv);
-            const uint32_t qq = pre >> 5, sh = pre & 31;
-            const uint32_t lo = piece << sh, hi = sh ? (piece >> (32 - sh)) : 0u;
-            place_piece<CW>(o, qq, lo, hi);
-        }
-        if (act) {
-            uint32_t *dst = x.mbuf + packed_base<CW>(q) + (uint32_t)lane * (CW - q);
-#pragma unroll
-            for (int t = q; t < CW; t++) dst[t - q] = o[t];
-        }
-    }
-    __syncwarp();
-}
-
-// Arcs inside the lane's set D (CW words; zero below word Q2) on packed rows; Y = the members
-// to visit (D without its highest member).
-template <int CW, bool WORK, int Q2>
-__device__ __forceinline__ void packed_leaf(const uint32_t *P, const uint32_t (&D)[CW],
-                                            const uint32_t (&Y)[CW], uint32_t &ones, uint32_t &s,
-                                            unsigned long long &work)
-{
-    if constexpr (Q2 < CW) {
-        uint32_t y = Y[Q2];
-        if (WORK) work += (unsigned long long)__popc(y) * (CW - Q2);
-        // two members per step (the highest and the lowest), their words paired in the adder
-        while (y & (y - 1u)) {
-            const uint32_t j1 = 31u - __clz(y);
-            const uint32_t lb = y & (0u - y);
-            const uint32_t j2 = 31u - __clz(lb);
-            y ^= (1u << j1) | lb;
-            const uint32_t *r1 = P + packed_base<CW>(Q2) + j1 * (CW - Q2);
-            const uint32_t *r2 = P + packed_base<CW>(Q2) + j2 * (CW - Q2);
-#pragma unroll
-            for (int w = Q2; w < CW; w++) csa_add(ones, D[w] & r1[w - Q2], D[w] & r2[w - Q2], s);
-        }
-        if (y) {
-            const uint32_t *rj = P + packed_base<CW>(Q2) + (31u - __clz(y)) * (CW - Q2);
-#pragma unroll
-            for (int w = Q2; w + 1 < CW; w += 2) csa_add(ones, D[w] & rj[w - Q2], D[w + 1] & rj[w + 1 - Q2], s);
-            if ((CW - Q2) & 1) s += __popc(D[CW - 1] & rj[CW - 1 - Q2]);
-        }
-        packed_leaf<CW, WORK, Q2 + 1>(P, D, Y, ones, s, work);
-    }
-}
-
-// Triangles of a dense compact set of s members (members 0..s-1) on packed rows: lane l takes
-// member 32q + l of each word q, forms D = C ∧ row and adds the arcs inside D.
-template <int CW, bool WORK, int Q>
-__device__ __forceinline__ void packed_r3(const uint32_t *P, uint32_t s_members, int lane,
-                                          uint32_t &s, unsigned long long &work)
-{
-    if constexpr (Q < CW) {
-        const uint32_t m = (uint32_t)Q * 32 + lane;
-        if (m < s_members) {
-            const uint32_t *rm = P + packed_base<CW>(Q) + (uint32_t)lane * (CW - Q);
-            uint32_t D[CW];
-#pragma unroll
-            for (int w = 0; w < CW; w++) {
-                const uint32_t cw = (uint32_t)w * 32 >= s_members ? 0u
-                                    : (s_members >= (uint32_t)w * 32 + 32 ? kFull : ((1u << (s_members - w * 32)) - 1));
-                D[w] = w < Q ? 0u : (cw & rm[w - Q]);
-            }
-            uint32_t Y[CW];
-#pragma unroll
-            for (int w = 0; w < CW; w++) Y[w] = D[w];
-            drop_top<CW>(Y);
-            uint32_t ones = 0, t = 0;
-            packed_leaf<CW, WORK, Q>(P, D, Y, ones, t, work);
-            s += t + __popc(ones);
-        }
-        packed_r3<CW, WORK, Q + 1>(P, s_members, lane, s, work);
-    }
-}
-
 // Sum of popc(a[w] & b[w]) over words w in [FROM, CW).
 template <int CW, int FROM>
 __device__ __forceinline__ uint32_t popc_and(const uint32_t (&a)[CW], const uint4 &b)
@@ -508,50 +360,6 @@ __device__ __forceinline__ uint32_t popc_and(const uint32_t (&a)[CW], const uint
     if (CW > 2 && FROM <= 2) s += __popc(a[2] & b.z);
     if (CW > 3 && FROM <= 3) s += __popc(a[3] & b.w);
     return s;
-}
-
-// popc_and with carry-save pairs: words [FROM, CW) of a & b, two at a time.
-template <int CW, int FROM>
-__device__ __forceinline__ void popc_and_csa(const uint32_t (&a)[CW], const uint4 &b, uint32_t &ones, uint32_t &s)
-{
-    const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
-    int w = FROM;
-#pragma unroll
-    for (int p = 0; p < 2; p++) {
-        if (w + 1 < CW) {
-            csa_add(ones, a[w] & bw[w], a[w + 1] & bw[w + 1], s);
-            w += 2;
-        }
-    }
-    if (w < CW) s += __popc(a[w] & bw[w]);
-}
-
-// Two leaf members at once: words [FROM, CW) of D & b1 and of D & b2 paired in the carry-save
-// adder (one POPC per word pair).
-template <int CW, int FROM>
-__device__ __forceinline__ void popc_and_csa2(const uint32_t (&a)[CW], const uint4 &b1, const uint4 &b2,
-                                              uint32_t &ones, uint32_t &s)
-{
-    const uint32_t v1[4] = {b1.x, b1.y, b1.z, b1.w}, v2[4] = {b2.x, b2.y, b2.z, b2.w};
-#pragma unroll
-    for (int w = FROM; w < CW; w++) csa_add(ones, a[w] & v1[w], a[w] & v2[w], s);
-}
-
-// Arcs from the members y of word q2 (FROM = q2 on triangular rows, else 0) into D, on compact
-// rows M: two members per step, the highest and the lowest, whose bit scans and row loads are
-// independent of each other.
-template <int CW, int FROM>
-__device__ __forceinline__ void leaf_word(const uint4 *M, const uint32_t (&D)[CW], uint32_t y, uint32_t base,
-                                          uint32_t &ones, uint32_t &s)
-{
-    while (y & (y - 1u)) {
-        const uint32_t b1 = 31u - __clz(y);
-        const uint32_t lb = y & (0u - y);
-        const uint32_t b2 = 31u - __clz(lb);
-        y ^= (1u << b1) | lb;
-        popc_and_csa2<CW, FROM>(D, M[base + b1], M[base + b2], ones, s);
-    }
-    if (y) popc_and_csa<CW, FROM>(D, M[base + 31u - __clz(y)], ones, s);
 }
 
 template <int CW, bool TRI>
@@ -768,37 +576,155 @@ __device__ __forceinline__ void cdfs_all(const WarpCtx &x, uint32_t s, int lane,
     else cdfs<R, CW, TRI, WORK>(x, C, lane, acc, work);
 }
 
+// A compact set's complement rows (chunk-major, dense.cuh): S rows per chunk, nch chunks.
+struct CompSet {
+    uint32_t *m32;
+    uint32_t S, nch;
+};
+
+// Lane word of (set c) ∧ (members adjacent to b, above b); c has its words on the lanes below 4 nch.
+__device__ __forceinline__ uint32_t adjacent_above(const CompSet &cs, uint32_t c, uint32_t b, int lane)
+{
+    if ((uint32_t)lane < (b >> 5) || (uint32_t)lane >= cs.nch * 4) return 0u;
+    const uint32_t r = c & ~comp_word(cs.m32, cs.S, b, lane);
+    return (uint32_t)lane == (b >> 5) ? r & above_bit(b & 31u) : r;
+}
+
+// R-cliques (R >= 4) of the compact set c (lane word) on complement rows: warp-uniform walk over
+// the members down to R = 4, which is counted in one step.  CW: words of the sets (1..4), or 0 for
+// a wide set.  Totals are added on lane 0.
+template <int R, int CW, bool WORK>
+__device__ __forceinline__ void dense_dfs(const WarpCtx &x, const CompSet &cs, uint32_t c, uint32_t cnt, int lane,
+                                          unsigned long long &acc, unsigned long long &work)
+{
+    if constexpr (R == 4) {
+        uint32_t *Bs = x.cbuf;
+        __syncwarp();
+        Bs[lane] = c;
+        __syncwarp();
+        const uint4 *M = reinterpret_cast<const uint4 *>(cs.m32);
+        if constexpr (CW > 0) {
+            const CompCount o = comp4<CW, WORK>(M, Bs, cnt, x.mv, lane);
+            if (lane == 0) add_acc(acc, o.n, x.err);
+            if (WORK && lane == 0) work += o.work;
+        } else {
+            const uint32_t ng = 32 - __clz(__ballot_sync(kFull, c != 0));
+            CompSums o = comp4_wide<WORK>(M, cs.S, cs.nch, Bs, cnt, ng, 0, 1, x.mv, lane);
+            if (WORK) work += o.work;
+            unsigned long long n = 0;
+            if (__any_sync(kFull, o.over)) {
+                // a complement degree beyond the planes: one level further down
+                for (uint32_t b = 0; b < ng * 32; b++) {
+                    if (!((__shfl_sync(kFull, c, b >> 5) >> (b & 31u)) & 1u)) continue;
+                    const uint32_t nc = adjacent_above(cs, c, b, lane);
+                    const uint32_t m = __reduce_add_sync(kFull, __popc(nc));
+                    if (m < 3) continue;
+                    __syncwarp();
+                    Bs[lane] = nc;
+                    __syncwarp();
+                    const CompCount t = comp3_wide<WORK>(M, cs.S, cs.nch, Bs, m, ng, 0, 1, lane);
+                    if (WORK) work += t.work;
+                    n += n3_finish(m, __reduce_add_sync(kFull, t.n));
+                }
+            } else {
+                unsigned long long sl = o.sl;
+#pragma unroll
+                for (int k = 16; k > 0; k >>= 1) sl += __shfl_xor_sync(kFull, sl, k);
+                n = n4_finish(cnt, __reduce_add_sync(kFull, o.sd), __reduce_add_sync(kFull, o.st), sl);
+            }
+            if (lane == 0) add_acc(acc, n, x.err);
+        }
+    } else {
+        uint32_t rem = c;
+        for (;;) {
+            const uint32_t nz = __ballot_sync(kFull, rem != 0);
+            if (!nz) break;
+            const int wl = __ffs(nz) - 1;
+            const uint32_t word = __shfl_sync(kFull, rem, wl);
+            const uint32_t b = wl * 32 + __ffs(word) - 1;
+            if (lane == wl) rem &= rem - 1;
+            const uint32_t nc = adjacent_above(cs, c, b, lane);
+            if (WORK && (uint32_t)lane < cs.nch * 4) work += 1;
+            const uint32_t m = __reduce_add_sync(kFull, __popc(nc));
+            if (m >= R - 1) dense_dfs<R - 1, CW, WORK>(x, cs, nc, m, lane, acc, work);
+        }
+    }
+}
+
+// C(s, R) for s <= 128 and R <= 11 (below 2^51).
+template <int R>
+__device__ __forceinline__ unsigned long long choose(uint32_t s)
+{
+    unsigned long long v = 1;
+#pragma unroll
+    for (uint32_t i = 0; i < (uint32_t)R; i++) v = v * (s - i) / (i + 1);
+    return v;
+}
+
+struct LaneSums {
+    unsigned long long acc, work;
+};
+
+// A set with more than half of its pairs missing: its rows are turned back and enumerated.  Out of
+// line: sets of an edge task are seldom sparse, and the code would push the others' out of the
+// instruction cache.
+template <int R, int CW, bool WORK>
+__device__ __noinline__ LaneSums sparse_count(const WarpCtx x, uint32_t s, int lane)
+{
+    LaneSums o = {0, 0};
+    complement_to_rows(x, s, lane);
+    cdfs_all<R, CW, true, WORK>(x, s, lane, o.acc, o.work);
+    return o;
+}
+
+// Counts a set of s members with CW words: its complement rows are in mbuf.
+template <int R, int CW, bool WORK>
+__device__ __forceinline__ void compact_count(const WarpCtx &x, uint32_t s, bool dense, int lane,
+                                              unsigned long long &acc, unsigned long long &work)
+{
+    if (!dense) {
+        const LaneSums o = sparse_count<R, CW, WORK>(x, s, lane);
+        acc += o.acc;
+        if (WORK) work += o.work;
+    } else if constexpr (R == 3) {
+        x.cbuf[lane] = word_mask(s, lane);
+        __syncwarp();
+        const CompCount o = comp3<CW, WORK>(reinterpret_cast<const uint4 *>(x.mbuf), x.cbuf, s, lane);
+        if (lane == 0) add_acc(acc, o.n, x.err);
+        if (WORK && lane == 0) work += o.work;
+    } else {
+        const CompSet cs = {x.mbuf, 0, 1};
+        dense_dfs<R, CW, WORK>(x, cs, word_mask(s, lane), s, lane, acc, work);
+    }
+}
+
 // Entry for a candidate set of at most compact_max members (lane word c), triangular layout.
+// The complement is worked when it has at most half of the pairs: its levels cost its edges, the
+// enumeration's cost the adjacent pairs.
 template <int R, bool WORK>
 __device__ __forceinline__ void compact_entry(const WarpCtx &x, uint32_t c, int lane,
                                               unsigned long long &acc, unsigned long long &work)
 {
     int clo, chi;
     const uint32_t s = compact(x, c, lane, clo, chi);
-    if (s <= 128) {
-        build_compact<4>(x, s, clo, chi, lane);
-        if (s <= 32) cdfs_all<R, 1, true, WORK>(x, s, lane, acc, work);
-        else if (s <= 64) cdfs_all<R, 2, true, WORK>(x, s, lane, acc, work);
-        else if (s <= 96) cdfs_all<R, 3, true, WORK>(x, s, lane, acc, work);
-        else cdfs_all<R, 4, true, WORK>(x, s, lane, acc, work);
-    } else if constexpr (R == 3) {
-        uint32_t t = 0;
-        if (s <= 160) {
-            build_packed<5>(x, s, clo, chi, lane);
-            packed_r3<5, WORK, 0>(x.mbuf, s, lane, t, work);
+    if (s >= (uint32_t)R) {
+        const uint32_t twice = __reduce_add_sync(kFull, build_complement(x, s, clo, chi, lane));
+        if (twice == 0) {  // a clique
+            if (lane == 0) add_acc(acc, choose<R>(s), x.err);
         } else {
-            build_packed<6>(x, s, clo, chi, lane);
-            packed_r3<6, WORK, 0>(x.mbuf, s, lane, t, work);
+            const bool dense = 2 * twice <= s * (s - 1);
+            if (s <= 32) compact_count<R, 1, WORK>(x, s, dense, lane, acc, work);
+            else if (s <= 64) compact_count<R, 2, WORK>(x, s, dense, lane, acc, work);
+            else compact_count<R, 4, WORK>(x, s, dense, lane, acc, work);
         }
-        acc += t;
     }
     __syncwarp();
 }
 
 // Counts the R-cliques inside the candidate set whose word w sits in lane w (words >= W are
 // zero); adds lane-partial sums to acc.
-//   R >= 3, triangular layout, at most compact_max (R >= 4) or compact3_max (R == 3) members:
-//           re-encoded compactly (compact_entry) and finished on the compact rows.
+//   R >= 3, triangular layout, at most compact_max members: re-encoded compactly
+//           (compact_entry) and finished on the compact rows.
 //   R >= 4: warp-uniform walk over the members a; the next candidate set c ∧ row_a is again
 //           spread over the lanes (one shared-memory load per lane).
 //   R == 3: members are compacted and dealt to lanes; each lane builds its own c ∧ row_a and
@@ -809,7 +735,7 @@ __device__ __forceinline__ void warp_dfs(const WarpCtx &x, uint32_t c, int lane,
                                          unsigned long long &acc, unsigned long long &work)
 {
     if constexpr (R >= 3) {
-        if (x.tri && __reduce_add_sync(kFull, __popc(c)) <= (R == 3 ? x.compact3_max : x.compact_max)) {
+        if (x.tri && __reduce_add_sync(kFull, __popc(c)) <= x.compact_max) {
             compact_entry<R, WORK>(x, c, lane, acc, work);
             return;
         }
@@ -896,19 +822,32 @@ __device__ __forceinline__ void warp_dfs(const WarpCtx &x, uint32_t c, int lane,
     }
 }
 
-// Shared-memory words one warp needs for roots of out-degree <= dcap (dcap multiple of 32).
-// Layout: elem (dcap uint16) | cbuf (32) | compress masks + prefixes (192) | lbuf/mbuf, where
-// mbuf holds compact_max rows of 4 words or the packed rows of an R = 3 set of up to 192 members.
+// Shared-memory words one warp needs for roots of out-degree <= dcap (dcap multiple of 32), in two
+// parts: its own lists, cbuf (32) | mv (compress masks, 192) | the member list of a neighbourhood |
+// elem (dcap uint16, or the rows of a neighbourhood once the set's rows are built), and its
+// lbuf/mbuf, which holds compact_max rows of 4 words.  The second parts of all warps are
+// consecutive, so that a group of neighbouring warps can take its members' parts as one buffer.
+__host__ __device__ __forceinline__ uint32_t warp_list_words(uint32_t dcap, uint32_t compact_max)
+{
+    return 32 + kMaskWords + kNbhdList + (compact_max && kNbhdWords > dcap / 2 ? kNbhdWords : dcap / 2);
+}
+__host__ __device__ __forceinline__ uint32_t warp_buf_words(uint32_t dcap, uint32_t compact_max)
+{
+    return dcap > compact_max * 4 ? dcap : compact_max * 4;
+}
 __host__ __device__ __forceinline__ uint32_t warp_scratch_words(uint32_t dcap, uint32_t compact_max)
 {
-    const uint32_t m = compact_max ? (compact_max * 4 > packed_words(6) ? compact_max * 4 : packed_words(6)) : 0u;
-    return dcap / 2 + 32 + 192 + (dcap > m ? dcap : m);
+    return warp_list_words(dcap, compact_max) + warp_buf_words(dcap, compact_max);
 }
 
 constexpr int kMidMaxWarps = 32;
-constexpr uint32_t kSplitMembers = 128;  // k >= 6: rows above this many members split per member
+constexpr uint32_t kMidStaticSmem = 2048;  // room left for the kernel's static shared memory
 constexpr uint32_t kNoHelpSlot = 0xffffffffu;
 constexpr uint32_t kHelpSlots = 8192;    // heavy roots that can take help, per launch
+constexpr uint32_t kMaxGroups = 15;      // pairs of warps that can head a group (named barriers 1..15)
+
+// Words of the complement rows of a wide set of s members.
+__host__ __device__ __forceinline__ uint32_t wide_words(uint32_t s) { return ((s + 127) >> 7) * s * 4; }
 
 // Position of the r-th (from 0) set bit of x (r < popc(x)).
 __device__ __forceinline__ uint32_t select_bit(uint32_t x, uint32_t r)
@@ -935,12 +874,13 @@ __device__ __forceinline__ uint32_t pick_help_slot(const HelpTable &ht, int lane
         const uint32_t sl = s0 + lane;
         uint32_t rem = 0;
         if (sl < ns) {
-            cuda::atomic_ref<uint32_t, cuda::thread_scope_device> ready(ht.slots[sl].ready);
-            if (ready.load(cuda::memory_order_acquire)) {
-                const uint32_t units = ht.slots[sl].units;
-                const uint32_t cur = *(volatile uint32_t *)&ht.slots[sl].cursor;
-                rem = cur < units ? units - cur : 0u;
-            }
+            cuda::atomic_ref<uint32_t, cuda::thread_scope_device> units(ht.slots[sl].units);
+            const uint32_t un = units.load(cuda::memory_order_acquire);
+            const uint32_t cw = *(volatile uint32_t *)&ht.slots[sl].wide_cursor;
+            const uint32_t cn = *(volatile uint32_t *)&ht.slots[sl].cursor;
+            const uint32_t big = (un >> 21) & 1023u, mid = (un >> 11) & 1023u, narrow = un & 2047u;
+            const uint32_t cb = cw & 0xffffu, cm = cw >> 16;
+            rem = (cb < big ? big - cb : 0u) + (cm < mid ? mid - cm : 0u) + (cn < narrow ? narrow - cn : 0u);
         }
         uint32_t bsl = sl;
 #pragma unroll
@@ -959,17 +899,152 @@ __device__ __forceinline__ uint32_t pick_help_slot(const HelpTable &ht, int lane
     return best;
 }
 
+// Shared state of a group of warps on a wide row.
+struct GroupShared {
+    unsigned long long sl;
+    uint32_t unit, mbar, sd, st, next, over;
+};
+
+// A group's place: gw warps (a power of two), this warp's index gi, its named barrier.
+struct Group {
+    GroupShared *sh;
+    uint32_t *buf;  // the members' scratch buffers as one
+    uint32_t gw, gi, bar;
+
+    __device__ __forceinline__ void sync() const
+    {
+        __syncwarp();
+        asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(gw * 32u) : "memory");
+    }
+};
+
+// Member number r (from 0, in index order) of a set whose word w sits in lane w.
+__device__ __forceinline__ uint32_t select_member(uint32_t c, uint32_t r)
+{
+    const uint32_t pc = __popc(c);
+    const uint32_t incl = warp_incl_scan(pc);
+    const int wl = __ffs(__ballot_sync(kFull, incl > r)) - 1;
+    const uint32_t before = __shfl_sync(kFull, incl - pc, wl);
+    const uint32_t word = __shfl_sync(kFull, c, wl);
+    return (uint32_t)wl * 32 + select_bit(word, r - before);
+}
+
+// R-cliques (R >= 3) of a row c (lane word, more than 128 members; triangular layout), counted by
+// the warps of a group together: the complement rows are built 32 x 32 block by block, then R = 3
+// and R = 4 are one pass over (32 members, chunk of 128 codegrees) units, and for R >= 5 the warps
+// take the members one at a time and walk down from there.  Every warp of the group calls this.
+template <int R, bool WORK>
+__device__ __forceinline__ void wide_row(const WarpCtx &x, const Group &g, uint32_t c, int lane,
+                                         unsigned long long &acc, unsigned long long &work)
+{
+    int clo, chi;
+    const uint32_t s = compact(x, c, lane, clo, chi);
+    prepare_masks(x, clo, chi, lane);
+    const CompSet cs = {g.buf, s, (s + 127) >> 7};
+    const uint32_t nblk = (s + 31) >> 5;
+    uint32_t bits = 0, u = 0;
+    for (uint32_t a = 0; a < nblk; a++) {
+        const uint32_t i = (a << 5) + lane;
+        const uint32_t *row = x.rows + (uint32_t)x.elem[i < s ? i : s - 1] * x.RS;
+        for (uint32_t ow = a; ow < nblk; ow++) {
+            if ((u++ & (g.gw - 1)) != g.gi) continue;
+            const uint32_t j0 = ow << 5, j1 = min(j0 + 31, s - 1);
+            uint32_t cur = 0;
+            for (int w = (int)(x.elem[j0] >> 5); w <= (int)(x.elem[j1] >> 5); w++) {
+                const uint32_t m = x.cbuf[w];
+                if (!m) continue;
+                const uint32_t piece = member_bits(x, row[w], m, w);
+                const int at = (int)x.mv[160 + w] - (int)j0;  // > -32
+                cur |= at >= 0 ? piece << at : piece >> -at;
+            }
+            bits += put_block(cs.m32, s, s, a, ow, cur, lane);
+        }
+    }
+    bits = __reduce_add_sync(kFull, bits);
+    if (lane == 0) atomicAdd(&g.sh->mbar, bits);
+    __syncwarp();
+    x.cbuf[lane] = word_mask(s, lane);
+    g.sync();
+    const bool dense = 2 * g.sh->mbar <= s * (s - 1);
+    const uint4 *M = reinterpret_cast<const uint4 *>(cs.m32);
+    bool counted = false;
+    if (dense) {
+        if constexpr (R == 3) {
+            CompCount o = comp3_wide<WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, lane);
+            if (WORK) work += o.work;
+            o.n = __reduce_add_sync(kFull, o.n);
+            if (lane == 0) atomicAdd(&g.sh->sd, o.n);
+            g.sync();
+            if (g.gi == 0 && lane == 0) add_acc(acc, n3_finish(s, g.sh->sd), x.err);
+            counted = true;
+        } else if constexpr (R == 4) {
+            CompSums o = comp4_wide<WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, x.mv, lane);
+            if (WORK) work += o.work;
+            const bool over = __any_sync(kFull, o.over);
+            o.sd = __reduce_add_sync(kFull, o.sd);
+            o.st = __reduce_add_sync(kFull, o.st);
+#pragma unroll
+            for (int k = 16; k > 0; k >>= 1) o.sl += __shfl_xor_sync(kFull, o.sl, k);
+            if (lane == 0) {
+                if (over) atomicOr(&g.sh->over, 1u);
+                atomicAdd(&g.sh->sd, o.sd);
+                atomicAdd(&g.sh->st, o.st);
+                atomicAdd(&g.sh->sl, o.sl);
+            }
+            g.sync();
+            counted = !g.sh->over;
+            if (counted && g.gi == 0 && lane == 0)
+                add_acc(acc, n4_finish(s, g.sh->sd, g.sh->st, g.sh->sl), x.err);
+        }
+    }
+    if (!counted) {
+        // member by member: on the complement rows when they are sparse, else on the root's rows
+        for (;;) {
+            uint32_t r = 0;
+            if (lane == 0) r = atomicAdd(&g.sh->next, 1u);
+            r = __shfl_sync(kFull, r, 0);
+            if (r >= s) break;
+            if (dense) {
+                if constexpr (R >= 4) {
+                    const uint32_t nc = adjacent_above(cs, word_mask(s, lane), r, lane);
+                    const uint32_t m = __reduce_add_sync(kFull, __popc(nc));
+                    if (m < R - 1) continue;
+                    if constexpr (R == 4) {
+                        __syncwarp();
+                        x.cbuf[lane] = nc;
+                        __syncwarp();
+                        const CompCount o = comp3_wide<WORK>(M, s, cs.nch, x.cbuf, m, nblk, 0, 1, lane);
+                        if (WORK) work += o.work;
+                        const uint32_t sum = __reduce_add_sync(kFull, o.n);
+                        if (lane == 0) add_acc(acc, n3_finish(m, sum), x.err);
+                    } else {
+                        dense_dfs<R - 1, 0, WORK>(x, cs, nc, m, lane, acc, work);
+                    }
+                }
+            } else {
+                const uint32_t b = select_member(c, r);
+                const uint32_t c2 = lane < (int)x.W ? (c & x.rows[b * x.RS + lane]) : 0u;
+                if (WORK && lane < (int)x.W) work += 1;
+                const uint32_t m = __reduce_add_sync(kFull, __popc(c2));
+                if (m >= R - 1) warp_dfs<R - 1, WORK>(x, c2, lane, acc, work);
+            }
+        }
+    }
+}
+
 // Bitmap path (small_max < D <= dcap): one block per root, roots taken largest-D first from the
 // queue.  The block builds the root's local subgraph as D x D bitmap rows in shared memory
 // (row i = V(g_u) ∩ N+(a_i), Algorithm GenSub-CITRON by sorted-list intersection) and its warps
-// count the (K-2)-cliques of every row.
-//   D < split_min: the rows (edge tasks (u, a_t)) are taken from a counter in shared memory.
-//   D >= split_min (heavy roots, K >= 6): the root's work is a space of units -- one per edge
-//       task, or one per member b of a row of more than 128 members (the edge sub-task
-//       (u, a_t, b): the (K-3)-cliques of row_t ∧ row_b) -- taken from a cursor in a global
-//       table.  Blocks that find the root queue empty pick the published heavy root with the
-//       most units left, rebuild its rows and take units from the same cursor (work stealing
-//       across blocks); every block adds its own part of the root's count.
+// count the (K-2)-cliques of every row: the edge tasks (u, a_t).
+//   K >= 5, triangular layout: rows of more than 128 members (wide rows) are counted first, each
+//       by a group of warps whose scratch buffers together hold its complement rows: as many warps
+//       as the root's widest row needs for the rows that two warps cannot hold, then two warps each;
+//       the other rows by one warp each.
+//   D < split_min: the rows are taken from counters in shared memory.
+//   D >= split_min (heavy roots, K >= 6): the rows are taken from cursors in a global table.
+//       Blocks that find the root queue empty pick the published heavy root with the most rows
+//       left, rebuild its rows and take from the same cursors (work stealing across blocks);
+//       every block adds its own part of the root's count.
 // block_ns (optional): each block's start and end on the global timer.
 template <int K, bool WORK>
 __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
@@ -983,23 +1058,27 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     const uint32_t rs_cap = (dcap / 32) | 1;
     uint32_t *sL = smem;
     uint32_t *rows = smem + dcap;
-    __shared__ uint32_t s_idx, s_task, s_tri, s_slot, s_u, s_units;
+    __shared__ uint32_t s_idx, s_task, s_wide[2], s_tri, s_slot, s_u, s_most;
+    __shared__ uint32_t s_cls[2][kBitmapCap / 32];  // wide rows of either class, one bit each
     __shared__ unsigned long long s_acc[32], s_arc[32];
+    __shared__ GroupShared s_group[kMaxGroups];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const uint32_t wsw = warp_scratch_words(dcap, compact_max);
-    uint32_t *wscr = rows + (size_t)dcap * rs_cap + (size_t)w * wsw;
-    // unit prefix of a heavy root's rows: it reuses sL, which is dead once the rows are built
-    uint32_t *s_upre = sL;
+    uint32_t *lists = rows + (size_t)dcap * rs_cap;
+    uint32_t *wscr = lists + (size_t)w * warp_list_words(dcap, compact_max);
+    const uint32_t buf_words = warp_buf_words(dcap, compact_max);
+    uint32_t *bufs = lists + (size_t)nw * warp_list_words(dcap, compact_max);
+    // order of a root's rows, wide ones first: it reuses sL, which is dead once the rows are built
+    uint16_t *s_order = reinterpret_cast<uint16_t *>(sL);
     WarpCtx x;
     x.rows = rows;
-    x.elem = reinterpret_cast<uint16_t *>(wscr);
-    x.cbuf = wscr + dcap / 2;
-    x.mv = wscr + dcap / 2 + 32;
-    x.lbuf = wscr + dcap / 2 + 32 + 192;
+    x.cbuf = wscr;
+    x.mv = wscr + 32;
+    x.elem = reinterpret_cast<uint16_t *>(wscr + 32 + kMaskWords + kNbhdList);
+    x.lbuf = bufs + (size_t)w * buf_words;
     x.mbuf = x.lbuf;
     x.compact_max = compact_max;
-    x.compact3_max = compact_max ? 192u : 0u;
     x.pair_cap = dcap;
+    x.err = err;
     const uint32_t nlist = st->n_mid;
     if (WORK && lane == 0) s_arc[w] = 0;
     if (block_ns && threadIdx.x == 0) block_ns[2 * blockIdx.x] = global_ns();
@@ -1009,6 +1088,8 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
         if (threadIdx.x == 0) {
             s_idx = queue_empty || budget.over(err) ? 0xfffffffeu : atomicAdd(next, 1u);
             s_task = 0;
+            s_wide[0] = s_wide[1] = 0;
+            s_most = 0;
             s_tri = 1;
             s_slot = kNoHelpSlot;
         }
@@ -1078,96 +1159,148 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             x.RS = RS;
             x.W = W;
             x.tri = s_tri != 0;
-            // Units: edge tasks (u, a_t) -- count (K-2)-cliques in row t -- one per row for a light
-            // root; for a heavy root the unit space of its rows (prefix in s_upre), shared with
-            // helping blocks through its slot.
-            uint32_t U = D;
-            if (heavy) {
-                for (uint32_t t = w; t < D; t += nw) {
-                    const uint32_t c = lane < W ? rows[t * RS + lane] : 0u;
-                    const uint32_t m = __reduce_add_sync(kFull, __popc(c));
-                    if (lane == 0)
-                        s_upre[t] = m < (uint32_t)(K - 2) ? 0u : ((K >= 6 && m > kSplitMembers) ? m : 1u);
-                }
-                __syncthreads();
-                if (w == 0) {
-                    uint32_t run = 0;
-                    for (uint32_t t0 = 0; t0 < D; t0 += 32) {
-                        const uint32_t v = t0 + lane < D ? s_upre[t0 + lane] : 0u;
-                        const uint32_t inc = warp_incl_scan(v);
-                        if (t0 + lane < D) s_upre[t0 + lane] = run + inc - v;
-                        run += __shfl_sync(kFull, inc, 31);
+            // Wide rows come first in the order of the rows: those that need more than two warps'
+            // buffers, the other ones, then the rows of one warp.  A root of at most 129
+            // out-neighbours has no wide row.
+            uint32_t nbig = 0, nmid = 0, narrow = D;
+            const uint32_t most_gw = 1u << (31 - __clz(nw));  // warps of the largest group
+            if constexpr (K >= 5) {
+                if (x.tri && compact_max && D > kNarrow + 1) {
+                    for (uint32_t q = w; q < W; q += nw) {
+                        const uint32_t t = q * 32 + lane;
+                        uint32_t m = 0;
+                        if (t < D)
+                            for (uint32_t v = q; v < W; v++) m += __popc(rows[t * RS + v]);
+                        // a row too wide for the block's buffers is left to one warp
+                        const bool wide = m > kNarrow && wide_words(m) <= buf_words * most_gw;
+                        const bool big = wide && wide_words(m) > buf_words * 2;
+                        const uint32_t bb = __ballot_sync(kFull, big), mb = __ballot_sync(kFull, wide && !big);
+                        const uint32_t most = __reduce_max_sync(kFull, wide ? m : 0u);
+                        if (lane == 0) {
+                            s_cls[0][q] = bb;
+                            s_cls[1][q] = mb;
+                            if (most) atomicMax(&s_most, most);
+                        }
                     }
-                    if (lane == 0) s_units = run;
+                    __syncthreads();
+                    if (s_most) {
+                        for (uint32_t q = 0; q < W; q++) {
+                            nbig += __popc(s_cls[0][q]);
+                            nmid += __popc(s_cls[1][q]);
+                        }
+                        for (uint32_t q = w; q < W; q += nw) {
+                            uint32_t rb = 0, rm = 0;
+                            for (uint32_t v = 0; v < q; v++) {
+                                rb += __popc(s_cls[0][v]);
+                                rm += __popc(s_cls[1][v]);
+                            }
+                            const uint32_t t = q * 32 + lane, bb = s_cls[0][q], mb = s_cls[1][q];
+                            rb += __popc(bb & lanemask_lt());
+                            rm += __popc(mb & lanemask_lt());
+                            const uint32_t at = (bb >> lane) & 1u   ? rb
+                                                : (mb >> lane) & 1u ? nbig + rm
+                                                                    : nbig + nmid + (t - rb - rm);
+                            if (t < D) s_order[at] = (uint16_t)t;
+                        }
+                        __syncthreads();
+                    }
                 }
-                __syncthreads();
-                U = s_units;
+                narrow = D - nbig - nmid;
+            }
+            const uint32_t nwide = nbig + nmid;
+            if (heavy) {
                 if (threadIdx.x == 0) {
+                    const uint32_t units = 0x80000000u | (nbig << 21) | (nmid << 11) | narrow;
                     if (owner && ht.slots) {
                         const uint32_t sl = atomicAdd(ht.nslots, 1u);
                         if (sl < ht.cap) {
                             ht.slots[sl].u = u;
-                            ht.slots[sl].units = U;
-                            ht.slots[sl].cursor = 0;
-                            cuda::atomic_ref<uint32_t, cuda::thread_scope_device> ready(ht.slots[sl].ready);
-                            ready.store(1u, cuda::memory_order_release);
+                            cuda::atomic_ref<uint32_t, cuda::thread_scope_device> pub(ht.slots[sl].units);
+                            pub.store(units, cuda::memory_order_release);
                             s_slot = sl;
                         }
-                    } else if (!owner && ht.slots[s_slot].units != U) {
+                    } else if (!owner && ht.slots[s_slot].units != units) {
                         set_error(err, kDevBadInput);  // the rebuilt root differs from the published one
-                        s_task = U;                    // take nothing
+                        s_task = narrow;               // take nothing
+                        s_wide[0] = nbig;
+                        s_wide[1] = nmid;
+                        s_slot = kNoHelpSlot;
                     }
                 }
                 __syncthreads();
             }
-            // the units of a published heavy root come from its slot's cursor in global memory,
-            // the others from the block's counter in shared memory
-            uint32_t *gcursor = (s_slot != kNoHelpSlot && (owner || s_task == 0)) ? &ht.slots[s_slot].cursor
-                                                                                    : nullptr;
-            // a warp claims its next unit before it works on the current one, so that the
+            // the rows of a published heavy root are taken from its slot's cursors in global
+            // memory, the others from the block's counters in shared memory
+            HeavySlot *slot = s_slot != kNoHelpSlot ? &ht.slots[s_slot] : nullptr;
+            if constexpr (K >= 5) {
+                // Rows s_order[first .. first + count) of class cls by groups of gw warps.  A group is
+                // named by its first warp (barrier and shared state), so that a warp can go on to
+                // the next class while other groups are still at this one: every warp of the new
+                // group has left its old group, whose last barrier it shared with the rest.
+                auto run_wide = [&](int cls, uint32_t first, uint32_t count, uint32_t gw) {
+                    const uint32_t w0 = (uint32_t)w & ~(gw - 1);
+                    if (w0 + gw > (uint32_t)nw || w0 >= 2 * kMaxGroups) return;
+                    Group g;
+                    g.gw = gw;
+                    g.gi = (uint32_t)w - w0;
+                    g.bar = 1 + w0 / 2;
+                    g.sh = &s_group[w0 / 2];
+                    g.buf = bufs + (size_t)w0 * buf_words;
+                    for (;;) {
+                        if (g.gi == 0 && lane == 0) {
+                            uint32_t v = count;
+                            if (!(heavy && budget.over(err))) {
+                                if (!slot) v = atomicAdd(&s_wide[cls], 1u);
+                                else v = cls == 0 ? atomicAdd(&slot->wide_cursor, 1u) & 0xffffu
+                                                  : atomicAdd(&slot->wide_cursor, 0x10000u) >> 16;
+                            }
+                            *g.sh = {0, v, 0, 0, 0, 0, 0};
+                        }
+                        g.sync();
+                        const uint32_t i = g.sh->unit;
+                        if (i >= count) break;
+                        const uint32_t t = s_order[first + i];
+                        const uint32_t c = lane < W ? rows[t * RS + lane] : 0u;
+                        wide_row<K - 2, WORK>(x, g, c, lane, acc, work);
+                        if (WORK && sink.per_arc) {
+                            const unsigned long long d = warp_sum_u64(acc, err);
+                            if (lane == 0) {
+                                if (d) atomicAdd(&sink.per_arc[base + t], d);
+                                s_arc[w] += d;
+                            }
+                            acc = 0;
+                        }
+                        g.sync();
+                    }
+                    g.sync();  // every warp has read the last claim before the state is used again
+                };
+                if (nwide) {
+                    uint32_t gw = 2;
+                    if (nbig) {
+                        while (gw * buf_words < wide_words(s_most) && gw < most_gw) gw *= 2;
+                    }
+#pragma unroll 1
+                    for (int cls = nbig ? 0 : 1; cls < 2; cls++)
+                        run_wide(cls, cls ? nbig : 0u, cls ? nmid : nbig, cls ? 2u : gw);
+                }
+            }
+            // a warp claims its next row before it works on the current one, so that the
             // atomic's round trip (global memory for a published heavy root) overlaps the work
             auto claim = [&]() -> uint32_t {
                 uint32_t v = 0;
                 if (lane == 0)
-                    v = heavy && budget.over(err) ? U : (gcursor ? atomicAdd(gcursor, 1u) : atomicAdd(&s_task, 1u));
+                    v = heavy && budget.over(err) ? narrow : (slot ? atomicAdd(&slot->cursor, 1u) : atomicAdd(&s_task, 1u));
                 return v;
             };
             uint32_t next_i = claim();
             for (;;) {
                 const uint32_t i = __shfl_sync(kFull, next_i, 0);
-                if (i >= U) break;
+                if (i >= narrow) break;
                 next_i = claim();
-                uint32_t t = i, j = 0;
-                bool whole = true;
-                if (heavy) {
-                    // the row of unit i: the last t with s_upre[t] <= i
-                    uint32_t lo = 0, hi = D - 1;
-                    while (lo < hi) {
-                        const uint32_t mid = (lo + hi + 1) >> 1;
-                        if (s_upre[mid] <= i) lo = mid;
-                        else hi = mid - 1;
-                    }
-                    t = lo;
-                    j = i - s_upre[t];
-                    whole = (t + 1 < D ? s_upre[t + 1] : U) - s_upre[t] == 1u;
-                }
+                const uint32_t t = nwide ? s_order[nwide + i] : i;
                 const uint32_t c = lane < W ? rows[t * RS + lane] : 0u;
-                if (whole) {
-                    const uint32_t cnt = __reduce_add_sync(kFull, __popc(c));
-                    if (cnt >= K - 2) warp_dfs<K - 2, WORK>(x, c, lane, acc, work);
-                } else if constexpr (K >= 6) {
-                    // the j-th member b of row t: the sub-task (u, a_t, b)
-                    const uint32_t pc = __popc(c);
-                    const uint32_t incl = warp_incl_scan(pc);
-                    const int wl = __ffs(__ballot_sync(kFull, incl > j)) - 1;
-                    const uint32_t before = __shfl_sync(kFull, incl - pc, wl);
-                    const uint32_t word = __shfl_sync(kFull, c, wl);
-                    const uint32_t b = (uint32_t)wl * 32 + select_bit(word, j - before);
-                    const uint32_t c2 = lane < W ? (c & rows[b * RS + lane]) : 0u;
-                    if (WORK && lane < (int)W) work += 1;
-                    const uint32_t cnt = __reduce_add_sync(kFull, __popc(c2));
-                    if (cnt >= K - 3) warp_dfs<K - 3, WORK>(x, c2, lane, acc, work);
-                }
+                const uint32_t cnt = __reduce_add_sync(kFull, __popc(c));
+                if (cnt >= K - 2) warp_dfs<K - 2, WORK>(x, c, lane, acc, work);
                 if (WORK && sink.per_arc) {
                     // debug output (instrumented kernel only): acc holds this unit's part of edge
                     // task t alone (it restarts from zero after every unit; the warp's running
@@ -1391,9 +1524,9 @@ static cudaError_t launch_mid(uint32_t grid_cap, uint32_t block_cap, uint32_t dc
     int dev = 0, optin = 0;
     if ((e = cudaGetDevice(&dev))) return e;
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
-    if ((size_t)(optin - 1024) < smem) return cudaErrorInvalidValue;
+    if ((size_t)optin < smem + kMidStaticSmem) return cudaErrorInvalidValue;
     if ((e = cudaFuncSetAttribute(k_count_mid<K, WORK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  optin - 1024)))
+                                  optin - (int)kMidStaticSmem)))
         return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_count_mid<K, WORK>, warps * 32,
@@ -1430,10 +1563,12 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
         cudaGetDevice(&dev);
         if ((e = cudaDeviceGetAttribute(&smem_cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)))
             return e;
-        smem_cap -= 1024;  // static shared memory of the kernel
+        smem_cap -= (int)kMidStaticSmem;
+        // k = 4 ends at R = 2 and re-encodes no set: its warps need no room for one
+        const uint32_t compact_max = K >= 5 ? plan.compact_max : 0u;
         auto smem_for = [&](uint32_t warps) {
             return ((size_t)dcap +
-                    (K > 3 ? (size_t)dcap * rs + (size_t)warps * warp_scratch_words(dcap, plan.compact_max) : 0)) *
+                    (K > 3 ? (size_t)dcap * rs + (size_t)warps * warp_scratch_words(dcap, compact_max) : 0)) *
                    sizeof(uint32_t);
         };
         uint32_t warps = plan.warps_per_cta > (uint32_t)kMidMaxWarps ? kMidMaxWarps : plan.warps_per_cta;
@@ -1445,14 +1580,14 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
         // of the plain kernel)
         if (run.count_work || run.sink.per_arc) {
             if constexpr (K <= (int)kInstrumentedMaxK)
-                e = launch_mid<K, true>(hs.n_mid, plan.max_blocks, dcap, plan.compact_max, plan.split_min,
+                e = launch_mid<K, true>(hs.n_mid, plan.max_blocks, dcap, compact_max, plan.split_min,
                                         aux.help, warps, smem_for(warps), dag_off, dag_cols, mid_list, st,
                                         next + 0, result, run.sink, work, block_ns, aux.budget, &grid, err,
                                         s, num_sms);
             else
                 e = cudaErrorNotSupported;  // refused by citron_count_ex before any launch
         } else
-            e = launch_mid<K, false>(hs.n_mid, plan.max_blocks, dcap, plan.compact_max, plan.split_min,
+            e = launch_mid<K, false>(hs.n_mid, plan.max_blocks, dcap, compact_max, plan.split_min,
                                      aux.help, warps, smem_for(warps), dag_off, dag_cols, mid_list, st,
                                      next + 0, result, run.sink, work, block_ns, aux.budget, &grid, err, s,
                                     num_sms);

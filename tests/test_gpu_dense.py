@@ -1,0 +1,48 @@
+"""Dense candidate sets counted on their complement (csrc/dense.cuh): one edge task whose set has
+exactly s members, at the sizes where the layout changes (words of 32, the 128 members of one warp,
+the chunks of wide sets), from sparse to complete, against the CPU oracle."""
+import numpy as np
+import pytest
+
+from paper_2112_10913_gb300 import graphgen as gg
+
+pytestmark = pytest.mark.gpu
+
+
+def one_set(s, p, seed, hubs=0):
+    """Vertices 0 and 1 adjacent to every vertex; the others form G(s, p), the first `hubs` of them
+    with a third of those edges only (a skewed complement)."""
+    rng = np.random.default_rng(seed)
+    i, j = np.triu_indices(s, 1)
+    keep = rng.random(i.size) < np.where((i < hubs) | (j < hubs), p / 3, p)
+    src = np.concatenate([[0], np.zeros(s, int), np.ones(s, int), i[keep] + 2])
+    dst = np.concatenate([[1], np.arange(s) + 2, np.arange(s) + 2, j[keep] + 2])
+    return gg.csr_from_edges(s + 2, src, dst, name=f"set{s}-{p}-{hubs}")
+
+
+CASES = [(s, p, 0, k) for s in (31, 32, 33, 64, 65, 96, 127, 128) for p in (0.3, 0.6, 0.93) for k in (5, 6)]
+CASES += [(s, p, 0, k) for s in (129, 160, 193) for p in (0.3, 0.55, 0.8) for k in (5, 6)]
+CASES += [(40, 0.9, 0, 7), (96, 0.7, 0, 7), (128, 0.6, 0, 7), (129, 0.7, 0, 7), (150, 0.6, 0, 7)]
+CASES += [(s, 0.95, 24, k) for s in (33, 64, 128) for k in (5, 6)]
+CASES += [(140, 0.9, 24, 6), (256, 0.8, 24, 5), (257, 0.75, 40, 6), (50, 0.95, 10, 8), (140, 0.6, 10, 8)]
+CASES += [(40, 1.0, 0, 9), (100, 1.0, 0, 6), (140, 1.0, 0, 5)]
+# a third and more chunks, members of more than 255 missing neighbours, more than 128 of them
+CASES += [(300, 0.7, 40, 6), (385, 0.52, 0, 6), (530, 0.5, 0, 6), (520, 0.55, 0, 5)]
+
+
+@pytest.mark.parametrize("s,p,hubs,k", CASES)
+def test_one_dense_set(gpu, oracle_lib, s, p, hubs, k):
+    import paper_2112_10913_gb300 as cg
+
+    g = one_set(s, p, s * 7 + k, hubs)
+    rank = np.arange(g.n, dtype=np.uint32)
+    off, cols = oracle_lib.dag_by_rank(g.off, g.cols, g.n, rank, relabel=True)
+    want = oracle_lib.count(off, cols, g.n, k)
+    G = cg.DeviceGraph(g, rank=rank)
+    assert G.count(k) == want
+    # few warps per block (groups of warps at the block's edge) and every root split
+    assert G.count(k, warps_per_cta=3) == want
+    assert G.count(k, split_min=33, small_max=1) == want
+    if k <= 6 and s <= 200:
+        total, per_arc = G.count_per_arc(k)
+        assert total == want and int(per_arc.sum()) == want
