@@ -11,8 +11,9 @@
 //       degrees for all candidates in one step (Counting's l = 2 branch, Sec. V-B last paragraph).
 //   D <= bitmap_max (<= 1024) k_count_mid: one block per root, roots taken largest-D first from
 //       a device queue.  The local subgraph is a D x D bitmap in shared memory built by
-//       intersecting the sorted list N+(u) with every N+(a_i) (binary search of each element of
-//       N+(a_i) in N+(u), lists kept sorted as in the paper).  Its edges (u, a_i) are the tasks
+//       intersecting the sorted list N+(u) with every N+(a_i): each element of N+(a_i) is looked up
+//       in a bitmap of the ids just below N+(u)'s largest (binary search for the few ids under
+//       it).  Its edges (u, a_i) are the tasks
 //       of the block's warps (edge-parallel counting); a warp recurses with the candidate set
 //       spread over its lanes, one 32-bit word per lane, using ballot / popc / shuffles.
 //   D > bitmap_max  k_count_list: one warp per root, candidate sets kept as sorted lists in
@@ -95,6 +96,7 @@ __global__ __launch_bounds__(1024) void k_mid_bins(const uint32_t *hist, uint32_
     for (uint32_t i = lo; i < hi; i++) {
         const uint32_t d = bins - 1 - i;
         cursor[d] = run;
+        if (d == kLowMax) st->n_high = run;  // (zero when no degree above kLowMax has a bin)
         run += hist[d];
     }
     if (threadIdx.x == 0) st->n_mid = total;
@@ -347,6 +349,9 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     hs.n_small = max_outdeg >= need ? n : 0;
     hs.max_mid = max_outdeg < plan.bitmap_max ? max_outdeg : plan.bitmap_max;
     hs.n_mid = hs.max_mid > plan.small_max ? n : 0;
+    // upper bounds of both parts of the queue: the kernels read the real ones on the device
+    hs.n_high = hs.max_mid > kLowMax ? n : 0;
+    hs.bound = 1;
     hs.max_big = max_outdeg;
     hs.n_big = max_outdeg > plan.bitmap_max ? n : 0;
     run.time_kernels = false;

@@ -14,12 +14,24 @@ constexpr int kMaxK = CITRON_MAX_K;
 constexpr uint32_t kBitmapCap = 1024;  // largest root handled by the bitmap path
 constexpr int kSmallWarps = 8;         // warps per block of k_count_small
 constexpr int kListWarps = 4;          // warps per block of k_count_list
+constexpr uint32_t kSmallWindow = 16384;  // ids in a warp's membership bitmap (k_count_small), and ...
+constexpr uint32_t kMidWindow = 32768;    // ... in a block's (k_count_mid)
 
 struct CountStats {
     uint32_t n_small, n_mid, n_big;
     uint32_t max_mid, max_big, max_all;
-    uint32_t pad[2];
+    uint32_t n_high;  // bitmap-path roots above kLowMax, the first n_high of the queue
+    uint32_t bound;   // host copy only: the numbers are upper bounds (each part may hold n_mid roots)
 };
+
+// Up to k = 6, bitmap-path roots of at most kLowMax out-neighbours run in a launch of their own, in
+// blocks of 8 warps, several per SM: a block of 32 warps has a handful of rows per warp to build
+// for them and waits at its barriers instead.  R-MAT 15, k = 6: 0.70 ms in one launch, 0.64 in two
+// (0.79 with 4 warps).  Above that a root's counting outweighs its build and two launches end in
+// two tails: R-MAT 15, k = 8: 69 ms in one launch, 129 in two.
+constexpr uint32_t kLowMax = 128;
+constexpr uint32_t kLowWarps = 8;
+constexpr int kPartsMaxK = 6;
 
 // ------------------------------------------------------------------------------------------
 // Warp-register path (D <= 32).
@@ -60,6 +72,33 @@ __device__ __forceinline__ uint32_t lower_bound_smem(const uint32_t *a, uint32_t
     return lo;
 }
 
+// Membership of ids in a sorted list L[0..D) (the out-neighbours of a root), for the intersections
+// N+(u) ∩ N+(a).  The ids of the largest `span` values below L's maximum are looked up in a bitmap
+// (one load and a bit test; the place in L is the place of the word's first member plus the bits
+// below), the smaller ones by binary search.  In a degree-ordered, relabelled DAG the heads of the
+// paths u -> a -> y crowd at the top ranks: on R-MAT 20 97 % of them (by paths) lie in the last 2^14
+// ranks below the root's largest neighbour and 99 % in the last 2^15, where a binary search took
+// log2 D dependent loads.
+template <typename Place>
+struct Window {
+    uint32_t *bits;   // bitmap words
+    Place *first;     // place in L of each word's first member
+    uint32_t base;    // id of bit 0
+    uint32_t span;    // ids base .. base + span - 1 are in the bitmap
+    uint32_t nlow;    // members below base
+
+    __device__ __forceinline__ bool has(uint32_t y) const
+    {
+        const uint32_t p = y - base;
+        return p < span && ((bits[p >> 5] >> (p & 31u)) & 1u);
+    }
+    __device__ __forceinline__ uint32_t place(uint32_t y) const
+    {
+        const uint32_t p = y - base;
+        return first[p >> 5] + __popc(bits[p >> 5] & ((1u << (p & 31u)) - 1u));
+    }
+};
+
 template <int K>
 __global__ __launch_bounds__(kSmallWarps * 32) void k_count_small(
     const uint64_t *__restrict__ dag_off, const uint32_t *__restrict__ dag_cols,
@@ -67,9 +106,16 @@ __global__ __launch_bounds__(kSmallWarps * 32) void k_count_small(
     RootSink sink, Budget budget, uint32_t *err)
 {
     __shared__ uint32_t sL[kSmallWarps][32];
+    __shared__ uint32_t s_bits[kSmallWarps][kSmallWindow / 32];
+    __shared__ uint8_t s_first[kSmallWarps][kSmallWindow / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t nlist = st->n_small;
     const uint32_t gw = blockIdx.x * kSmallWarps + w, nwarps = gridDim.x * kSmallWarps;
+    Window<uint8_t> win;
+    win.bits = s_bits[w];
+    win.first = s_first[w];
+    for (uint32_t i = lane; i < kSmallWindow / 32; i += 32) s_bits[w][i] = 0;
+    __syncwarp();
     unsigned long long total = 0;
     for (uint32_t idx = gw; idx < nlist; idx += nwarps) {
         int stop = 0;
@@ -79,29 +125,50 @@ __global__ __launch_bounds__(kSmallWarps * 32) void k_count_small(
         const uint64_t base = dag_off[u];
         const uint32_t D = (uint32_t)(dag_off[u + 1] - base);
         const uint32_t x = lane < D ? dag_cols[base + lane] : 0xffffffffu;
-        sL[w][lane] = x;
-        __syncwarp();
-        const uint32_t lmax = __shfl_sync(kFull, x, D - 1);
         uint64_t rb = 0, re = 0;
         if (lane < D) {
             rb = dag_off[x];
             re = dag_off[x + 1];
         }
+        sL[w][lane] = x;
+        const uint32_t lmax = __shfl_sync(kFull, x, D - 1);
+        win.base = lmax >= kSmallWindow ? lmax - (kSmallWindow - 1) : 0u;
+        win.span = lmax - win.base + 1;
+        const bool in_win = lane < D && x >= win.base;
+        win.nlow = __popc(__ballot_sync(kFull, lane < D && !in_win));
+        const uint32_t xw = in_win ? (x - win.base) >> 5 : 0xffffffffu;
+        const uint32_t prev = __shfl_up_sync(kFull, xw, 1);
+        if (in_win) {
+            atomicOr(&win.bits[xw], 1u << ((x - win.base) & 31u));
+            if (lane == 0 || prev != xw) win.first[xw] = (uint8_t)lane;
+        }
+        __syncwarp();
         uint32_t myrow = 0;
         for (uint32_t i = 0; i < D; i++) {
-            const uint64_t b = __shfl_sync(kFull, rb, i), e = __shfl_sync(kFull, re, i);
+            const uint64_t b = __shfl_sync(kFull, rb, i);
+            const uint32_t len = (uint32_t)(__shfl_sync(kFull, re, i) - b);
             uint32_t bits = 0;
-            for (uint64_t p = b; p < e; p += 32) {
-                const uint32_t y = p + lane < e ? dag_cols[p + lane] : 0xffffffffu;
-                if (__shfl_sync(kFull, y, 0) > lmax) break;
-                if (y <= lmax) {
-                    const uint32_t j = lower_bound_smem(sL[w], D, y);
-                    if (sL[w][j] == y) bits |= 1u << j;
+            // four loads in flight per lane
+            for (uint32_t p = lane; __any_sync(kFull, p < len); p += 128) {
+                uint32_t y[4];
+#pragma unroll
+                for (int h = 0; h < 4; h++) y[h] = p + 32 * h < len ? dag_cols[b + p + 32 * h] : 0xffffffffu;
+                if (__shfl_sync(kFull, y[0], 0) > lmax) break;
+#pragma unroll
+                for (int h = 0; h < 4; h++) {
+                    if (win.has(y[h])) {
+                        bits |= 1u << win.place(y[h]);
+                    } else if (win.nlow && y[h] < win.base) {
+                        const uint32_t j = lower_bound_smem(sL[w], win.nlow, y[h]);
+                        if (j < win.nlow && sL[w][j] == y[h]) bits |= 1u << j;
+                    }
                 }
             }
             bits = __reduce_or_sync(kFull, bits);
             if (lane == i) myrow = bits;
         }
+        __syncwarp();
+        if (in_win) win.bits[xw] = 0;
         unsigned long long acc = 0;
         const uint32_t all = D == 32 ? kFull : ((1u << D) - 1);
         if (sink.per_arc) {
@@ -1049,8 +1116,8 @@ __device__ __forceinline__ void wide_row(const WarpCtx &x, const Group &g, uint3
 template <int K, bool WORK>
 __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     const uint64_t *__restrict__ dag_off, const uint32_t *__restrict__ dag_cols,
-    const uint32_t *__restrict__ list, const CountStats *st, uint32_t *next, uint32_t dcap,
-    uint32_t compact_max, uint32_t split_min, HelpTable ht, unsigned long long *result,
+    const uint32_t *__restrict__ list, const CountStats *st, uint32_t *next, int low, uint32_t dcap,
+    uint32_t window, uint32_t compact_max, uint32_t split_min, HelpTable ht, unsigned long long *result,
     RootSink sink, unsigned long long *work_out, unsigned long long *block_ns, Budget budget,
     uint32_t *err)
 {
@@ -1063,7 +1130,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     __shared__ unsigned long long s_acc[32], s_arc[32];
     __shared__ GroupShared s_group[kMaxGroups];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    uint32_t *lists = rows + (size_t)dcap * rs_cap;
+    uint32_t *lists = K > 3 ? rows + (size_t)dcap * rs_cap : rows;  // k = 3 keeps no rows
     uint32_t *wscr = lists + (size_t)w * warp_list_words(dcap, compact_max);
     const uint32_t buf_words = warp_buf_words(dcap, compact_max);
     uint32_t *bufs = lists + (size_t)nw * warp_list_words(dcap, compact_max);
@@ -1079,7 +1146,14 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     x.compact_max = compact_max;
     x.pair_cap = dcap;
     x.err = err;
-    const uint32_t nlist = st->n_mid;
+    // the membership window of the root being built lies over the warps' lists and buffers
+    Window<uint16_t> win;
+    win.bits = lists;
+    win.first = reinterpret_cast<uint16_t *>(lists + window / 32);
+    // this launch's part of the queue (largest out-degree first)
+    const uint32_t first_root = low ? st->n_high : 0u;
+    const uint32_t nlist = (low || K > kPartsMaxK ? st->n_mid : st->n_high) - first_root;
+    list += first_root;
     if (WORK && lane == 0) s_arc[w] = 0;
     if (block_ns && threadIdx.x == 0) block_ns[2 * blockIdx.x] = global_ns();
     unsigned long long block_total = 0;  // meaningful in thread 0
@@ -1118,36 +1192,82 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
         }
         const bool heavy = K >= 6 && (!owner || D >= split_min);
         const uint32_t W = (D + 31) >> 5, RS = W | 1;
+        // the rows this warp builds (w, w + nw, ..): lane r holds the place of the r-th one's list
+        const uint32_t mine = w + (uint32_t)nw * lane;
         for (uint32_t i = threadIdx.x; i < D; i += blockDim.x) sL[i] = dag_cols[base + i];
         if (K > 3)
             for (uint32_t i = threadIdx.x; i < D * RS; i += blockDim.x) rows[i] = 0;
+        for (uint32_t i = threadIdx.x; i < window / 32; i += blockDim.x) win.bits[i] = 0;
         __syncthreads();
         const uint32_t lmax = sL[D - 1];
+        win.base = lmax >= window ? lmax - (window - 1) : 0u;
+        win.span = lmax - win.base + 1;
+        uint64_t rb = 0;
+        uint32_t rlen = 0;
+        if (mine < D) {
+            const uint32_t a = sL[mine];
+            rb = dag_off[a];
+            rlen = (uint32_t)(dag_off[a + 1] - rb);
+        }
+        for (uint32_t i = threadIdx.x; i < D; i += blockDim.x) {
+            const uint32_t v = sL[i];
+            if (v >= win.base) {
+                const uint32_t p = v - win.base;
+                atomicOr(&win.bits[p >> 5], 1u << (p & 31u));
+                if (K > 3 && (i == 0 || sL[i - 1] < win.base || ((sL[i - 1] - win.base) >> 5) != (p >> 5)))
+                    win.first[p >> 5] = (uint16_t)i;
+            }
+        }
+        __syncthreads();
+        win.nlow = win.base ? lower_bound_smem(sL, D, win.base) : 0u;
         unsigned long long acc = 0, work = 0;
         // Build the local subgraph: row i = V(g_u) ∩ N+(a_i) (CITRON's GenSubgraph).  Each step
-        // loads 64 entries of N+(a_i) (two per lane) so that two loads are in flight.  (A block
-        // helping with a heavy root rebuilds the same rows; its triangles are not counted here.)
+        // loads 128 entries of N+(a_i), four per lane in flight.  The places found by a step's 32
+        // entries are consecutive in order, so the row's words are gathered and stored whole: the
+        // row belongs to this warp.  (A block helping with a heavy root rebuilds the same rows;
+        // its triangles are not counted here.)
         bool tri = true;
-        for (uint32_t i = w; i < D; i += nw) {
-            const uint32_t a = sL[i];
-            const uint64_t b = dag_off[a], e = dag_off[a + 1];
-            for (uint64_t p = b; p < e; p += 64) {
-                const uint32_t y0 = p + lane < e ? dag_cols[p + lane] : 0xffffffffu;
-                const uint32_t y1 = p + 32 + lane < e ? dag_cols[p + 32 + lane] : 0xffffffffu;
-                if (__shfl_sync(kFull, y0, 0) > lmax) break;
+        for (uint32_t i = w, r = 0; i < D; i += nw, r++) {
+            if (r == 32) {  // more rows than lanes: the places of the next 32
+                r = 0;
+                rb = 0;
+                rlen = 0;
+                if (i + (uint32_t)nw * lane < D) {
+                    const uint32_t a = sL[i + (uint32_t)nw * lane];
+                    rb = dag_off[a];
+                    rlen = (uint32_t)(dag_off[a + 1] - rb);
+                }
+            }
+            const uint64_t b = __shfl_sync(kFull, rb, r);
+            const uint32_t len = __shfl_sync(kFull, rlen, r);
+            for (uint32_t p = 0; p < len; p += 128) {
+                uint32_t y[4];
 #pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    const uint32_t y = h ? y1 : y0;
-                    if (y <= lmax) {
-                        const uint32_t j = lower_bound_smem(sL, D, y);
-                        if (sL[j] == y) {
-                            if (K == 3) {
-                                acc += 1;
-                                if (WORK && sink.per_arc) atomicAdd(&sink.per_arc[base + i], 1ull);
-                            } else {
-                                atomicOr(&rows[i * RS + (j >> 5)], 1u << (j & 31));
-                                tri &= j > i;
-                            }
+                for (int h = 0; h < 4; h++) {
+                    const uint32_t q = p + 32 * h + lane;
+                    y[h] = q < len ? dag_cols[b + q] : 0xffffffffu;
+                }
+                if (__shfl_sync(kFull, y[0], 0) > lmax) break;
+#pragma unroll
+                for (int h = 0; h < 4; h++) {
+                    bool hit = win.has(y[h]);
+                    uint32_t j = 0;
+                    if (K > 3 && hit) j = win.place(y[h]);
+                    if (win.nlow && y[h] < win.base) {
+                        j = lower_bound_smem(sL, win.nlow, y[h]);
+                        hit = j < win.nlow && sL[j] == y[h];
+                    }
+                    if (K == 3) {
+                        acc += hit;
+                        if (WORK && sink.per_arc && hit) atomicAdd(&sink.per_arc[base + i], 1ull);
+                    } else {
+                        tri &= !hit || j > i;
+                        for (uint32_t left = __ballot_sync(kFull, hit); left;) {
+                            const uint32_t jw = __shfl_sync(kFull, j >> 5, __ffs(left) - 1);
+                            const bool in = hit && (j >> 5) == jw;
+                            const uint32_t word = __reduce_or_sync(kFull, in ? 1u << (j & 31u) : 0u);
+                            if (lane == 0) rows[i * RS + jw] |= word;
+                            left &= ~__ballot_sync(kFull, in);
                         }
                     }
                 }
@@ -1508,8 +1628,8 @@ struct Timer {
 };
 
 template <int K, bool WORK>
-static cudaError_t launch_mid(uint32_t grid_cap, uint32_t block_cap, uint32_t dcap,
-                              uint32_t compact_max, uint32_t split_min, const HelpTable &ht,
+static cudaError_t launch_mid(uint32_t grid_cap, uint32_t block_cap, int low, uint32_t dcap,
+                              uint32_t window, uint32_t compact_max, uint32_t split_min, const HelpTable &ht,
                               uint32_t warps, size_t smem, const uint64_t *dag_off,
                               const uint32_t *dag_cols, const uint32_t *mid_list,
                               const CountStats *st, uint32_t *next, unsigned long long *result,
@@ -1538,8 +1658,8 @@ static cudaError_t launch_mid(uint32_t grid_cap, uint32_t block_cap, uint32_t dc
     if (block_cap && grid > block_cap) grid = block_cap;
     if (grid > (uint32_t)num_sms * kMidBlocksPerSmCap) grid = (uint32_t)num_sms * kMidBlocksPerSmCap;
     *grid_out = grid;
-    k_count_mid<K, WORK><<<grid, warps * 32, smem, s>>>(dag_off, dag_cols, mid_list, st, next, dcap,
-                                                        compact_max, split_min, ht, result, sink,
+    k_count_mid<K, WORK><<<grid, warps * 32, smem, s>>>(dag_off, dag_cols, mid_list, st, next, low, dcap,
+                                                        window, compact_max, split_min, ht, result, sink,
                                                         work, block_ns, budget, err);
     note_launches(1);
     return cudaGetLastError();
@@ -1557,8 +1677,6 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
     cudaError_t e = cudaSuccess;
     const CountPlan &plan = run.plan;
     if (hs.n_mid) {
-        const uint32_t dcap = (hs.max_mid + 31) & ~31u;
-        const uint32_t rs = (dcap / 32) | 1;
         int smem_cap = 0, dev = 0;
         cudaGetDevice(&dev);
         if ((e = cudaDeviceGetAttribute(&smem_cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)))
@@ -1566,32 +1684,48 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
         smem_cap -= (int)kMidStaticSmem;
         // k = 4 ends at R = 2 and re-encodes no set: its warps need no room for one
         const uint32_t compact_max = K >= 5 ? plan.compact_max : 0u;
-        auto smem_for = [&](uint32_t warps) {
-            return ((size_t)dcap +
-                    (K > 3 ? (size_t)dcap * rs + (size_t)warps * warp_scratch_words(dcap, compact_max) : 0)) *
-                   sizeof(uint32_t);
-        };
-        uint32_t warps = plan.warps_per_cta > (uint32_t)kMidMaxWarps ? kMidMaxWarps : plan.warps_per_cta;
-        while (warps > 1 && smem_for(warps) > (size_t)smem_cap) warps--;
         Timer t(run.time_kernels, s);
         unsigned long long *block_ns = run.balance ? aux.block_ns : nullptr;
         uint32_t grid = 0;
-        // the instrumented kernel also serves the per-arc debug output (its code is compiled out
-        // of the plain kernel)
-        if (run.count_work || run.sink.per_arc) {
-            if constexpr (K <= (int)kInstrumentedMaxK)
-                e = launch_mid<K, true>(hs.n_mid, plan.max_blocks, dcap, compact_max, plan.split_min,
-                                        aux.help, warps, smem_for(warps), dag_off, dag_cols, mid_list, st,
-                                        next + 0, result, run.sink, work, block_ns, aux.budget, &grid, err,
-                                        s, num_sms);
-            else
-                e = cudaErrorNotSupported;  // refused by citron_count_ex before any launch
-        } else
-            e = launch_mid<K, false>(hs.n_mid, plan.max_blocks, dcap, compact_max, plan.split_min,
-                                     aux.help, warps, smem_for(warps), dag_off, dag_cols, mid_list, st,
-                                     next + 0, result, run.sink, work, block_ns, aux.budget, &grid, err, s,
-                                    num_sms);
-        if (e) return e;
+        const bool parts = K <= kPartsMaxK;
+        for (int low = 0; low < (parts ? 2 : 1); low++) {
+            const uint32_t n_roots = !parts ? hs.n_mid : !low ? hs.n_high : hs.bound ? hs.n_mid : hs.n_mid - hs.n_high;
+            if (!n_roots) continue;
+            const uint32_t dmax = low && hs.max_mid > kLowMax ? kLowMax : hs.max_mid;
+            const uint32_t dcap = (dmax + 31) & ~31u, rs = (dcap / 32) | 1;
+            uint32_t warps = plan.warps_per_cta > (uint32_t)kMidMaxWarps ? kMidMaxWarps : plan.warps_per_cta;
+            if (low && warps > kLowWarps) warps = kLowWarps;
+            auto scratch = [&](uint32_t nw) {  // words for the warps' lists and buffers
+                return K > 3 ? (size_t)nw * warp_scratch_words(dcap, compact_max) : (size_t)kMidWindow / 32;
+            };
+            auto smem_for = [&](uint32_t nw) {
+                return ((size_t)dcap + (K > 3 ? (size_t)dcap * rs : 0) + scratch(nw)) * sizeof(uint32_t);
+            };
+            while (warps > 1 && smem_for(warps) > (size_t)smem_cap) warps--;
+            // the window's bitmap and first places (k > 3) have to fit the scratch
+            uint32_t window = kMidWindow;
+            while ((size_t)window / 32 + (K > 3 ? window / 64 : 0) > scratch(warps)) window /= 2;
+            unsigned long long *ns = grid ? nullptr : block_ns;  // timed: the first launch's blocks
+            uint32_t this_grid = 0;
+            uint32_t *queue = next + (low ? 3 : 0);
+            // the instrumented kernel also serves the per-arc debug output (its code is compiled
+            // out of the plain kernel)
+            if (run.count_work || run.sink.per_arc) {
+                if constexpr (K <= (int)kInstrumentedMaxK)
+                    e = launch_mid<K, true>(n_roots, plan.max_blocks, low, dcap, window, compact_max, plan.split_min,
+                                            aux.help, warps, smem_for(warps), dag_off, dag_cols, mid_list, st,
+                                            queue, result, run.sink, work, ns, aux.budget, &this_grid, err,
+                                            s, num_sms);
+                else
+                    e = cudaErrorNotSupported;  // refused by citron_count_ex before any launch
+            } else
+                e = launch_mid<K, false>(n_roots, plan.max_blocks, low, dcap, window, compact_max, plan.split_min,
+                                         aux.help, warps, smem_for(warps), dag_off, dag_cols, mid_list, st,
+                                         queue, result, run.sink, work, ns, aux.budget, &this_grid, err, s,
+                                         num_sms);
+            if (e) return e;
+            if (!grid) grid = this_grid;
+        }
         t.stop();
         run.kernel_ms[1] = t.ms();
         if (block_ns && grid) {
