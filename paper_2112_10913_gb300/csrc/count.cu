@@ -251,6 +251,7 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
     uint32_t *list_scratch = (uint32_t *)(c.base + c.used);
     const size_t list_words = c.cap > c.used ? (c.cap - c.used) / sizeof(uint32_t) : 0;
     unsigned long long *work = result + 1;
+    if (!run.plan.small_max) run.plan.small_max = small_default(k);
     const CountPlan &plan = run.plan;
 
     cudaError_t e;
@@ -329,6 +330,7 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     uint32_t *list_scratch = (uint32_t *)(c.base + c.used);
     const size_t list_words = c.cap > c.used ? (c.cap - c.used) / sizeof(uint32_t) : 0;
     unsigned long long *work = result + 1;
+    if (!run.plan.small_max) run.plan.small_max = small_default(k);
     const CountPlan &plan = run.plan;
     cudaError_t e;
     if ((e = cudaMemsetAsync(st, 0, sizeof(CountStats), s))) return e;

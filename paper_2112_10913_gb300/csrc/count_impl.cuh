@@ -14,8 +14,7 @@ constexpr int kMaxK = CITRON_MAX_K;
 constexpr uint32_t kBitmapCap = 1024;  // largest root handled by the bitmap path
 constexpr int kSmallWarps = 8;         // warps per block of k_count_small
 constexpr int kListWarps = 4;          // warps per block of k_count_list
-constexpr uint32_t kSmallWindow = 16384;  // ids in a warp's membership bitmap (k_count_small), and ...
-constexpr uint32_t kMidWindow = 32768;    // ... in a block's (k_count_mid)
+constexpr uint32_t kMidWindow = 32768;  // ids in a block's membership bitmap (k_count_mid)
 
 struct CountStats {
     uint32_t n_small, n_mid, n_big;
@@ -99,23 +98,21 @@ struct Window {
     }
 };
 
+// One warp per root; the D (D - 1) / 2 pairs of its members are looked up (binary search of one
+// member in the other's list).  Scanning the members' whole lists instead costs their length:
+// R-MAT 20, roots of 9..32 out-neighbours: 3061 list entries per root on average, 116 pairs.
 template <int K>
 __global__ __launch_bounds__(kSmallWarps * 32) void k_count_small(
     const uint64_t *__restrict__ dag_off, const uint32_t *__restrict__ dag_cols,
     const uint32_t *__restrict__ list, const CountStats *st, unsigned long long *result,
     RootSink sink, Budget budget, uint32_t *err)
 {
-    __shared__ uint32_t sL[kSmallWarps][32];
-    __shared__ uint32_t s_bits[kSmallWarps][kSmallWindow / 32];
-    __shared__ uint8_t s_first[kSmallWarps][kSmallWindow / 32];
+    // per member: its id, its list and the list's first entry; its row as it fills
+    __shared__ uint64_t s_rb[kSmallWarps][32];
+    __shared__ uint32_t s_x[kSmallWarps][32], s_len[kSmallWarps][32], s_min[kSmallWarps][32], s_row[kSmallWarps][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t nlist = st->n_small;
     const uint32_t gw = blockIdx.x * kSmallWarps + w, nwarps = gridDim.x * kSmallWarps;
-    Window<uint8_t> win;
-    win.bits = s_bits[w];
-    win.first = s_first[w];
-    for (uint32_t i = lane; i < kSmallWindow / 32; i += 32) s_bits[w][i] = 0;
-    __syncwarp();
     unsigned long long total = 0;
     for (uint32_t idx = gw; idx < nlist; idx += nwarps) {
         int stop = 0;
@@ -124,51 +121,80 @@ __global__ __launch_bounds__(kSmallWarps * 32) void k_count_small(
         const uint32_t u = list[idx];
         const uint64_t base = dag_off[u];
         const uint32_t D = (uint32_t)(dag_off[u + 1] - base);
-        const uint32_t x = lane < D ? dag_cols[base + lane] : 0xffffffffu;
-        uint64_t rb = 0, re = 0;
         if (lane < D) {
-            rb = dag_off[x];
-            re = dag_off[x + 1];
+            const uint32_t x = dag_cols[base + lane];
+            const uint64_t rb = dag_off[x];
+            const uint32_t len = (uint32_t)(dag_off[x + 1] - rb);
+            s_x[w][lane] = x;
+            s_rb[w][lane] = rb;
+            s_len[w][lane] = len;
+            s_min[w][lane] = len ? dag_cols[rb] : 0xffffffffu;
         }
-        sL[w][lane] = x;
-        const uint32_t lmax = __shfl_sync(kFull, x, D - 1);
-        win.base = lmax >= kSmallWindow ? lmax - (kSmallWindow - 1) : 0u;
-        win.span = lmax - win.base + 1;
-        const bool in_win = lane < D && x >= win.base;
-        win.nlow = __popc(__ballot_sync(kFull, lane < D && !in_win));
-        const uint32_t xw = in_win ? (x - win.base) >> 5 : 0xffffffffu;
-        const uint32_t prev = __shfl_up_sync(kFull, xw, 1);
-        if (in_win) {
-            atomicOr(&win.bits[xw], 1u << ((x - win.base) & 31u));
-            if (lane == 0 || prev != xw) win.first[xw] = (uint8_t)lane;
-        }
+        s_row[w][lane] = 0;
         __syncwarp();
-        uint32_t myrow = 0;
-        for (uint32_t i = 0; i < D; i++) {
-            const uint64_t b = __shfl_sync(kFull, rb, i);
-            const uint32_t len = (uint32_t)(__shfl_sync(kFull, re, i) - b);
-            uint32_t bits = 0;
-            // four loads in flight per lane
-            for (uint32_t p = lane; __any_sync(kFull, p < len); p += 128) {
-                uint32_t y[4];
+        // Every pair of members once, two per lane and round: pair p is (c, c + r + 1 mod D) with
+        // r = p / D, c = p mod D.  An arc between them is in the row of one of the two: the one
+        // of lower index if rows only hold larger ids (a relabelled DAG), else either.
+        const uint32_t npairs = D * (D - 1) / 2;
+        const float inv = 1.0f / (float)D;
+        for (uint32_t p0 = 0; p0 < npairs; p0 += 64) {
+            uint32_t src[2], dst[2], lo[2], left[2];
+            const uint32_t *row[2];
+            uint32_t want[2];
 #pragma unroll
-                for (int h = 0; h < 4; h++) y[h] = p + 32 * h < len ? dag_cols[b + p + 32 * h] : 0xffffffffu;
-                if (__shfl_sync(kFull, y[0], 0) > lmax) break;
+            for (int h = 0; h < 2; h++) {
+                const uint32_t p = p0 + 32 * h + lane;
+                const uint32_t r = (uint32_t)(((float)p + 0.5f) * inv), c = p - r * D;
+                const uint32_t o = c + r + 1 >= D ? c + r + 1 - D : c + r + 1;
+                const bool in = p < npairs;
+                src[h] = in ? min(c, o) : 0u;
+                dst[h] = in ? max(c, o) : 0u;
+                lo[h] = 0;
+                left[h] = in ? s_len[w][src[h]] : 0u;
+                row[h] = dag_cols + s_rb[w][src[h]];
+                want[h] = s_x[w][dst[h]];
+            }
+            for (;;) {
+                // both searches step together, so that two loads are in flight
+                while (left[0] | left[1]) {
+                    uint32_t y[2];
 #pragma unroll
-                for (int h = 0; h < 4; h++) {
-                    if (win.has(y[h])) {
-                        bits |= 1u << win.place(y[h]);
-                    } else if (win.nlow && y[h] < win.base) {
-                        const uint32_t j = lower_bound_smem(sL[w], win.nlow, y[h]);
-                        if (j < win.nlow && sL[w][j] == y[h]) bits |= 1u << j;
+                    for (int h = 0; h < 2; h++) y[h] = left[h] ? row[h][lo[h] + (left[h] >> 1)] : 0u;
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const uint32_t half = left[h] >> 1;
+                        if (left[h] && y[h] == want[h]) {
+                            atomicOr(&s_row[w][src[h]], 1u << dst[h]);
+                            left[h] = 0;
+                            dst[h] = src[h];  // found
+                        } else if (y[h] < want[h]) {
+                            lo[h] += left[h] ? half + 1 : 0u;
+                            left[h] -= left[h] ? half + 1 : 0u;
+                        } else {
+                            left[h] = half;
+                        }
                     }
                 }
+                // the other direction, where the row's ids reach down to it
+                bool more = false;
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    if (dst[h] > src[h] && s_min[w][dst[h]] <= s_x[w][src[h]]) {
+                        const uint32_t t = src[h];
+                        src[h] = dst[h];
+                        dst[h] = t;
+                        lo[h] = 0;
+                        left[h] = s_len[w][src[h]];
+                        row[h] = dag_cols + s_rb[w][src[h]];
+                        want[h] = s_x[w][t];
+                        more = true;
+                    }
+                }
+                if (!more) break;
             }
-            bits = __reduce_or_sync(kFull, bits);
-            if (lane == i) myrow = bits;
         }
         __syncwarp();
-        if (in_win) win.bits[xw] = 0;
+        const uint32_t myrow = s_row[w][lane];
         unsigned long long acc = 0;
         const uint32_t all = D == 32 ? kFull : ((1u << D) - 1);
         if (sink.per_arc) {
