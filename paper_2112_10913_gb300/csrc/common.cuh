@@ -304,6 +304,7 @@ struct CountRun {
     bool balance = false;                    // record when each bitmap-path block starts and ends
     unsigned long long budget_ns = 0;        // device time the count may take (0: no limit)
     unsigned long long work = 0;             // out: word operations (AND + POPC of 32-bit words)
+    uint32_t dev_error = 0;                  // out: the device error word after the count
     float kernel_ms[3] = {0, 0, 0};          // out: warp-register, bitmap, sorted-list kernels
     float busy_ms[2] = {0, 0};               // out: bitmap kernel's span (first start to last end)
                                              // and tail (first block end to last block end)

@@ -231,13 +231,14 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
                       CountRun &run, uint32_t *err, Carver &c, cudaStream_t s, int num_sms,
                       unsigned long long *h_result)
 {
+    // (everything a count has to clear comes first, so that one memset does it)
     CountStats *st = c.take<CountStats>(1);
-    unsigned long long *result = c.take<unsigned long long>(4);  // total, work, budget clock
+    unsigned long long *result = c.take<unsigned long long>(4);  // total, work, budget clock, error word
     uint32_t *next = c.take<uint32_t>(8);
+    uint32_t *hist = c.take<uint32_t>(kBitmapCap + 2);
     uint32_t *small_list = c.take<uint32_t>((size_t)n + 1);
     uint32_t *mid_list = c.take<uint32_t>((size_t)n + 1);
     uint32_t *big_list = c.take<uint32_t>((size_t)n + 1);
-    uint32_t *hist = c.take<uint32_t>(kBitmapCap + 2);
     uint32_t *cursor = c.take<uint32_t>(kBitmapCap + 2);
     MidAux aux;
     aux.help.slots = c.take<HeavySlot>(kHelpSlots);
@@ -255,12 +256,9 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
     const CountPlan &plan = run.plan;
 
     cudaError_t e;
-    if ((e = cudaMemsetAsync(st, 0, sizeof(CountStats), s))) return e;
-    if ((e = cudaMemsetAsync(result, 0, 4 * sizeof(unsigned long long), s))) return e;
+    if ((e = cudaMemsetAsync(st, 0, (char *)(hist + kBitmapCap + 2) - (char *)st, s))) return e;
     if ((e = seed_totals(result, 1, s))) return e;
-    if ((e = cudaMemsetAsync(next, 0, 8 * sizeof(uint32_t), s))) return e;
-    if ((e = cudaMemsetAsync(hist, 0, (kBitmapCap + 2) * sizeof(uint32_t), s))) return e;
-    if ((e = cudaMemsetAsync(aux.help.slots, 0, kHelpSlots * sizeof(HeavySlot), s))) return e;
+    if (k >= 6 && (e = cudaMemsetAsync(aux.help.slots, 0, kHelpSlots * sizeof(HeavySlot), s))) return e;
     const uint32_t need = k - 1;
     const uint32_t blocks = (n + 255) / 256;
     if (n) {
@@ -296,28 +294,33 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
     }
 #undef CITRON_CASE
     if (e) return e;
-    unsigned long long out[2] = {0, 0};
+    // the error word goes with the totals: one copy and one wait instead of two
+    unsigned long long out[4] = {0, 0, 0, 0};
+    if ((e = cudaMemcpyAsync(result + 3, err, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s))) return e;
     if ((e = cudaMemcpyAsync(out, result, sizeof(out), cudaMemcpyDeviceToHost, s))) return e;
     if ((e = cudaStreamSynchronize(s))) return e;
     *h_result = out[0];
     run.work = out[1];
+    run.dev_error = (uint32_t)out[3];
     return cudaSuccess;
 }
 
 // Capture-safe variant of run_count: no host synchronisation.  Launch configurations come from
 // upper bounds (every row a root, the largest row max_outdeg) instead of the classification's
 // statistics; the kernels read the real list sizes on the device and exit when they are done.
+// *d_total (optional) is where the grand total will be.
 cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_cols, uint32_t k,
                             uint32_t max_outdeg, CountRun &run, uint32_t *err, Carver &c,
-                            cudaStream_t s, int num_sms)
+                            cudaStream_t s, int num_sms, unsigned long long **d_total)
 {
+    // (everything a count has to clear comes first, so that one memset does it)
     CountStats *st = c.take<CountStats>(1);
-    unsigned long long *result = c.take<unsigned long long>(4);  // total, work, budget clock
+    unsigned long long *result = c.take<unsigned long long>(4);  // total, work, budget clock, error word
     uint32_t *next = c.take<uint32_t>(8);
+    uint32_t *hist = c.take<uint32_t>(kBitmapCap + 2);
     uint32_t *small_list = c.take<uint32_t>((size_t)n + 1);
     uint32_t *mid_list = c.take<uint32_t>((size_t)n + 1);
     uint32_t *big_list = c.take<uint32_t>((size_t)n + 1);
-    uint32_t *hist = c.take<uint32_t>(kBitmapCap + 2);
     uint32_t *cursor = c.take<uint32_t>(kBitmapCap + 2);
     MidAux aux;
     aux.help.slots = c.take<HeavySlot>(kHelpSlots);
@@ -333,11 +336,9 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     if (!run.plan.small_max) run.plan.small_max = small_default(k);
     const CountPlan &plan = run.plan;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(st, 0, sizeof(CountStats), s))) return e;
-    if ((e = cudaMemsetAsync(result, 0, 4 * sizeof(unsigned long long), s))) return e;
-    if ((e = cudaMemsetAsync(next, 0, 8 * sizeof(uint32_t), s))) return e;
-    if ((e = cudaMemsetAsync(hist, 0, (kBitmapCap + 2) * sizeof(uint32_t), s))) return e;
-    if ((e = cudaMemsetAsync(aux.help.slots, 0, kHelpSlots * sizeof(HeavySlot), s))) return e;
+    if ((e = cudaMemsetAsync(st, 0, (char *)(hist + kBitmapCap + 2) - (char *)st, s))) return e;
+    if (k >= 6 && (e = cudaMemsetAsync(aux.help.slots, 0, kHelpSlots * sizeof(HeavySlot), s))) return e;
+    if (d_total) *d_total = result;
     if (n == 0 || max_outdeg < k - 1) return cudaSuccess;
     const uint32_t need = k - 1;
     const uint32_t blocks = (n + 255) / 256;
