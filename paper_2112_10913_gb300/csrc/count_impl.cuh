@@ -377,37 +377,44 @@ __device__ __forceinline__ uint32_t member_bits(const WarpCtx &x, uint32_t bits,
     return compress_with(bits, m, mv);
 }
 
-// Complement rows of the s <= 128 members of the candidate set (words in cbuf, members in elem,
-// non-zero words [clo, chi); triangular layout) in mbuf, one uint4 per row.  Each round of 32
-// members streams its packed row words: the member prefix of a candidate word is the same on every
-// lane, so the words fill and leave at warp-uniform places.  Returns the complement's bits written
-// by this lane (in all, twice its edges).
+// Complement rows of the members 32a .. 32a + 31 of a set of s members (words in cbuf, members in
+// elem, masks prepared, no words from chi on; triangular layout) in m32 (rows of S per chunk), from
+// their own blocks on, and the mirror images below.  The packed row words are streamed: the member
+// prefix of a candidate word is the same on every lane, so the words fill and leave at warp-uniform
+// places.  Returns the complement's bits written by this lane (over all rounds, twice its edges).
+// (Setting the missing pairs one by one in both rows instead: k = 5 on R-MAT 20 65 ms against 33.)
+__device__ __forceinline__ uint32_t complement_round(const WarpCtx &x, uint32_t *m32, uint32_t S, uint32_t s, uint32_t a,
+                                                     int chi, int lane)
+{
+    const uint32_t i0 = a << 5, i = i0 + lane;
+    const uint32_t *row = x.rows + (uint32_t)x.elem[i < s ? i : s - 1] * x.RS;
+    uint32_t bits = 0;
+    // rows hold bits above their own member only: start at the word of the first member
+    int w = (int)(x.elem[i0] >> 5);
+    uint32_t ow = x.mv[160 + w] >> 5, sh = x.mv[160 + w] & 31u, cur = 0;
+    for (; w < chi; w++) {
+        const uint32_t m = x.cbuf[w];
+        if (!m) continue;
+        const uint32_t piece = member_bits(x, row[w], m, w);
+        cur |= piece << sh;
+        const uint32_t end = sh + __popc(m);
+        if (end >= 32) {
+            if (ow >= a) bits += put_block(m32, S, s, a, ow, cur, lane);
+            ow++;
+            cur = sh ? piece >> (32 - sh) : 0u;
+        }
+        sh = end & 31u;
+    }
+    if (sh && ow >= a) bits += put_block(m32, S, s, a, ow, cur, lane);
+    return bits;
+}
+
+// Complement rows of the s <= 128 members of a set by one warp, one uint4 per row in mbuf.
 __device__ __forceinline__ uint32_t build_complement(const WarpCtx &x, uint32_t s, int clo, int chi, int lane)
 {
     prepare_masks(x, clo, chi, lane);
-    const uint32_t nblk = (s + 31) >> 5;
     uint32_t bits = 0;
-    for (uint32_t a = 0; a < nblk; a++) {
-        const uint32_t i0 = a << 5, i = i0 + lane;
-        const uint32_t *row = x.rows + (uint32_t)x.elem[i < s ? i : s - 1] * x.RS;
-        // rows hold bits above their own member only: start at the word of the first member
-        int w = (int)(x.elem[i0] >> 5);
-        uint32_t ow = x.mv[160 + w] >> 5, sh = x.mv[160 + w] & 31u, cur = 0;
-        for (; w < chi; w++) {
-            const uint32_t m = x.cbuf[w];
-            if (!m) continue;
-            const uint32_t piece = member_bits(x, row[w], m, w);
-            cur |= piece << sh;
-            const uint32_t end = sh + __popc(m);
-            if (end >= 32) {
-                if (ow >= a) bits += put_block(x.mbuf, 0, s, a, ow, cur, lane);
-                ow++;
-                cur = sh ? piece >> (32 - sh) : 0u;
-            }
-            sh = end & 31u;
-        }
-        if (sh && ow >= a) bits += put_block(x.mbuf, 0, s, a, ow, cur, lane);
-    }
+    for (uint32_t a = 0; a << 5 < s; a++) bits += complement_round(x, x.mbuf, 0, s, a, chi, lane);
     __syncwarp();
     return bits;
 }
@@ -715,9 +722,9 @@ __device__ __forceinline__ void dense_dfs(const WarpCtx &x, const CompSet &cs, u
                     __syncwarp();
                     Bs[lane] = nc;
                     __syncwarp();
-                    const CompCount t = comp3_wide<WORK>(M, cs.S, cs.nch, Bs, m, ng, 0, 1, lane);
+                    const CompCount t = comp3_wide<false, WORK>(M, cs.S, cs.nch, Bs, m, ng, 0, 1, lane);
                     if (WORK) work += t.work;
-                    n += n3_finish(m, __reduce_add_sync(kFull, t.n));
+                    n += n3_finish(m, __reduce_add_sync(kFull, t.n), false);
                 }
             } else {
                 unsigned long long sl = o.sl;
@@ -1002,6 +1009,7 @@ struct GroupShared {
 struct Group {
     GroupShared *sh;
     uint32_t *buf;  // the members' scratch buffers as one
+    uint32_t *lists;  // the first warp's lists
     uint32_t gw, gi, bar;
 
     __device__ __forceinline__ void sync() const
@@ -1023,54 +1031,69 @@ __device__ __forceinline__ uint32_t select_member(uint32_t c, uint32_t r)
 }
 
 // R-cliques (R >= 3) of a row c (lane word, more than 128 members; triangular layout), counted by
-// the warps of a group together: the complement rows are built 32 x 32 block by block, then R = 3
+// the warps of a group together: they build the complement rows (32 members per round), then R = 3
 // and R = 4 are one pass over (32 members, chunk of 128 codegrees) units, and for R >= 5 the warps
 // take the members one at a time and walk down from there.  Every warp of the group calls this.
+// k = 5 (R = 3), k_count_mid: R-MAT 20 32.8 ms, Chung-Lu 4M 120.1 ms when every warp made the lists for
+// itself, the rows were built 32 x 32 block by block and each pair of a triangle's edges was seen
+// twice; 32.0 and 114.3 with the pairs seen once and sets sparser than one half counted as they
+// are; 30.9 and 107.0 with shared lists and whole rounds.
 template <int R, bool WORK>
 __device__ __forceinline__ void wide_row(const WarpCtx &x, const Group &g, uint32_t c, int lane,
                                          unsigned long long &acc, unsigned long long &work)
 {
-    int clo, chi;
-    const uint32_t s = compact(x, c, lane, clo, chi);
-    prepare_masks(x, clo, chi, lane);
+    // the set's lists are made once, in the first warp's scratch: its words and masks by that warp,
+    // the members by all
+    WarpCtx y = x;
+    y.cbuf = g.lists;
+    y.mv = g.lists + 32;
+    y.elem = reinterpret_cast<uint16_t *>(g.lists + 32 + kMaskWords + kNbhdList);
+    const uint32_t nz = __ballot_sync(kFull, c != 0);
+    const int chi = 32 - __clz(nz);
+    const uint32_t pc = __popc(c), incl = warp_incl_scan(pc), s = __shfl_sync(kFull, incl, 31);
+    if (g.gi == 0) {
+        uint32_t mv[5];
+        compress_masks(c, mv);
+        y.cbuf[lane] = c;
+#pragma unroll
+        for (int i = 0; i < 5; i++) y.mv[i * 32 + lane] = mv[i];
+        y.mv[160 + lane] = incl - pc;
+    }
+    for (uint32_t rest = nz; rest; rest &= rest - 1) {
+        const int w = __ffs(rest) - 1;
+        const uint32_t m = __shfl_sync(kFull, c, w), at = __shfl_sync(kFull, incl - pc, w);
+        if (((uint32_t)w & (g.gw - 1)) == g.gi && ((m >> lane) & 1u))
+            y.elem[at + __popc(m & lanemask_lt())] = (uint16_t)((w << 5) + lane);
+    }
+    g.sync();
     const CompSet cs = {g.buf, s, (s + 127) >> 7};
     const uint32_t nblk = (s + 31) >> 5;
-    uint32_t bits = 0, u = 0;
+    uint32_t bits = 0;
+    // rounds get shorter: dealt forth and back
     for (uint32_t a = 0; a < nblk; a++) {
-        const uint32_t i = (a << 5) + lane;
-        const uint32_t *row = x.rows + (uint32_t)x.elem[i < s ? i : s - 1] * x.RS;
-        for (uint32_t ow = a; ow < nblk; ow++) {
-            if ((u++ & (g.gw - 1)) != g.gi) continue;
-            const uint32_t j0 = ow << 5, j1 = min(j0 + 31, s - 1);
-            uint32_t cur = 0;
-            for (int w = (int)(x.elem[j0] >> 5); w <= (int)(x.elem[j1] >> 5); w++) {
-                const uint32_t m = x.cbuf[w];
-                if (!m) continue;
-                const uint32_t piece = member_bits(x, row[w], m, w);
-                const int at = (int)x.mv[160 + w] - (int)j0;  // > -32
-                cur |= at >= 0 ? piece << at : piece >> -at;
-            }
-            bits += put_block(cs.m32, s, s, a, ow, cur, lane);
-        }
+        const uint32_t p = a & (g.gw - 1);
+        if ((a & g.gw ? g.gw - 1 - p : p) == g.gi) bits += complement_round(y, cs.m32, s, s, a, chi, lane);
     }
     bits = __reduce_add_sync(kFull, bits);
     if (lane == 0) atomicAdd(&g.sh->mbar, bits);
-    __syncwarp();
-    x.cbuf[lane] = word_mask(s, lane);
     g.sync();
+    x.cbuf[lane] = word_mask(s, lane);
+    __syncwarp();
     const bool dense = 2 * g.sh->mbar <= s * (s - 1);
     const uint4 *M = reinterpret_cast<const uint4 *>(cs.m32);
     bool counted = false;
-    if (dense) {
-        if constexpr (R == 3) {
-            CompCount o = comp3_wide<WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, lane);
-            if (WORK) work += o.work;
-            o.n = __reduce_add_sync(kFull, o.n);
-            if (lane == 0) atomicAdd(&g.sh->sd, o.n);
-            g.sync();
-            if (g.gi == 0 && lane == 0) add_acc(acc, n3_finish(s, g.sh->sd), x.err);
-            counted = true;
-        } else if constexpr (R == 4) {
+    if constexpr (R == 3) {
+        // either side of the pairs: the complement's triangles and Goodman's identity, or the set's
+        CompCount o = dense ? comp3_wide<false, WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, lane)
+                            : comp3_wide<true, WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, lane);
+        if (WORK) work += o.work;
+        o.n = __reduce_add_sync(kFull, o.n);
+        if (lane == 0) atomicAdd(&g.sh->sd, o.n);
+        g.sync();
+        if (g.gi == 0 && lane == 0) add_acc(acc, n3_finish(s, g.sh->sd, !dense), x.err);
+        counted = true;
+    } else if (dense) {
+        if constexpr (R == 4) {
             CompSums o = comp4_wide<WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, x.mv, lane);
             if (WORK) work += o.work;
             const bool over = __any_sync(kFull, o.over);
@@ -1106,10 +1129,10 @@ __device__ __forceinline__ void wide_row(const WarpCtx &x, const Group &g, uint3
                         __syncwarp();
                         x.cbuf[lane] = nc;
                         __syncwarp();
-                        const CompCount o = comp3_wide<WORK>(M, s, cs.nch, x.cbuf, m, nblk, 0, 1, lane);
+                        const CompCount o = comp3_wide<false, WORK>(M, s, cs.nch, x.cbuf, m, nblk, 0, 1, lane);
                         if (WORK) work += o.work;
                         const uint32_t sum = __reduce_add_sync(kFull, o.n);
-                        if (lane == 0) add_acc(acc, n3_finish(m, sum), x.err);
+                        if (lane == 0) add_acc(acc, n3_finish(m, sum, false), x.err);
                     } else {
                         dense_dfs<R - 1, 0, WORK>(x, cs, nc, m, lane, acc, work);
                     }
@@ -1386,6 +1409,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                     g.bar = 1 + w0 / 2;
                     g.sh = &s_group[w0 / 2];
                     g.buf = bufs + (size_t)w0 * buf_words;
+                    g.lists = lists + (size_t)w0 * warp_list_words(dcap, compact_max);
                     for (;;) {
                         if (g.gi == 0 && lane == 0) {
                             uint32_t v = count;

@@ -401,27 +401,40 @@ __device__ __noinline__ CompCount comp_nbhd(const uint4 *M, uint32_t S, uint32_t
 
 // ---- Narrow sets (at most 128 members): one uint4 per complement row --------------------------
 
-template <int CW, bool WORK, int Q>
-__device__ __forceinline__ void comp3_word(const uint4 *M, const uint32_t (&B)[CW], uint32_t s, int lane,
-                                           uint32_t &lin, uint32_t &ones, uint32_t &twice, uint32_t &work)
+// Adjacent pairs (x, y) inside D (CW words), x in D's word T (bits b): y in a later word into `once`,
+// y in the same word into `twice` (both orders).  Two members x per step, the highest and the
+// lowest.  INV: the rows hold the complement of the adjacency meant (x itself is then counted once
+// in `twice`; the caller takes that off).
+struct PairSums {
+    uint32_t ones, once, ones2, twice;
+    __device__ __forceinline__ uint32_t both() const { return 2 * (once + __popc(ones)) + twice + __popc(ones2); }
+};
+
+template <int CW, int T, bool INV>
+__device__ __forceinline__ void pair_word(const uint4 *M, const uint32_t (&D)[CW], uint32_t b, uint32_t base, PairSums &p)
 {
-    if constexpr (Q < CW) {
-        if ((B[Q] >> lane) & 1u) {
-            uint32_t h[CW], d = 0;
-            load_row<CW>(M, (uint32_t)(Q << 5) + lane, h);
+    while (b) {
+        const uint32_t b1 = 31u - __clz(b), lb = b & (0u - b), b2 = 31u - __clz(lb);
+        const uint32_t two = b1 == b2 ? 0u : kFull;
+        b &= ~((1u << b1) | lb);
+        uint32_t r1[CW], r2[CW];
+        load_row<CW>(M, base + b1, r1);
+        load_row<CW>(M, base + b2, r2);
 #pragma unroll
-            for (int t = 0; t < CW; t++) {
-                h[t] &= B[t];
-                d += __popc(h[t]);
-                if (t < Q) h[t] = 0;
-            }
-            h[Q] &= above_bit(lane);
-            lin += d * (s - 1 - d);
-            if (WORK) work += CW * (d + 1);
-#pragma unroll
-            for (int t = Q; t < CW; t++) leaf_word<CW, Q>(M, h, h[t], (uint32_t)t << 5, ones, twice);
+        for (int w = T < 0 ? 0 : T; w < CW; w++) {
+            const uint32_t x1 = D[w] & (INV ? ~r1[w] : r1[w]), x2 = D[w] & (INV ? ~r2[w] : r2[w]) & two;
+            if (w == T) csa_add(p.ones2, x1, x2, p.twice);
+            else csa_add(p.ones, x1, x2, p.once);
         }
-        comp3_word<CW, WORK, Q + 1>(M, B, s, lane, lin, ones, twice, work);
+    }
+}
+
+template <int CW, int T>
+__device__ __forceinline__ void pair_words(const uint4 *M, const uint32_t (&D)[CW], PairSums &p)
+{
+    if constexpr (T < CW) {
+        pair_word<CW, T, false>(M, D, D[T], (uint32_t)T << 5, p);
+        pair_words<CW, T + 1>(M, D, p);
     }
 }
 
@@ -430,11 +443,28 @@ __device__ __forceinline__ void comp3_word(const uint4 *M, const uint32_t (&B)[C
 template <int CW, bool WORK>
 __device__ __noinline__ CompCount comp3(const uint4 *M, const uint32_t *Bs, uint32_t s, int lane)
 {
-    uint32_t B[CW], lin = 0, ones = 0, twice = 0, work = 0;
+    uint32_t B[CW], lin = 0, work = 0;
+    PairSums p = {0, 0, 0, 0};
 #pragma unroll
     for (int t = 0; t < CW; t++) B[t] = Bs[t];
-    comp3_word<CW, WORK, 0>(M, B, s, lane, lin, ones, twice, work);
-    const uint32_t sum = __reduce_add_sync(kFull, lin + twice + __popc(ones));
+#pragma unroll 1
+    for (int q = 0; q < CW; q++) {
+        if ((Bs[q] >> lane) & 1u) {
+            uint32_t h[CW], d = 0;
+            load_row<CW>(M, (uint32_t)(q << 5) + lane, h);
+#pragma unroll
+            for (int t = 0; t < CW; t++) {
+                h[t] &= B[t];
+                d += __popc(h[t]);
+                h[t] &= t > q ? kFull : (t == q ? above_bit(lane) : 0u);
+            }
+            lin += d * (s - 1 - d);
+            if (WORK) work += CW * (d + 1);
+            pair_words<CW, 0>(M, h, p);
+        }
+        __syncwarp();
+    }
+    const uint32_t sum = __reduce_add_sync(kFull, lin + p.both());
     CompCount o;
     o.n = (s * (s - 1) * (s - 2) / 3 - sum) >> 1;
     o.work = WORK ? __reduce_add_sync(kFull, work) : 0u;
@@ -707,59 +737,71 @@ __device__ __forceinline__ unsigned long long n4_finish(uint32_t s32, uint32_t s
     return (s * (s - 1) * (s - 2) * (s - 3) / 6 - 2 * m * (s - 2) * (s - 3) + 2 * m * (m - 1) - 4 * s * (st / 6) + sl) >> 2;
 }
 
-// As comp4_wide, for N3: lane-partial sum of d(s-1-d) + 2 t over the warp's share.
-template <bool WORK>
+// As comp4_wide, for N3: lane-partial sum over the warp's share of d(s-1-d) + 2 t, or with INV, for a
+// set that is the sparse side itself, twice its triangles (n3_finish).
+template <bool INV, bool WORK>
 __device__ __noinline__ CompCount comp3_wide(const uint4 *M, uint32_t S, uint32_t nch, const uint32_t *Bs,
                                              uint32_t s, uint32_t ngroups, uint32_t u0, uint32_t ustep, int lane)
 {
     CompCount o = {0, 0};
     const uint4 *B4 = reinterpret_cast<const uint4 *>(Bs);
-    uint32_t ones = 0;
     const uint32_t nunits = ngroups * nch;
+    PairSums p = {0, 0, 0, 0};
+    uint32_t lin = 0;
     for (uint32_t u = u0; u < nunits; u += ustep) {
         const uint32_t g = u / nch, q = u - g * nch;
         const uint32_t v = (g << 5) + lane;
         if ((Bs[g] >> lane) & 1u) {
-            if ((v >> 7) == q) {
+            if (!INV && (v >> 7) == q) {
                 uint32_t d = 0;
                 for (uint32_t c = 0; c < nch; c++) {
                     const uint4 h = M[c * S + v], b = B4[c];
                     d += __popc(h.x & b.x) + __popc(h.y & b.y) + __popc(h.z & b.z) + __popc(h.w & b.w);
                 }
-                o.n += d * (s - 1 - d);
+                lin += d * (s - 1 - d);
                 if (WORK) o.work += 4 * nch;
             }
+            // v's later neighbours in chunk c
+            auto later = [&](uint32_t c, uint32_t (&h)[4]) {
+                const uint4 a = M[c * S + v], b = B4[c];
+                const uint32_t x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int t = 0; t < 4; t++) h[t] = (INV ? ~x[t] : x[t]) & y[t] & above_word(v, (c << 2) + t);
+            };
             if (q >= (g >> 2)) {
                 const uint4 *Mq = M + q * S;
-                const uint4 a = Mq[v], b = B4[q];
-                uint32_t hq[4] = {a.x & b.x, a.y & b.y, a.z & b.z, a.w & b.w};
-#pragma unroll
-                for (int t = 0; t < 4; t++) hq[t] &= above_word(v, (q << 2) + t);
-                if (hq[0] | hq[1] | hq[2] | hq[3]) {
-                    for (uint32_t c = g >> 2; c < nch; c++) {
-                        const uint4 xa = M[c * S + v], xb = B4[c];
-                        uint32_t h[4] = {xa.x & xb.x, xa.y & xb.y, xa.z & xb.z, xa.w & xb.w};
-#pragma unroll
-                        for (int t = 0; t < 4; t++) h[t] &= above_word(v, (c << 2) + t);
+                uint32_t D[4];
+                later(q, D);
+                if (D[0] | D[1] | D[2] | D[3]) {
+                    for (uint32_t c = g >> 2; c < q; c++) {
+                        uint32_t h[4];
+                        later(c, h);
 #pragma unroll
                         for (int t = 0; t < 4; t++) {
-                            leaf_word<4, 0>(Mq, hq, h[t], (c << 7) + (t << 5), ones, o.n);
+                            pair_word<4, -1, INV>(Mq, D, h[t], (c << 7) + (t << 5), p);
                             if (WORK) o.work += 4 * __popc(h[t]);
                         }
                     }
+                    pair_word<4, 0, INV>(Mq, D, D[0], (q << 7), p);
+                    pair_word<4, 1, INV>(Mq, D, D[1], (q << 7) + 32, p);
+                    pair_word<4, 2, INV>(Mq, D, D[2], (q << 7) + 64, p);
+                    pair_word<4, 3, INV>(Mq, D, D[3], (q << 7) + 96, p);
+                    if (INV) lin -= __popc(D[0]) + __popc(D[1]) + __popc(D[2]) + __popc(D[3]);
+                    if (WORK) o.work += 3 * (__popc(D[0]) + __popc(D[1]) + __popc(D[2]) + __popc(D[3]));
                 }
             }
         }
         __syncwarp();
     }
-    o.n += __popc(ones);
+    o.n = lin + p.both();
     return o;
 }
 
-__device__ __forceinline__ unsigned long long n3_finish(uint32_t s32, uint32_t sum)
+// N3 of a set of s members from its sum.
+__device__ __forceinline__ unsigned long long n3_finish(uint32_t s32, uint32_t sum, bool inv)
 {
     const unsigned long long s = s32;
-    return (uint32_t)((uint32_t)(s * (s - 1) * (s - 2) / 3) - sum) >> 1;
+    return (inv ? sum : (uint32_t)(s * (s - 1) * (s - 2) / 3) - sum) >> 1;
 }
 
 }  // namespace citron
