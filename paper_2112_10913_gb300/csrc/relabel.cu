@@ -12,10 +12,9 @@
 //                   barrier.  Per arc u->v the keep-test rank[v] > rank[u] (the 16 rank gathers
 //                   of a lane are all in flight before any is used); the kept ranks of each row
 //                   are placed IN the row's own input range (kept[off[u] ..]), so no global
-//                   prefix is needed: a warp-aggregated shared counter per row gives each kept
-//                   arc its place in its row piece, and every (row, chunk) piece takes its place
-//                   in the row with one atomicAdd on rowlen[rank[u]], which ends up holding the
-//                   row's out-degree in rank order;
+//                   prefix is needed: ballots give each kept arc its place in its row piece, and
+//                   every (row, chunk) piece takes its place in the row with one atomicAdd on
+//                   rowlen[rank[u]], which ends up holding the row's out-degree in rank order;
 //   k_scan_rowlen : dag_off = exclusive prefix of rowlen (single pass, decoupled look-back) and
 //                   the largest row;
 //   k_rl_fill     : rows in RANK order, one row per lane: a row of <= 32 entries is sorted by its
@@ -48,9 +47,9 @@ __global__ void k_rl_prologue(uint32_t n, const uint32_t *__restrict__ rank, uin
 
 // A chunk of 512 arcs per warp; no block-wide barrier anywhere, so every warp runs at its own
 // pace and the per-arc rank gathers of many warps overlap.
-constexpr uint32_t kWkArcs = 512;    // arcs per warp chunk (4 quads of 4 arcs per lane)
+constexpr uint32_t kWkArcs = 512;    // arcs per warp chunk (16 per lane)
 constexpr uint32_t kWkRowCap = 64;   // rows of a chunk handled in shared memory
-constexpr int kWkWarps = 8;          // warps per block
+constexpr int kWkWarps = 4;          // warps per block
 
 // A chunk overlapping more than kWkRowCap rows (long runs of empty rows): every kept arc takes
 // its place in its row with its own atomic; offsets come from global memory.
@@ -87,21 +86,29 @@ __device__ __noinline__ void rl_keep_uncached(uint32_t n, uint64_t arcs, const u
     }
 }
 
-// first_row[c] = min{u : off[u] >= c * 512} (k_tile_rows, order.cu).  Lane l holds the 16
-// consecutive arcs 16l .. 16l+15 of its chunk.  The place of a kept arc inside its row piece is
-// the number of kept arcs before it in the chunk (a warp prefix over the keep flags) minus that
-// number at the piece's start; every (row, chunk) piece reserves its place in the row with one
-// global atomic.
-__global__ __launch_bounds__(kWkWarps * 32) void k_rl_keep(
+// first_row[c] = min{u : off[u] >= c * 512} (k_tile_rows, order.cu).  Lane l holds the arcs l, 32 + l,
+// 64 + l, .. of its chunk, so that the reads of cols are whole lines and everything that concerns 32
+// consecutive arcs is one ballot word: the rows' first arcs are marked in 16 words (the row of arc p
+// is the number of marks up to p), and the kept arcs are 16 more.  The place of a kept arc inside
+// its row piece is the number of kept arcs before it in the chunk minus that number at the
+// piece's start; every (row, chunk) piece reserves its place in the row with one global atomic.
+// What bounds it: one random L2 sector per arc for rank[v].  With 16 consecutive arcs per lane, a
+// walk over the rows and a warp scan it issued three times the instructions and read every line
+// of cols in four strided passes: the ordering phase took 545 us on R-MAT 20 and 1530 us on the
+// 4M-vertex Chung-Lu graph against 492 and 1356 (at 40 warps per SM; 508 and 1402 at 28).
+__global__ __launch_bounds__(kWkWarps * 32, 10) void k_rl_keep(
     uint32_t n, uint64_t arcs, const uint64_t *__restrict__ off, const uint32_t *__restrict__ cols,
     const uint32_t *__restrict__ rank, const uint32_t *__restrict__ first_row, uint32_t nchunks,
-    uint32_t *kept, uint32_t *rowlen, uint32_t *err, int vec4)
+    uint32_t *kept, uint32_t *rowlen, uint32_t *err)
 {
-    __shared__ uint32_t s_rel[kWkWarps][kWkRowCap + 1];  // row starts - c0, clamped to [0, len]
-    __shared__ uint32_t s_key[kWkWarps][kWkRowCap];      // rank of each row
-    __shared__ int32_t s_place[kWkWarps][kWkRowCap];     // place of the row's piece minus P(start)
-    __shared__ uint32_t s_excl[kWkWarps][33];            // kept arcs before each lane's arcs
-    __shared__ uint16_t s_keep[kWkWarps][32];            // each lane's keep flags
+    constexpr int kWords = kWkArcs / 32;
+    // rows with arcs in the chunk: first arc - c0, rank, length, and where kept arc number 0 of
+    // the chunk would lie in `kept` if it were the row's
+    __shared__ uint32_t s_f[kWkWarps][kWkRowCap], s_key[kWkWarps][kWkRowCap], s_lim[kWkWarps][kWkRowCap];
+    __shared__ int64_t s_dst[kWkWarps][kWkRowCap];
+    // per 32 arcs: marks of first arcs, rows before, keep flags, kept arcs before
+    __shared__ uint32_t s_mark[kWkWarps][kWords], s_rows[kWkWarps][kWords];
+    __shared__ uint32_t s_keep[kWkWarps][kWords + 1], s_pre[kWkWarps][kWords + 1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t c = blockIdx.x * kWkWarps + w;
     if (c >= nchunks) return;
@@ -119,109 +126,97 @@ __global__ __launch_bounds__(kWkWarps * 32) void k_rl_keep(
         rl_keep_uncached(n, arcs, off, cols, rank, r0, u_next, c0, c1, kept, rowlen, err);
         return;
     }
-    for (uint32_t i = lane; i <= nrows; i += 32) {
-        const uint64_t o = off[r0 + i];
-        s_rel[w][i] = o <= c0 ? 0u : (o - c0 >= len ? len : (uint32_t)(o - c0));
-        if (i < nrows) s_key[w][i] = rank[r0 + i];
-    }
-    const uint64_t row0_start = off[r0];
-    const uint32_t p0 = 16u * lane;
-    uint32_t v[16], kv[16];
-    if (vec4 && p0 + 16 <= len) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(cols + c0 + p0);
+    uint32_t v[kWords];
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const uint4 x = __ldg(src + q);
-            v[4 * q] = x.x;
-            v[4 * q + 1] = x.y;
-            v[4 * q + 2] = x.z;
-            v[4 * q + 3] = x.w;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 16; j++) v[j] = p0 + j < len ? cols[c0 + p0 + j] : 0u;
-    }
-#pragma unroll
-    for (int j = 0; j < 16; j++) kv[j] = (p0 + j < len && v[j] < n) ? __ldg(rank + v[j]) : 0u;
+    for (int j = 0; j < kWords; j++) v[j] = 32u * j + lane < len ? __ldg(cols + c0 + 32 * j + lane) : 0u;
+    if (lane < kWords) s_mark[w][lane] = 0;
     __syncwarp();
-    // the row of this lane's first arc: the last i with s_rel[i] <= p0
-    uint32_t ri0 = 0;
-    if (p0 < len) {
-        uint32_t lo = 0, hi = nrows - 1;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi + 1) >> 1;
-            if (s_rel[w][mid] <= p0) lo = mid;
-            else hi = mid - 1;
-        }
-        ri0 = lo;
-    }
-    uint32_t keep = 0;
-    if (p0 < len) {
-        uint32_t ri = ri0, re = s_rel[w][ri + 1], ku = s_key[w][ri];
+    uint32_t nne = 0;  // rows with arcs here
 #pragma unroll
-        for (int j = 0; j < 16; j++) {
-            const uint32_t p = p0 + j;
-            if (p < len) {
-                while (re <= p && ri + 1 < nrows) {
-                    re = s_rel[w][++ri + 1];
-                    ku = s_key[w][ri];
-                }
-                if (v[j] >= n) set_error(err, kDevBadInput);
-                else if (kv[j] > ku) keep |= 1u << j;
-            }
+    for (int h = 0; h < (int)kWkRowCap / 32; h++) {
+        const uint32_t i = 32 * h + lane;
+        uint64_t b = 0, t = 0;
+        uint32_t f = 0, e = 0;
+        if (i < nrows) {
+            b = off[r0 + i];
+            t = off[r0 + i + 1];
+            f = b <= c0 ? 0u : (b - c0 >= len ? len : (uint32_t)(b - c0));
+            e = t <= c0 ? 0u : (t - c0 >= len ? len : (uint32_t)(t - c0));
         }
+        const uint32_t ne = __ballot_sync(kFull, e > f);
+        if (e > f) {
+            const uint32_t k = nne + __popc(ne & lanemask_lt());
+            s_f[w][k] = f;
+            s_key[w][k] = rank[r0 + i];
+            s_lim[w][k] = (b <= t && t <= arcs) ? (uint32_t)min(t - b, (uint64_t)0x40000000u) : 0u;
+            s_dst[w][k] = (int64_t)b;
+            atomicOr(&s_mark[w][f >> 5], 1u << (f & 31u));
+        }
+        nne += __popc(ne);
     }
-    const uint32_t cnt = __popc(keep);
-    const uint32_t incl = warp_incl_scan(cnt);
-    s_excl[w][lane] = incl - cnt;
-    if (lane == 31) s_excl[w][32] = incl;
-    s_keep[w][lane] = (uint16_t)keep;
+    uint32_t kv[kWords];
+#pragma unroll
+    for (int j = 0; j < kWords; j++) kv[j] = (32u * j + lane < len && v[j] < n) ? __ldg(rank + v[j]) : 0u;
+    bool range = false;
+#pragma unroll
+    for (int j = 0; j < kWords; j++) range |= 32u * j + lane < len && v[j] >= n;
+    if (range) set_error(err, kDevBadInput);
     __syncwarp();
-    // P(x): kept arcs of the chunk before position x
-    auto P = [&](uint32_t x) -> uint32_t {
-        const uint32_t q = x >> 4, b = x & 15;
-        return q >= 32 ? s_excl[w][32] : s_excl[w][q] + __popc((uint32_t)s_keep[w][q] & ((1u << b) - 1u));
+    {
+        const uint32_t m = lane < kWords ? __popc(s_mark[w][lane]) : 0u;
+        const uint32_t incl = warp_incl_scan(m);
+        if (lane < kWords) s_rows[w][lane] = incl - m;
+    }
+    __syncwarp();
+    const uint32_t upto = lanemask_lt() | (1u << lane);
+    // the row (index in s_f) of arc 32 j + lane; offsets that are not monotone may mark no row
+    auto row_of = [&](int j) -> uint32_t {
+        const uint32_t k = s_rows[w][j] + __popc(s_mark[w][j] & upto);
+        return k ? k - 1 : 0u;
     };
-    for (uint32_t i = lane; i < nrows; i += 32) {
-        const uint32_t f = s_rel[w][i], e = s_rel[w][i + 1];
-        int32_t place = INT32_MIN;
-        const uint32_t pf = P(f), k = e > f ? P(e) - pf : 0u;
-        if (k) {
+    uint32_t mine = 0;
+#pragma unroll
+    for (int j = 0; j < kWords; j++) {
+        const uint32_t keep = __ballot_sync(kFull, 32u * j + lane < len && v[j] < n && kv[j] > s_key[w][row_of(j)]);
+        if (lane == j) mine = keep;
+    }
+    {
+        const uint32_t m = __popc(mine), incl = warp_incl_scan(m);  // zero from lane kWords on
+        if (lane <= kWords) {
+            s_keep[w][lane] = mine;
+            s_pre[w][lane] = incl - m;
+        }
+    }
+    __syncwarp();
+    // kept arcs of the chunk before position x
+    auto P = [&](uint32_t x) -> uint32_t {
+        return s_pre[w][x >> 5] + __popc(s_keep[w][x >> 5] & ((1u << (x & 31u)) - 1u));
+    };
+    constexpr int64_t kNowhere = INT64_MIN;
+    for (uint32_t i = lane; i < nne; i += 32) {
+        const uint32_t pf = P(s_f[w][i]), k = P(i + 1 < nne ? s_f[w][i + 1] : len) - pf;
+        int64_t dst = kNowhere;
+        if (k && k <= kWkArcs) {
             const uint32_t key = s_key[w][i];
-            uint64_t rowlen_true = e - f;
-            if (i == 0 || i == nrows - 1) {  // the first and the last row may extend beyond the chunk
-                const uint64_t b = off[r0 + i], t = off[r0 + i + 1];
-                rowlen_true = (b <= t && t <= arcs) ? t - b : 0;
-            }
             if (key < n) {
                 const uint32_t base = atomicAdd(&rowlen[key], k);
                 // a row cannot keep more arcs than it has (else the rank is not a permutation)
-                if ((uint64_t)base + k <= rowlen_true && base < 0x40000000u) place = (int32_t)base - (int32_t)pf;
+                if ((uint64_t)base + k <= s_lim[w][i]) dst = s_dst[w][i] + (int64_t)base - (int64_t)pf;
                 else set_error(err, kDevBadInput);
             } else {
                 set_error(err, kDevBadInput);
             }
         }
-        s_place[w][i] = place;
+        s_dst[w][i] = dst;
     }
     __syncwarp();
-    if (keep) {
-        uint32_t ri = ri0, re = s_rel[w][ri + 1];
-        uint32_t q = s_excl[w][lane];
 #pragma unroll
-        for (int j = 0; j < 16; j++) {
-            const uint32_t p = p0 + j;
-            if (p < len) {
-                while (re <= p && ri + 1 < nrows) re = s_rel[w][++ri + 1];
-                if ((keep >> j) & 1) {
-                    const int32_t place = s_place[w][ri];
-                    if (place != INT32_MIN) {
-                        const uint64_t rs = ri == 0 ? row0_start : c0 + s_rel[w][ri];
-                        kept[rs + (uint64_t)(int64_t)((int64_t)place + q)] = kv[j];
-                    }
-                    q++;
-                }
-            }
+    for (int j = 0; j < kWords; j++) {
+        const uint32_t keep = s_keep[w][j];
+        if ((keep >> lane) & 1u) {
+            const int64_t dst = s_dst[w][row_of(j)];
+            const uint64_t at = (uint64_t)(dst + s_pre[w][j] + __popc(keep & lanemask_lt()));
+            if (dst != kNowhere && at < arcs) kept[at] = kv[j];  // (at is in the row unless offsets are not monotone)
         }
     }
 }
@@ -439,31 +434,44 @@ __global__ __launch_bounds__(kFiWarps * 32) void k_rl_fill(
     }
 }
 
-// Listed rows, one per warp, in the order the warps claim them (one atomic per row; a row's sort
-// costs far more).  Two instances: rows of 33..256 entries (8 registers of values per lane, so
-// that 32 warps fit an SM), then rows of 257..1024 (32 per lane, 128 registers); each lists the
-// rows it cannot take for the next (k_rl_fill_long above 1024).
-template <uint32_t MAXLEN, int MINB>
+// Listed rows, one per warp, BATCH of them per claim: their places come through one chain of
+// dependent loads (list, vertex, offsets) instead of one per row, which is what the kernel waited
+// for (ordering phase on R-MAT 20 586 -> 559 us, with blocks of 4 warps in k_rl_keep 545).  Two
+// instances: rows of 33..256 entries (8 registers of values per lane, so that 32 warps fit an SM),
+// then rows of 257..1024 (32 per lane, 128 registers); each lists the rows it cannot take for the
+// next (k_rl_fill_long above 1024).
+template <uint32_t MAXLEN, int MINB, uint32_t BATCH>
 __global__ __launch_bounds__(kFmWarps * 32, MINB) void k_rl_fill_mid(
     const uint32_t *__restrict__ perm, const uint32_t *__restrict__ kept,
     const uint64_t *__restrict__ off, const uint64_t *__restrict__ dag_off,
     uint32_t *__restrict__ dag_cols, const uint32_t *in_rows, const uint32_t *n_in, uint32_t *cursor,
     uint32_t *out_rows, uint32_t *n_out, uint32_t *err)
 {
-    const int lane = threadIdx.x & 31;
+    const uint32_t lane = threadIdx.x & 31;
     if (*(volatile uint32_t *)err) return;
     const uint32_t total = *n_in;
     for (;;) {
         uint32_t it = 0;
-        if (lane == 0) it = atomicAdd(cursor, 1u);
+        if (lane == 0) it = atomicAdd(cursor, BATCH);
         it = __shfl_sync(kFull, it, 0);
         if (it >= total) break;
-        const uint32_t r = in_rows[it];
-        // listed by k_rl_fill after its bounds checks: r < n, perm[r] < n, the row fits
-        const uint64_t src = off[perm[r]], dst = dag_off[r];
-        const uint32_t len = (uint32_t)(dag_off[r + 1] - dst);
-        if (!warp_sort_upto<MAXLEN>(kept + src, len, dag_cols + dst, lane) && lane == 0)
-            out_rows[atomicAdd(n_out, 1u)] = r;
+        // the places of BATCH rows at once: one chain of dependent loads for all of them
+        uint32_t r = 0, len = 0;
+        uint64_t src = 0, dst = 0;
+        if (lane < BATCH && it + lane < total) {
+            r = in_rows[it + lane];
+            // listed by k_rl_fill after its bounds checks: r < n, perm[r] < n, the row fits
+            src = off[perm[r]];
+            dst = dag_off[r];
+            len = (uint32_t)(dag_off[r + 1] - dst);
+        }
+        const int rows = (int)min(BATCH, total - it);
+        for (int q = 0; q < rows; q++) {
+            const uint64_t s1 = __shfl_sync(kFull, src, q), d1 = __shfl_sync(kFull, dst, q);
+            const uint32_t l1 = __shfl_sync(kFull, len, q), r1 = __shfl_sync(kFull, r, q);
+            if (!warp_sort_upto<MAXLEN>(kept + s1, l1, dag_cols + d1, lane) && lane == 0)
+                out_rows[atomicAdd(n_out, 1u)] = r1;
+        }
     }
 }
 
@@ -564,22 +572,21 @@ cudaError_t launch_relabel_dag(uint32_t n, uint64_t arcs, const uint64_t *off, c
     if ((e = cudaMemsetAsync(sc_status, 0, ((size_t)sc_tiles + 1) * sizeof(unsigned long long), st)))
         return e;
     const uint32_t ntiles = (uint32_t)ntiles64;
-    const int vec4 = ((uintptr_t)cols % 16) == 0;
     uint32_t *ticket = ctr, *max_len = ctr + 2, *n_long = ctr + 3, *n_mid = ctr + 4, *cursor = ctr + 5,
              *n_big = ctr + 6, *cursor_big = ctr + 7;
     if ((e = launch_tile_rows(n, arcs, off, kWkArcs, ntiles, first_row, st))) return e;
     k_rl_prologue<<<(n + 255) / 256, 256, 0, st>>>(n, rank, rowlen, perm, err);
     k_rl_keep<<<(ntiles + kWkWarps - 1) / kWkWarps, kWkWarps * 32, 0, st>>>(n, arcs, off, cols, rank, first_row,
-                                                                         ntiles, kept, rowlen, err, vec4);
+                                                                         ntiles, kept, rowlen, err);
     k_scan_rowlen<<<sc_tiles, kScThreads, 0, st>>>(n, rowlen, dag_off, sc_tiles, sc_status, ticket,
                                                    max_len, err, wait_cfg());
     uint32_t grid = (uint32_t)(((uint64_t)n + kFiWarps * 32 - 1) / (kFiWarps * 32));
     if (grid > (uint32_t)num_sms * 8) grid = (uint32_t)num_sms * 8;
     k_rl_fill<<<grid, kFiWarps * 32, 0, st>>>(n, arcs, off, perm, kept, dag_off, dag_cols, arcs / 2,
                                               mid_rows, n_mid, err);
-    k_rl_fill_mid<256, kFmMidBlocks><<<(uint32_t)num_sms * kFmMidBlocks, kFmWarps * 32, 0, st>>>(
+    k_rl_fill_mid<256, kFmMidBlocks, 4><<<(uint32_t)num_sms * kFmMidBlocks, kFmWarps * 32, 0, st>>>(
         perm, kept, off, dag_off, dag_cols, mid_rows, n_mid, cursor, big_rows, n_big, err);
-    k_rl_fill_mid<1024, 4><<<(uint32_t)num_sms * 4, kFmWarps * 32, 0, st>>>(
+    k_rl_fill_mid<1024, 4, 2><<<(uint32_t)num_sms * 4, kFmWarps * 32, 0, st>>>(
         perm, kept, off, dag_off, dag_cols, big_rows, n_big, cursor_big, long_rows, n_long, err);
     const uint32_t cap_bytes = kLongCap * sizeof(uint32_t);
     if ((e = cudaFuncSetAttribute(k_rl_fill_long, cudaFuncAttributeMaxDynamicSharedMemorySize, cap_bytes)))

@@ -36,3 +36,21 @@ def test_rows_inside_and_below_the_window(gpu, oracle_lib, core, span):
         assert G.count(k, warps_per_cta=1) == want
     H = cg.DeviceGraph(g, relabel=False)  # rows that are not upper-triangular
     assert H.count(4) == oracle_lib.count(off, cols, g.n, 4)
+
+
+@pytest.mark.parametrize("arcs", [2, 64, 510, 512, 514, 1024, 1536, 4094])
+@pytest.mark.parametrize("width", [1, 31, 32, 33, 255, 600])
+def test_relabelled_dag_at_chunk_edges(gpu, oracle_lib, arcs, width):
+    """Rows of about `width` arcs beside empty rows, with the arcs ending at and around the 512-arc chunks."""
+    import paper_2112_10913_gb300 as cg
+
+    rng = np.random.default_rng(arcs * 7 + width)
+    m = arcs // 2
+    hubs = -(-m // width)
+    src = np.repeat(np.arange(hubs) * 3, width)[:m]  # two empty rows between the hubs
+    dst = 3 * hubs + np.concatenate([rng.permutation(max(width, 8))[:width] for _ in range(hubs)])[:m]
+    g = gg.csr_from_edges(3 * hubs + max(width, 8) + 5, src, dst)
+    for rank in (oracle_lib.degree_rank(g.off, g.n), rng.permutation(g.n).astype(np.uint32)):
+        off, cols = oracle_lib.dag_by_rank(g.off, g.cols, g.n, rank, relabel=True)
+        goff, gcols = cg.DeviceGraph(g, rank=rank).dag_numpy()
+        assert np.array_equal(goff, off) and np.array_equal(gcols, cols)
