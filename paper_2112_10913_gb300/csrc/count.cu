@@ -344,10 +344,13 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     const uint32_t blocks = (n + 255) / 256;
     k_classify<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max, small_list,
                                       big_list, hist, st, nullptr, nullptr, run.filter);
-    k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, cursor, st);
-    k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max, cursor,
-                                         mid_list, run.filter);
-    note_launches(3);
+    note_launches(1);
+    if (max_outdeg > plan.small_max) {  // else no row is on the bitmap path
+        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, cursor, st);
+        k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max, cursor,
+                                             mid_list, run.filter);
+        note_launches(2);
+    }
     CountStats hs = {};
     hs.n_small = max_outdeg >= need ? n : 0;
     hs.max_mid = max_outdeg < plan.bitmap_max ? max_outdeg : plan.bitmap_max;

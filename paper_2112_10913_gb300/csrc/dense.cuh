@@ -37,7 +37,7 @@ constexpr uint32_t kNbhdWords = kNbhdMax * kNbhdMax / 32;  // its rows, and ...
 constexpr uint32_t kNbhdList = kNbhdMax / 2;               // ... its member list (uint16)
 constexpr uint32_t kMaskWords = 192;   // compress masks (160 words) and one word per lane
 constexpr uint32_t kHubNarrow = 16;    // members of a higher complement degree come last in the order
-constexpr uint32_t kHubWide = 48;
+constexpr uint32_t kHubWide = 28;        // (k = 6 on R-MAT 20: 216 ms at 48, 209 at 28)
 constexpr uint32_t kNbhdMin = 16;      // wide sets: larger neighbourhoods are counted by comp_nbhd
 
 // Carry-save accumulation of bit counts (a full adder per bit position): the bits of
