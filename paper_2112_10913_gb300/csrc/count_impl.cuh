@@ -690,6 +690,13 @@ __device__ __forceinline__ uint32_t adjacent_above(const CompSet &cs, uint32_t c
     return (uint32_t)lane == (b >> 5) ? r & above_bit(b & 31u) : r;
 }
 
+struct LaneSums {
+    unsigned long long acc, work;
+};
+
+template <int R, int CW, bool WORK>
+__device__ __noinline__ LaneSums packed_dfs(const WarpCtx x, uint32_t *m32, uint32_t s, int lane);
+
 // R-cliques (R >= 4) of the compact set c (lane word) on complement rows: warp-uniform walk over
 // the members down to R = 4, which is counted in one step.  CW: words of the sets (1..4), or 0 for
 // a wide set.  Totals are added on lane 0.
@@ -746,9 +753,34 @@ __device__ __forceinline__ void dense_dfs(const WarpCtx &x, const CompSet &cs, u
             const uint32_t nc = adjacent_above(cs, c, b, lane);
             if (WORK && (uint32_t)lane < cs.nch * 4) work += 1;
             const uint32_t m = __reduce_add_sync(kFull, __popc(nc));
-            if (m >= R - 1) dense_dfs<R - 1, CW, WORK>(x, cs, nc, m, lane, acc, work);
+            if (m < R - 1) continue;
+            if constexpr (R >= 6 && (CW == 4 || CW == 2)) {
+                // two or more levels to go on a set that fits fewer words: packed first, so that
+                // the R = 4 sets below have their lanes full (k = 8 on R-MAT 15: 69 -> 55 ms)
+                if (m <= 16 * CW) {
+                    uint32_t *sub = x.mbuf + kNarrow * 4 + (CW == 4 ? 0 : 256);
+                    pack_subset<CW>(reinterpret_cast<const uint4 *>(cs.m32), nc, m, x.mv, sub, lane);
+                    LaneSums o;
+                    if (CW == 2 || m <= 32) o = packed_dfs<R - 1, 1, WORK>(x, sub, m, lane);
+                    else o = packed_dfs<R - 1, 2, WORK>(x, sub, m, lane);
+                    if (lane == 0) add_acc(acc, o.acc, x.err);
+                    if (WORK) work += o.work;
+                    continue;
+                }
+            }
+            dense_dfs<R - 1, CW, WORK>(x, cs, nc, m, lane, acc, work);
         }
     }
+}
+
+// dense_dfs on a whole set of s members packed by pack_subset (the count on lane 0).
+template <int R, int CW, bool WORK>
+__device__ __noinline__ LaneSums packed_dfs(const WarpCtx x, uint32_t *m32, uint32_t s, int lane)
+{
+    LaneSums o = {0, 0};
+    const CompSet cs = {m32, 0, 1};
+    dense_dfs<R, CW, WORK>(x, cs, word_mask(s, lane), s, lane, o.acc, o.work);
+    return o;
 }
 
 // C(s, R) for s <= 128 and R <= 11 (below 2^51).
@@ -760,10 +792,6 @@ __device__ __forceinline__ unsigned long long choose(uint32_t s)
     for (uint32_t i = 0; i < (uint32_t)R; i++) v = v * (s - i) / (i + 1);
     return v;
 }
-
-struct LaneSums {
-    unsigned long long acc, work;
-};
 
 // A set with more than half of its pairs missing: its rows are turned back and enumerated.  Out of
 // line: sets of an edge task are seldom sparse, and the code would push the others' out of the
@@ -931,13 +959,15 @@ __host__ __device__ __forceinline__ uint32_t warp_list_words(uint32_t dcap, uint
 {
     return 32 + kMaskWords + kNbhdList + (compact_max && kNbhdWords > dcap / 2 ? kNbhdWords : dcap / 2);
 }
-__host__ __device__ __forceinline__ uint32_t warp_buf_words(uint32_t dcap, uint32_t compact_max)
+// (deep, k >= 8: also room for the rows of a subset of 64 members and of one of 32 in it)
+__host__ __device__ __forceinline__ uint32_t warp_buf_words(uint32_t dcap, uint32_t compact_max, bool deep)
 {
-    return dcap > compact_max * 4 ? dcap : compact_max * 4;
+    const uint32_t m = compact_max ? compact_max * 4 + (deep ? 256 + 128 : 0) : 0u;
+    return dcap > m ? dcap : m;
 }
-__host__ __device__ __forceinline__ uint32_t warp_scratch_words(uint32_t dcap, uint32_t compact_max)
+__host__ __device__ __forceinline__ uint32_t warp_scratch_words(uint32_t dcap, uint32_t compact_max, bool deep)
 {
-    return warp_list_words(dcap, compact_max) + warp_buf_words(dcap, compact_max);
+    return warp_list_words(dcap, compact_max) + warp_buf_words(dcap, compact_max, deep);
 }
 
 constexpr int kMidMaxWarps = 32;
@@ -1181,7 +1211,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     uint32_t *lists = K > 3 ? rows + (size_t)dcap * rs_cap : rows;  // k = 3 keeps no rows
     uint32_t *wscr = lists + (size_t)w * warp_list_words(dcap, compact_max);
-    const uint32_t buf_words = warp_buf_words(dcap, compact_max);
+    const uint32_t buf_words = warp_buf_words(dcap, compact_max, K >= 8);
     uint32_t *bufs = lists + (size_t)nw * warp_list_words(dcap, compact_max);
     // order of a root's rows, wide ones first: it reuses sL, which is dead once the rows are built
     uint16_t *s_order = reinterpret_cast<uint16_t *>(sL);
@@ -1783,7 +1813,7 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
             uint32_t warps = plan.warps_per_cta > (uint32_t)kMidMaxWarps ? kMidMaxWarps : plan.warps_per_cta;
             if (low && warps > kLowWarps) warps = kLowWarps;
             auto scratch = [&](uint32_t nw) {  // words for the warps' lists and buffers
-                return K > 3 ? (size_t)nw * warp_scratch_words(dcap, compact_max) : (size_t)kMidWindow / 32;
+                return K > 3 ? (size_t)nw * warp_scratch_words(dcap, compact_max, K >= 8) : (size_t)kMidWindow / 32;
             };
             auto smem_for = [&](uint32_t nw) {
                 return ((size_t)dcap + (K > 3 ? (size_t)dcap * rs : 0) + scratch(nw)) * sizeof(uint32_t);

@@ -399,6 +399,50 @@ __device__ __noinline__ CompCount comp_nbhd(const uint4 *M, uint32_t S, uint32_t
     return o;
 }
 
+// The complement rows of a subset U (lane word uw, at most 64 members) of a narrow set, packed to
+// U's own numbering: rows of up to two words, one uint4 each, in out.  scr: kMaskWords and kNbhdList
+// words.
+template <int CW>
+__device__ __noinline__ void pack_subset(const uint4 *M, uint32_t uw, uint32_t u, uint32_t *scr, uint32_t *out, int lane)
+{
+    uint16_t *list = reinterpret_cast<uint16_t *>(scr + kMaskWords);
+    uint32_t mv[5];
+    compress_masks(uw, mv);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 5; i++) scr[i * 32 + lane] = mv[i];
+    uint32_t at = 0;
+#pragma unroll
+    for (int t = 0; t < CW; t++) {
+        const uint32_t m = __shfl_sync(kFull, uw, t);
+        if ((m >> lane) & 1u) list[at + __popc(m & lanemask_lt())] = (uint16_t)((t << 5) + lane);
+        at += __popc(m);
+    }
+    __syncwarp();
+    for (uint32_t i = lane; i < ((u + 31) & ~31u); i += 32) {
+        uint32_t row[CW], o[2] = {0, 0};
+        load_row<CW>(M, list[i < u ? i : u - 1], row);
+        uint32_t pre = 0;
+#pragma unroll
+        for (int t = 0; t < CW; t++) {
+            const uint32_t m = __shfl_sync(kFull, uw, t);
+            uint32_t k[5];
+#pragma unroll
+            for (int q = 0; q < 5; q++) k[q] = scr[q * 32 + t];
+            const unsigned long long piece = (unsigned long long)compress_with(row[t], m, k) << (pre & 31u);
+            if (pre < 32) {
+                o[0] |= (uint32_t)piece;
+                o[1] |= (uint32_t)(piece >> 32);
+            } else {
+                o[1] |= (uint32_t)piece;
+            }
+            pre += __popc(m);
+        }
+        if (i < u) reinterpret_cast<uint4 *>(out)[i] = make_uint4(o[0], o[1], 0u, 0u);
+    }
+    __syncwarp();
+}
+
 // ---- Narrow sets (at most 128 members): one uint4 per complement row --------------------------
 
 // Adjacent pairs (x, y) inside D (CW words), x in D's word T (bits b): y in a later word into `once`,

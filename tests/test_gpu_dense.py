@@ -25,6 +25,8 @@ CASES += [(s, p, 0, k) for s in (129, 160, 193) for p in (0.3, 0.55, 0.8) for k 
 CASES += [(40, 0.9, 0, 7), (96, 0.7, 0, 7), (128, 0.6, 0, 7), (129, 0.7, 0, 7), (150, 0.6, 0, 7)]
 CASES += [(s, 0.95, 24, k) for s in (33, 64, 128) for k in (5, 6)]
 CASES += [(140, 0.9, 24, 6), (256, 0.8, 24, 5), (257, 0.75, 40, 6), (50, 0.95, 10, 8), (140, 0.6, 10, 8)]
+# subsets packed again on the way down
+CASES += [(45, 0.9, 0, 8), (64, 0.85, 6, 8), (65, 0.8, 0, 8), (100, 0.75, 10, 8), (128, 0.62, 0, 8), (66, 0.75, 0, 9)]
 CASES += [(40, 1.0, 0, 9), (100, 1.0, 0, 6), (140, 1.0, 0, 5)]
 # a third and more chunks, members of more than 255 missing neighbours, more than 128 of them
 CASES += [(300, 0.7, 40, 6), (385, 0.52, 0, 6), (530, 0.5, 0, 6), (520, 0.55, 0, 5)]
