@@ -1825,18 +1825,20 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
             unsigned long long *ns = grid ? nullptr : block_ns;  // timed: the first launch's blocks
             uint32_t this_grid = 0;
             uint32_t *queue = next + (low ? 3 : 0);
+            // a cap on the blocks means blocks of 32 warps: as many small ones hold a quarter of that
+            const uint32_t cap = low ? plan.max_blocks * (kMidMaxWarps / kLowWarps) : plan.max_blocks;
             // the instrumented kernel also serves the per-arc debug output (its code is compiled
             // out of the plain kernel)
             if (run.count_work || run.sink.per_arc) {
                 if constexpr (K <= (int)kInstrumentedMaxK)
-                    e = launch_mid<K, true>(n_roots, plan.max_blocks, low, dcap, window, compact_max, plan.split_min,
+                    e = launch_mid<K, true>(n_roots, cap, low, dcap, window, compact_max, plan.split_min,
                                             aux.help, warps, smem_for(warps), dag_off, dag_cols, mid_list, st,
                                             queue, result, run.sink, work, ns, aux.budget, &this_grid, err,
                                             s, num_sms);
                 else
                     e = cudaErrorNotSupported;  // refused by citron_count_ex before any launch
             } else
-                e = launch_mid<K, false>(n_roots, plan.max_blocks, low, dcap, window, compact_max, plan.split_min,
+                e = launch_mid<K, false>(n_roots, cap, low, dcap, window, compact_max, plan.split_min,
                                          aux.help, warps, smem_for(warps), dag_off, dag_cols, mid_list, st,
                                          queue, result, run.sink, work, ns, aux.budget, &this_grid, err, s,
                                          num_sms);
