@@ -20,6 +20,12 @@
 // (plane j holds bit j of every codegree) and added with LOP3 full adders, so that one step adds
 // one neighbour to 32 codegrees per word.
 //
+// What bounds it: instruction issue (and, for the 4-clique form, instruction fetch): listing a set,
+// packing its rows and the adders outweigh the word operations.  k_count_mid, k = 6 on R-MAT 20:
+// 683 ms enumerating the sets' arcs, 231 ms when this came in, 209 ms now; k = 8 on R-MAT 15: 577 ms,
+// 69 and 55.  The line between the sides is one half of the pairs: the cost of either is about
+// its edges.
+//
 // All arithmetic is exact modulo 2^32 (sets of at most 128 members) or 2^64; the results are
 // below the modulus.
 #pragma once
