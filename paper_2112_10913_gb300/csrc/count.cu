@@ -82,7 +82,7 @@ __global__ void k_classify(uint32_t n, const uint64_t *__restrict__ dag_off, uin
 }
 
 // Bin starts for the mid roots in DESCENDING out-degree: cursor[d] = #roots with degree > d.
-__global__ __launch_bounds__(1024) void k_mid_bins(const uint32_t *hist, uint32_t bins,
+__global__ __launch_bounds__(1024) void k_mid_bins(const uint32_t *hist, uint32_t bins, uint32_t low,
                                                     uint32_t *cursor, CountStats *st)
 {
     __shared__ uint32_t scratch[33];
@@ -96,7 +96,7 @@ __global__ __launch_bounds__(1024) void k_mid_bins(const uint32_t *hist, uint32_
     for (uint32_t i = lo; i < hi; i++) {
         const uint32_t d = bins - 1 - i;
         cursor[d] = run;
-        if (d == kLowMax) st->n_high = run;  // (zero when no degree above kLowMax has a bin)
+        if (d == low) st->n_high = run;  // (zero when no degree above it has a bin)
         run += hist[d];
     }
     if (threadIdx.x == 0) st->n_mid = total;
@@ -265,7 +265,7 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
         k_classify<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max,
                                           small_list, big_list, hist, st, run.sink.per_root,
                                           run.sink.per_arc, run.filter);
-        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, cursor, st);
+        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, low_max(k), cursor, st);
         k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max,
                                              cursor, mid_list, run.filter);
         note_launches(3);
@@ -346,7 +346,7 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
                                       big_list, hist, st, nullptr, nullptr, run.filter);
     note_launches(1);
     if (max_outdeg > plan.small_max) {  // else no row is on the bitmap path
-        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, cursor, st);
+        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, low_max(k), cursor, st);
         k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max, cursor,
                                              mid_list, run.filter);
         note_launches(2);
@@ -356,7 +356,7 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     hs.max_mid = max_outdeg < plan.bitmap_max ? max_outdeg : plan.bitmap_max;
     hs.n_mid = hs.max_mid > plan.small_max ? n : 0;
     // upper bounds of both parts of the queue: the kernels read the real ones on the device
-    hs.n_high = hs.max_mid > kLowMax ? n : 0;
+    hs.n_high = hs.max_mid > low_max(k) ? n : 0;
     hs.bound = 1;
     hs.max_big = max_outdeg;
     hs.n_big = max_outdeg > plan.bitmap_max ? n : 0;

@@ -19,18 +19,18 @@ constexpr uint32_t kMidWindow = 32768;  // ids in a block's membership bitmap (k
 struct CountStats {
     uint32_t n_small, n_mid, n_big;
     uint32_t max_mid, max_big, max_all;
-    uint32_t n_high;  // bitmap-path roots above kLowMax, the first n_high of the queue
+    uint32_t n_high;  // bitmap-path roots above low_max, the first n_high of the queue
     uint32_t bound;   // host copy only: the numbers are upper bounds (each part may hold n_mid roots)
 };
 
-// Up to k = 6, bitmap-path roots of at most kLowMax out-neighbours run in a launch of their own, in
-// blocks of 8 warps, several per SM: a block of 32 warps has a handful of rows per warp to build
-// for them and waits at its barriers instead.  R-MAT 15, k = 6: 0.70 ms in one launch, 0.64 in two
-// (0.79 with 4 warps).  Above that a root's counting outweighs its build and two launches end in
-// two tails: R-MAT 15, k = 8: 69 ms in one launch, 129 in two.
-constexpr uint32_t kLowMax = 128;
+// Bitmap-path roots of at most low_max(k) out-neighbours run in a launch of their own, in blocks of 8
+// warps, several per SM: a block of 32 warps has a handful of rows per warp to build for them and
+// waits at its barriers instead.  R-MAT 15, k = 6: 0.70 ms in one launch, 0.64 in two (0.79 with 4
+// warps).  From k = 7 on a root's counting outweighs its build and two launches end in two tails
+// (R-MAT 15, k = 8: 69 ms in one launch, 129 in two at 128), so only the smallest roots, which the
+// warp-register path leaves to this one there, go in small blocks.
 constexpr uint32_t kLowWarps = 8;
-constexpr int kPartsMaxK = 6;
+__host__ __device__ constexpr uint32_t low_max(uint32_t k) { return k <= 6 ? 128 : 32; }
 
 // ------------------------------------------------------------------------------------------
 // Warp-register path (D <= 32).
@@ -132,10 +132,24 @@ __global__ __launch_bounds__(kSmallWarps * 32) void k_count_small(
         }
         s_row[w][lane] = 0;
         __syncwarp();
+        // Where rows reach down to smaller ids (a DAG that keeps vertex ids) a pair takes two lookups:
+        // there, short lists (one load per lane) are scanned, every entry searched among the members.
+        // 20,000 vertices of degree 40, such a DAG, k = 3: 0.23 ms by pairs, 0.17 by lists; a relabelled
+        // DAG is better off with pairs (micro-batch of 64 graphs 3.01 ms by pairs, 3.07 by lists).
+        const bool down = lane < D && s_len[w][lane] && s_min[w][lane] < s_x[w][lane];
+        const bool lists = __any_sync(kFull, down) && __all_sync(kFull, lane >= D || s_len[w][lane] <= 32);
+        if (lists) {
+            for (uint32_t i = 0; i < D; i++) {
+                const uint32_t y = lane < s_len[w][i] ? dag_cols[s_rb[w][i] + lane] : 0xffffffffu;
+                const uint32_t j = lower_bound_smem(s_x[w], D, y);
+                const uint32_t bits = __reduce_or_sync(kFull, j < D && s_x[w][j] == y ? 1u << j : 0u);
+                if (lane == 0) s_row[w][i] = bits;
+            }
+        }
         // Every pair of members once, two per lane and round: pair p is (c, c + r + 1 mod D) with
         // r = p / D, c = p mod D.  An arc between them is in the row of one of the two: the one
         // of lower index if rows only hold larger ids (a relabelled DAG), else either.
-        const uint32_t npairs = D * (D - 1) / 2;
+        const uint32_t npairs = lists ? 0u : D * (D - 1) / 2;
         const float inv = 1.0f / (float)D;
         for (uint32_t p0 = 0; p0 < npairs; p0 += 64) {
             uint32_t src[2], dst[2], lo[2], left[2];
@@ -1231,7 +1245,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     win.first = reinterpret_cast<uint16_t *>(lists + window / 32);
     // this launch's part of the queue (largest out-degree first)
     const uint32_t first_root = low ? st->n_high : 0u;
-    const uint32_t nlist = (low || K > kPartsMaxK ? st->n_mid : st->n_high) - first_root;
+    const uint32_t nlist = (low ? st->n_mid : st->n_high) - first_root;
     list += first_root;
     if (WORK && lane == 0) s_arc[w] = 0;
     if (block_ns && threadIdx.x == 0) block_ns[2 * blockIdx.x] = global_ns();
@@ -1804,11 +1818,10 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
         Timer t(run.time_kernels, s);
         unsigned long long *block_ns = run.balance ? aux.block_ns : nullptr;
         uint32_t grid = 0;
-        const bool parts = K <= kPartsMaxK;
-        for (int low = 0; low < (parts ? 2 : 1); low++) {
-            const uint32_t n_roots = !parts ? hs.n_mid : !low ? hs.n_high : hs.bound ? hs.n_mid : hs.n_mid - hs.n_high;
+        for (int low = 0; low < 2; low++) {
+            const uint32_t n_roots = !low ? hs.n_high : hs.bound ? hs.n_mid : hs.n_mid - hs.n_high;
             if (!n_roots) continue;
-            const uint32_t dmax = low && hs.max_mid > kLowMax ? kLowMax : hs.max_mid;
+            const uint32_t dmax = low && hs.max_mid > low_max(K) ? low_max(K) : hs.max_mid;
             const uint32_t dcap = (dmax + 31) & ~31u, rs = (dcap / 32) | 1;
             uint32_t warps = plan.warps_per_cta > (uint32_t)kMidMaxWarps ? kMidMaxWarps : plan.warps_per_cta;
             if (low && warps > kLowWarps) warps = kLowWarps;
