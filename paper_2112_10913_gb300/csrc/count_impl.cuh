@@ -1218,7 +1218,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     const uint32_t rs_cap = (dcap / 32) | 1;
     uint32_t *sL = smem;
     uint32_t *rows = smem + dcap;
-    __shared__ uint32_t s_idx, s_task, s_wide[2], s_tri, s_slot, s_u, s_most;
+    __shared__ uint32_t s_idx, s_task, s_wide[2], s_tri, s_slot, s_u, s_most, s_unsorted;
     __shared__ uint32_t s_cls[2][kBitmapCap / 32];  // wide rows of either class, one bit each
     __shared__ unsigned long long s_acc[32], s_arc[32];
     __shared__ GroupShared s_group[kMaxGroups];
@@ -1258,6 +1258,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             s_wide[0] = s_wide[1] = 0;
             s_most = 0;
             s_tri = 1;
+            s_unsorted = 0;
             s_slot = kNoHelpSlot;
         }
         __syncthreads();
@@ -1303,15 +1304,22 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             rlen = (uint32_t)(dag_off[a + 1] - rb);
         }
         for (uint32_t i = threadIdx.x; i < D; i += blockDim.x) {
-            const uint32_t v = sL[i];
-            if (v >= win.base) {
+            const uint32_t v = sL[i], prev = i ? sL[i - 1] : 0u;
+            // the window's places hold for ascending members only, and an id above the last one's
+            // would lie beyond its bitmap
+            if (v < prev || v > lmax) s_unsorted = 1;
+            else if (v >= win.base) {
                 const uint32_t p = v - win.base;
                 atomicOr(&win.bits[p >> 5], 1u << (p & 31u));
-                if (K > 3 && (i == 0 || sL[i - 1] < win.base || ((sL[i - 1] - win.base) >> 5) != (p >> 5)))
+                if (K > 3 && (i == 0 || prev < win.base || ((prev - win.base) >> 5) != (p >> 5)))
                     win.first[p >> 5] = (uint16_t)i;
             }
         }
         __syncthreads();
+        if (s_unsorted) {  // the DAG's rows have to be sorted
+            if (threadIdx.x == 0) set_error(err, kDevBadInput);
+            break;
+        }
         win.nlow = win.base ? lower_bound_smem(sL, D, win.base) : 0u;
         unsigned long long acc = 0, work = 0;
         // Build the local subgraph: row i = V(g_u) ∩ N+(a_i) (CITRON's GenSubgraph).  Each step

@@ -1,0 +1,58 @@
+"""Inputs that break a counting call's contract in ways a kernel can see: the call reports an error
+instead of a count, and the next call on the same workspace is exact."""
+import numpy as np
+import pytest
+
+from paper_2112_10913_gb300 import graphgen as gg
+
+pytestmark = pytest.mark.gpu
+
+
+def _dag(size, hubs, seed, n=50_000):
+    """A DAG with `hubs` roots (lowest ids) that all have the same `size` out-neighbours, spread over
+    the ids (some below a root's membership window), which form G(size, 0.4) among themselves."""
+    rng = np.random.default_rng(seed)
+    ids = np.sort(rng.choice(np.arange(hubs, n), size, replace=False))
+    keep = np.triu(rng.random((size, size)) < 0.4, 1)
+    rows = [ids] * hubs + [np.empty(0, ids.dtype)] * (n - hubs)
+    for i in range(size):
+        rows[ids[i]] = ids[keep[i]]
+    return rows
+
+
+def _count(gpu, rows, k, **tuned):
+    import torch
+
+    off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
+    cols = np.concatenate(rows).astype(np.int32)
+    d_off, d_cols = torch.from_numpy(off).cuda(), torch.from_numpy(cols).cuda()
+    n, widest = len(rows), max(len(r) for r in rows)
+    ws = gpu.alloc_workspace(n, 2 * len(cols), widest)
+    return lambda: gpu.citron_count_ex(n, d_off, d_cols, k, ws, widest, **tuned)[0], d_cols
+
+
+@pytest.mark.parametrize("k", [3, 4, 5, 6, 7])
+@pytest.mark.parametrize("size", [33, 64, 129, 400])
+@pytest.mark.parametrize("order", ["reversed", "first above the last", "two swapped"])
+def test_unsorted_rows_are_refused(gpu, oracle_lib, size, k, order):
+    """Rows of a bitmap-path root that are not ascending: their ids would fall outside the window of
+    the ids below the last one."""
+    import torch
+
+    rows = _dag(size, 3, size)
+    run, d_cols = _count(gpu, rows, k)
+    good = d_cols.clone()
+    row = rows[0].copy()
+    if order == "reversed":
+        row = row[::-1]
+    elif order == "first above the last":
+        row[0], row[-1] = row[-1], row[0]
+    else:
+        row[size // 2], row[size // 2 + 1] = row[size // 2 + 1], row[size // 2]
+    d_cols[:size] = torch.from_numpy(row.astype(np.int32)).cuda()  # the first root's row
+    with pytest.raises(gpu.CitronError) as e:
+        run()
+    assert e.value.name == "CITRON_E_INVALID"
+    d_cols.copy_(good)
+    off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.uint64)
+    assert run() == oracle_lib.count(off, np.concatenate(rows).astype(np.uint32), len(rows), k)
