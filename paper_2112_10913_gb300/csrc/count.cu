@@ -31,11 +31,13 @@ namespace citron {
 // ------------------------------------------------------------------------------------------
 // Root classification.
 
+// counted: the largest out-degree that the launches after this one can count (a caller's bound on
+// the rows may be too small); a root above it is an error.
 __global__ void k_classify(uint32_t n, const uint64_t *__restrict__ dag_off, uint32_t need,
                            uint32_t small_max, uint32_t bitmap_max, uint32_t *small_list,
                            uint32_t *big_list, uint32_t *mid_hist, CountStats *st,
                            unsigned long long *per_root, unsigned long long *per_arc,
-                           RootFilter filter)
+                           RootFilter filter, uint32_t counted, uint32_t *err)
 {
     __shared__ uint32_t s_cnt[2], s_base[2], s_max[3];
     const int lane = threadIdx.x & 31;
@@ -51,7 +53,10 @@ __global__ void k_classify(uint32_t n, const uint64_t *__restrict__ dag_off, uin
         if (per_root) per_root[u] = 0;
         if (per_arc)  // debug output: every arc of the row starts at zero
             for (uint64_t e = dag_off[u]; e < dag_off[u + 1]; e++) per_arc[e] = 0;
-        if (D >= need && filter.takes(u)) cls = D <= small_max ? 0 : (D <= bitmap_max ? 2 : 1);
+        if (D >= need && filter.takes(u)) {
+            cls = D <= small_max ? 0 : (D <= bitmap_max ? 2 : 1);
+            if (D > counted) set_error(err, kDevBadInput);
+        }
     }
     uint32_t off_in_warp[2] = {0, 0}, warp_base[2] = {0, 0};
 #pragma unroll
@@ -264,7 +269,7 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
     if (n) {
         k_classify<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max,
                                           small_list, big_list, hist, st, run.sink.per_root,
-                                          run.sink.per_arc, run.filter);
+                                          run.sink.per_arc, run.filter, 0xffffffffu, err);
         k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, low_max(k), cursor, st);
         k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max,
                                              cursor, mid_list, run.filter);
@@ -342,8 +347,14 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     if (n == 0 || max_outdeg < k - 1) return cudaSuccess;
     const uint32_t need = k - 1;
     const uint32_t blocks = (n + 255) / 256;
+    // What the launches below can count when max_outdeg is not the largest row after all: the
+    // warp-register path any of its roots, the bitmap path what its rows' capacity (a multiple of 32)
+    // holds, the sorted-list path (which reports what its scratch cannot hold) the rest.
+    uint32_t counted = plan.small_max;
+    if (max_outdeg > plan.bitmap_max) counted = 0xffffffffu;
+    else if (max_outdeg > plan.small_max) counted = min((max_outdeg + 31) & ~31u, plan.bitmap_max);
     k_classify<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max, small_list,
-                                      big_list, hist, st, nullptr, nullptr, run.filter);
+                                      big_list, hist, st, nullptr, nullptr, run.filter, counted, err);
     note_launches(1);
     if (max_outdeg > plan.small_max) {  // else no row is on the bitmap path
         k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, low_max(k), cursor, st);

@@ -56,3 +56,31 @@ def test_unsorted_rows_are_refused(gpu, oracle_lib, size, k, order):
     d_cols.copy_(good)
     off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.uint64)
     assert run() == oracle_lib.count(off, np.concatenate(rows).astype(np.uint32), len(rows), k)
+
+
+@pytest.mark.parametrize("k", [3, 5, 7])
+@pytest.mark.parametrize("bound", [12, 16, 17, 31, 32, 33, 64, 96, 127, 128, 129, 160, 192, 193, 200, 300])
+def test_understated_bound_of_a_batch(gpu, bound, k):
+    """citron_count_batch sizes its launches by the caller's largest row (here 200): a bound whose
+    launches leave a root out is reported, one that only rounds up to the row's capacity is not."""
+    import torch
+    from math import comb
+
+    G = gpu.DeviceGraph(gg.complete(201))  # a relabelled DAG with rows of 200, 199, .., 0
+    zeros = torch.zeros(G.n, dtype=torch.int32, device="cuda")
+    ks = torch.tensor([k], dtype=torch.int32, device="cuda")
+    counts = torch.zeros(1, dtype=torch.int64, device="cuda")
+    ws = gpu.alloc_workspace(G.n, G.arcs, 300)
+
+    def run(widest):
+        gpu.citron_count_batch(G.n, G.dag_off, G.dag_cols, G.rank, zeros, ks, 1, 1 << k, widest, counts, ws)
+        gpu.citron_workspace_status(ws)
+        return int(counts.item())
+
+    if bound >= 193:
+        assert run(bound) == comb(201, k)
+    else:
+        with pytest.raises(gpu.CitronError) as e:
+            run(bound)
+        assert e.value.name == "CITRON_E_INVALID"
+    assert run(200) == comb(201, k)
