@@ -200,8 +200,8 @@ typedef struct {
                                 sets of at most 128 members by one warp and wider ones by several,
                                 1 means never */
     uint32_t max_blocks;     /* in: cap on the blocks of each counting launch, so that work on
-                                other streams keeps some SMs (0: no cap); in blocks of 32 warps,
-                                launches of 8-warp blocks take up to four times as many */
+                                other streams keeps some SMs (0: no cap); the warp-register path
+                                (blocks of 8 warps) takes up to four times as many */
     uint64_t *d_per_root;    /* in: optional device array of n uint64, as in citron_count */
     uint64_t work_ops;       /* out: 32-bit AND+POPC word operations of the bitmap path */
     float kernel_ms[3];      /* out: device ms of the warp-register, bitmap, sorted-list kernels */

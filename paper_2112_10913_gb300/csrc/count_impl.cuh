@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "dense.cuh"
 
@@ -30,6 +32,13 @@ struct CountStats {
 // (R-MAT 15, k = 8: 69 ms in one launch, 129 in two at 128), so only the smallest roots, which the
 // warp-register path leaves to this one there, go in small blocks.
 constexpr uint32_t kLowWarps = 8;
+// Under a cap on the blocks, that launch's blocks hold up to kMaxTeams teams of 8 warps, each with roots
+// of its own: as many blocks of 8 warps as the cap's warps are spread over all SMs, and no block of
+// 32 warps of another stream finds an empty one.  114 blocks, 180,000 roots of at most 119, k = 4..6,
+// and counts of 0.13 ms on another stream: these take 4 to 21 ms at worst beside blocks of 8 warps,
+// 0.25 to 1.6 ms beside teams.  (Blocks of 32 warps on one root each leave the SMs free too, but
+// k = 3 on R-MAT 18 takes 1.7 ms with them, 1.3 with teams.)
+constexpr int kMaxTeams = 4;
 __host__ __device__ constexpr uint32_t low_max(uint32_t k) { return k <= 6 ? 128 : 32; }
 
 // ------------------------------------------------------------------------------------------
@@ -1192,7 +1201,7 @@ __device__ __forceinline__ void wide_row(const WarpCtx &x, const Group &g, uint3
     }
 }
 
-// Bitmap path (small_max < D <= dcap): one block per root, roots taken largest-D first from the
+// Bitmap path (small_max < D <= dcap): one block (or one of its `teams`) per root, roots taken largest-D first from the
 // queue.  The block builds the root's local subgraph as D x D bitmap rows in shared memory
 // (row i = V(g_u) ∩ N+(a_i), Algorithm GenSub-CITRON by sorted-list intersection) and its warps
 // count the (K-2)-cliques of every row: the edge tasks (u, a_t).
@@ -1206,23 +1215,36 @@ __device__ __forceinline__ void wide_row(const WarpCtx &x, const Group &g, uint3
 //       left, rebuild its rows and take from the same cursors (work stealing across blocks);
 //       every block adds its own part of the root's count.
 // block_ns (optional): each block's start and end on the global timer.
-template <int K, bool WORK>
+// TEAMED: the block is `team_count` teams instead of one (an instance of its own: the plain kernel has no
+// registers to spare).
+template <int K, bool WORK, bool TEAMED>
 __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     const uint64_t *__restrict__ dag_off, const uint32_t *__restrict__ dag_cols,
-    const uint32_t *__restrict__ list, const CountStats *st, uint32_t *next, int low, uint32_t dcap,
-    uint32_t window, uint32_t compact_max, uint32_t split_min, HelpTable ht, unsigned long long *result,
-    RootSink sink, unsigned long long *work_out, unsigned long long *block_ns, Budget budget,
+    const uint32_t *__restrict__ list, const CountStats *st, uint32_t *next, int low, int team_count, uint32_t dcap,
+    uint32_t team_words, uint32_t window, uint32_t compact_max, uint32_t split_min, HelpTable ht,
+    unsigned long long *result, RootSink sink, unsigned long long *work_out, unsigned long long *block_ns, Budget budget,
     uint32_t *err)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     const uint32_t rs_cap = (dcap / 32) | 1;
-    uint32_t *sL = smem;
-    uint32_t *rows = smem + dcap;
-    __shared__ uint32_t s_idx, s_task, s_wide[2], s_tri, s_slot, s_u, s_most, s_unsorted;
+    // this team: nw warps, of which this is number w (wb in the block); tx its thread
+    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
+    const int nw = TEAMED ? (int)(blockDim.x >> 5) / team_count : (int)(blockDim.x >> 5);
+    const int team = TEAMED ? wb / nw : 0, w = TEAMED ? wb - team * nw : wb;
+    const uint32_t tx = TEAMED ? (uint32_t)w * 32 + lane : threadIdx.x, tn = TEAMED ? (uint32_t)nw * 32 : blockDim.x;
+    auto sync = [&]() {
+        if (!TEAMED) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(tn) : "memory");
+    };
+    uint32_t *sL = smem + (size_t)team * team_words;
+    uint32_t *rows = sL + dcap;
+    __shared__ uint32_t s_idx[kMaxTeams], s_task[kMaxTeams], s_tri[kMaxTeams], s_slot[kMaxTeams], s_u[kMaxTeams],
+        s_unsorted[kMaxTeams];
+    // (roots with wide rows are not counted by teams)
+    __shared__ uint32_t s_wide[2], s_most;
     __shared__ uint32_t s_cls[2][kBitmapCap / 32];  // wide rows of either class, one bit each
     __shared__ unsigned long long s_acc[32], s_arc[32];
     __shared__ GroupShared s_group[kMaxGroups];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     uint32_t *lists = K > 3 ? rows + (size_t)dcap * rs_cap : rows;  // k = 3 keeps no rows
     uint32_t *wscr = lists + (size_t)w * warp_list_words(dcap, compact_max);
     const uint32_t buf_words = warp_buf_words(dcap, compact_max, K >= 8);
@@ -1247,22 +1269,22 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     const uint32_t first_root = low ? st->n_high : 0u;
     const uint32_t nlist = (low ? st->n_mid : st->n_high) - first_root;
     list += first_root;
-    if (WORK && lane == 0) s_arc[w] = 0;
+    if (WORK && lane == 0) s_arc[wb] = 0;
     if (block_ns && threadIdx.x == 0) block_ns[2 * blockIdx.x] = global_ns();
     unsigned long long block_total = 0;  // meaningful in thread 0
     bool queue_empty = false;
     for (;;) {
-        if (threadIdx.x == 0) {
-            s_idx = queue_empty || budget.over(err) ? 0xfffffffeu : atomicAdd(next, 1u);
-            s_task = 0;
+        if (tx == 0) {
+            s_idx[team] = queue_empty || budget.over(err) ? 0xfffffffeu : atomicAdd(next, 1u);
+            s_task[team] = 0;
             s_wide[0] = s_wide[1] = 0;
             s_most = 0;
-            s_tri = 1;
-            s_unsorted = 0;
-            s_slot = kNoHelpSlot;
+            s_tri[team] = 1;
+            s_unsorted[team] = 0;
+            s_slot[team] = kNoHelpSlot;
         }
-        __syncthreads();
-        const uint32_t idx = s_idx;
+        sync();
+        const uint32_t idx = s_idx[team];
         const bool owner = idx < nlist;
         if (!owner) {
             queue_empty = true;
@@ -1270,29 +1292,29 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             if (w == 0) {
                 const uint32_t sl = pick_help_slot(ht, lane);
                 if (lane == 0) {
-                    s_slot = sl;
-                    if (sl != kNoHelpSlot) s_u = ht.slots[sl].u;
+                    s_slot[team] = sl;
+                    if (sl != kNoHelpSlot) s_u[team] = ht.slots[sl].u;
                 }
             }
-            __syncthreads();
-            if (s_slot == kNoHelpSlot) break;
+            sync();
+            if (s_slot[team] == kNoHelpSlot) break;
         }
-        const uint32_t u = owner ? list[idx] : s_u;
+        const uint32_t u = owner ? list[idx] : s_u[team];
         const uint64_t base = dag_off[u];
         const uint32_t D = (uint32_t)(dag_off[u + 1] - base);
         if (D > dcap || D == 0) {  // a root is never larger than the launch's capacity
-            if (threadIdx.x == 0) set_error(err, kDevBadInput);
+            if (tx == 0) set_error(err, kDevBadInput);
             break;
         }
         const bool heavy = K >= 6 && (!owner || D >= split_min);
         const uint32_t W = (D + 31) >> 5, RS = W | 1;
         // the rows this warp builds (w, w + nw, ..): lane r holds the place of the r-th one's list
         const uint32_t mine = w + (uint32_t)nw * lane;
-        for (uint32_t i = threadIdx.x; i < D; i += blockDim.x) sL[i] = dag_cols[base + i];
+        for (uint32_t i = tx; i < D; i += tn) sL[i] = dag_cols[base + i];
         if (K > 3)
-            for (uint32_t i = threadIdx.x; i < D * RS; i += blockDim.x) rows[i] = 0;
-        for (uint32_t i = threadIdx.x; i < window / 32; i += blockDim.x) win.bits[i] = 0;
-        __syncthreads();
+            for (uint32_t i = tx; i < D * RS; i += tn) rows[i] = 0;
+        for (uint32_t i = tx; i < window / 32; i += tn) win.bits[i] = 0;
+        sync();
         const uint32_t lmax = sL[D - 1];
         win.base = lmax >= window ? lmax - (window - 1) : 0u;
         win.span = lmax - win.base + 1;
@@ -1303,11 +1325,11 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             rb = dag_off[a];
             rlen = (uint32_t)(dag_off[a + 1] - rb);
         }
-        for (uint32_t i = threadIdx.x; i < D; i += blockDim.x) {
+        for (uint32_t i = tx; i < D; i += tn) {
             const uint32_t v = sL[i], prev = i ? sL[i - 1] : 0u;
             // the window's places hold for ascending members only, and an id above the last one's
             // would lie beyond its bitmap
-            if (v < prev || v > lmax) s_unsorted = 1;
+            if (v < prev || v > lmax) s_unsorted[team] = 1;
             else if (v >= win.base) {
                 const uint32_t p = v - win.base;
                 atomicOr(&win.bits[p >> 5], 1u << (p & 31u));
@@ -1315,9 +1337,9 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                     win.first[p >> 5] = (uint16_t)i;
             }
         }
-        __syncthreads();
-        if (s_unsorted) {  // the DAG's rows have to be sorted
-            if (threadIdx.x == 0) set_error(err, kDevBadInput);
+        sync();
+        if (s_unsorted[team]) {  // the DAG's rows have to be sorted
+            if (tx == 0) set_error(err, kDevBadInput);
             break;
         }
         win.nlow = win.base ? lower_bound_smem(sL, D, win.base) : 0u;
@@ -1369,11 +1391,11 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             }
         }
         if (K > 3) {
-            if (!__all_sync(kFull, tri) && lane == 0) s_tri = 0;
-            __syncthreads();
+            if (!__all_sync(kFull, tri) && lane == 0) s_tri[team] = 0;
+            sync();
             x.RS = RS;
             x.W = W;
-            x.tri = s_tri != 0;
+            x.tri = s_tri[team] != 0;
             // Wide rows come first in the order of the rows: those that need more than two warps'
             // buffers, the other ones, then the rows of one warp.  A root of at most 129
             // out-neighbours has no wide row.
@@ -1397,7 +1419,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                             if (most) atomicMax(&s_most, most);
                         }
                     }
-                    __syncthreads();
+                    sync();
                     if (s_most) {
                         for (uint32_t q = 0; q < W; q++) {
                             nbig += __popc(s_cls[0][q]);
@@ -1417,14 +1439,14 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                                                                     : nbig + nmid + (t - rb - rm);
                             if (t < D) s_order[at] = (uint16_t)t;
                         }
-                        __syncthreads();
+                        sync();
                     }
                 }
                 narrow = D - nbig - nmid;
             }
             const uint32_t nwide = nbig + nmid;
             if (heavy) {
-                if (threadIdx.x == 0) {
+                if (tx == 0) {
                     const uint32_t units = 0x80000000u | (nbig << 21) | (nmid << 11) | narrow;
                     if (owner && ht.slots) {
                         const uint32_t sl = atomicAdd(ht.nslots, 1u);
@@ -1432,21 +1454,21 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                             ht.slots[sl].u = u;
                             cuda::atomic_ref<uint32_t, cuda::thread_scope_device> pub(ht.slots[sl].units);
                             pub.store(units, cuda::memory_order_release);
-                            s_slot = sl;
+                            s_slot[team] = sl;
                         }
-                    } else if (!owner && ht.slots[s_slot].units != units) {
+                    } else if (!owner && ht.slots[s_slot[team]].units != units) {
                         set_error(err, kDevBadInput);  // the rebuilt root differs from the published one
-                        s_task = narrow;               // take nothing
+                        s_task[team] = narrow;               // take nothing
                         s_wide[0] = nbig;
                         s_wide[1] = nmid;
-                        s_slot = kNoHelpSlot;
+                        s_slot[team] = kNoHelpSlot;
                     }
                 }
-                __syncthreads();
+                sync();
             }
             // the rows of a published heavy root are taken from its slot's cursors in global
             // memory, the others from the block's counters in shared memory
-            HeavySlot *slot = s_slot != kNoHelpSlot ? &ht.slots[s_slot] : nullptr;
+            HeavySlot *slot = s_slot[team] != kNoHelpSlot ? &ht.slots[s_slot[team]] : nullptr;
             if constexpr (K >= 5) {
                 // Rows s_order[first .. first + count) of class cls by groups of gw warps.  A group is
                 // named by its first warp (barrier and shared state), so that a warp can go on to
@@ -1482,7 +1504,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                             const unsigned long long d = warp_sum_u64(acc, err);
                             if (lane == 0) {
                                 if (d) atomicAdd(&sink.per_arc[base + t], d);
-                                s_arc[w] += d;
+                                s_arc[wb] += d;
                             }
                             acc = 0;
                         }
@@ -1509,7 +1531,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                     const uint32_t nunits = W * (W + 1) / 2;
                     for (;;) {
                         uint32_t v = 0, q = 0;
-                        if (lane == 0) v = atomicAdd(&s_task, 1u);
+                        if (lane == 0) v = atomicAdd(&s_task[team], 1u);
                         v = __shfl_sync(kFull, v, 0);
                         if (v >= nunits) break;
                         while (v >= W - q) {
@@ -1548,7 +1570,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             auto claim = [&]() -> uint32_t {
                 uint32_t v = 0;
                 if (lane == 0)
-                    v = heavy && budget.over(err) ? narrow : (slot ? atomicAdd(&slot->cursor, 1u) : atomicAdd(&s_task, 1u));
+                    v = heavy && budget.over(err) ? narrow : (slot ? atomicAdd(&slot->cursor, 1u) : atomicAdd(&s_task[team], 1u));
                 return v;
             };
             uint32_t next_i = claim();
@@ -1567,7 +1589,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                     const unsigned long long d = warp_sum_u64(acc, err);
                     if (lane == 0) {
                         if (d) atomicAdd(&sink.per_arc[base + t], d);
-                        s_arc[w] += d;
+                        s_arc[wb] += d;
                     }
                     acc = 0;
                 }
@@ -1579,18 +1601,18 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
         }
         const unsigned long long ws = warp_sum_u64(acc, err);
         if (lane == 0) {
-            s_acc[w] = ws;
+            s_acc[wb] = ws;
             if (WORK) {  // the per-arc mode's running sum (zero without it)
-                s_acc[w] += s_arc[w];
-                s_arc[w] = 0;
+                s_acc[wb] += s_arc[wb];
+                s_arc[wb] = 0;
             }
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        sync();
+        if (tx == 0) {
             unsigned long long r = 0;
             bool wrapped = false;
             for (int i = 0; i < nw; i++) {
-                const unsigned long long s2 = r + s_acc[i];
+                const unsigned long long s2 = r + s_acc[team * nw + i];
                 wrapped |= s2 < r;
                 r = s2;
             }
@@ -1603,11 +1625,11 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             if (s2 < block_total) set_error(err, kDevOverflow);
             block_total = s2;
         }
-        __syncthreads();
+        sync();
     }
-    if (threadIdx.x == 0) {
+    if (tx == 0) {
         add_checked(result, block_total, err);
-        if (block_ns) block_ns[2 * blockIdx.x + 1] = global_ns();
+        if (block_ns) atomicMax(&block_ns[2 * blockIdx.x + 1], global_ns());  // its last team's end
     }
 }
 
@@ -1766,10 +1788,10 @@ struct Timer {
     }
 };
 
-template <int K, bool WORK>
-static cudaError_t launch_mid(uint32_t grid_cap, uint32_t block_cap, int low, uint32_t dcap,
+template <int K, bool WORK, bool TEAMED>
+static cudaError_t launch_mid(uint32_t grid_cap, uint32_t block_cap, int low, uint32_t teams, uint32_t dcap,
                               uint32_t window, uint32_t compact_max, uint32_t split_min, const HelpTable &ht,
-                              uint32_t warps, size_t smem, const uint64_t *dag_off,
+                              uint32_t warps, size_t team_smem, const uint64_t *dag_off,
                               const uint32_t *dag_cols, const uint32_t *mid_list,
                               const CountStats *st, uint32_t *next, unsigned long long *result,
                               RootSink sink, unsigned long long *work, unsigned long long *block_ns,
@@ -1781,14 +1803,16 @@ static cudaError_t launch_mid(uint32_t grid_cap, uint32_t block_cap, int low, ui
     // the device's largest value, because host threads that count concurrently would otherwise
     // overwrite each other's smaller setting between the set and the launch
     int dev = 0, optin = 0;
+    const size_t smem = teams * team_smem;
+    warps *= teams;
     if ((e = cudaGetDevice(&dev))) return e;
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
     if ((size_t)optin < smem + kMidStaticSmem) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(k_count_mid<K, WORK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(k_count_mid<K, WORK, TEAMED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   optin - (int)kMidStaticSmem)))
         return e;
     int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_count_mid<K, WORK>, warps * 32,
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_count_mid<K, WORK, TEAMED>, warps * 32,
                                                            smem)))
         return e;
     if (per_sm < 1) per_sm = 1;
@@ -1797,9 +1821,9 @@ static cudaError_t launch_mid(uint32_t grid_cap, uint32_t block_cap, int low, ui
     if (block_cap && grid > block_cap) grid = block_cap;
     if (grid > (uint32_t)num_sms * kMidBlocksPerSmCap) grid = (uint32_t)num_sms * kMidBlocksPerSmCap;
     *grid_out = grid;
-    k_count_mid<K, WORK><<<grid, warps * 32, smem, s>>>(dag_off, dag_cols, mid_list, st, next, low, dcap,
-                                                        window, compact_max, split_min, ht, result, sink,
-                                                        work, block_ns, budget, err);
+    k_count_mid<K, WORK, TEAMED><<<grid, warps * 32, smem, s>>>(dag_off, dag_cols, mid_list, st, next, low, (int)teams, dcap,
+                                                        (uint32_t)(team_smem / sizeof(uint32_t)), window, compact_max,
+                                                        split_min, ht, result, sink, work, block_ns, budget, err);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -1825,6 +1849,8 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
         const uint32_t compact_max = K >= 5 ? plan.compact_max : 0u;
         Timer t(run.time_kernels, s);
         unsigned long long *block_ns = run.balance ? aux.block_ns : nullptr;
+        if (block_ns && (e = cudaMemsetAsync(block_ns, 0, 2 * sizeof(*block_ns) * kMidBlocksPerSmCap * num_sms, s)))
+            return e;
         uint32_t grid = 0;
         for (int low = 0; low < 2; low++) {
             const uint32_t n_roots = !low ? hs.n_high : hs.bound ? hs.n_mid : hs.n_mid - hs.n_high;
@@ -1846,23 +1872,29 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
             unsigned long long *ns = grid ? nullptr : block_ns;  // timed: the first launch's blocks
             uint32_t this_grid = 0;
             uint32_t *queue = next + (low ? 3 : 0);
-            // a cap on the blocks means blocks of 32 warps: as many small ones hold a quarter of that
-            const uint32_t cap = low ? plan.max_blocks * (kMidMaxWarps / kLowWarps) : plan.max_blocks;
+            // under a cap: teams of kLowWarps in blocks as wide as the other launch's
+            uint32_t teams = 1;
+            if (K <= 6 && low && plan.max_blocks && !run.count_work && !run.sink.per_arc)
+                while (teams < (uint32_t)kMaxTeams && 2 * teams * kLowWarps <= plan.warps_per_cta &&
+                       2 * teams * smem_for(warps) <= (size_t)smem_cap)
+                    teams *= 2;
+            auto launch = [&](auto kind) {
+                constexpr int v = decltype(kind)::value;  // 0 plain, 1 instrumented, 2 in teams
+                return launch_mid<K, v == 1, v == 2>((n_roots + teams - 1) / teams, plan.max_blocks, low, teams, dcap,
+                                                     window, compact_max, plan.split_min, aux.help, warps,
+                                                     smem_for(warps), dag_off, dag_cols, mid_list, st, queue, result,
+                                                     run.sink, work, ns, aux.budget, &this_grid, err, s, num_sms);
+            };
             // the instrumented kernel also serves the per-arc debug output (its code is compiled
             // out of the plain kernel)
             if (run.count_work || run.sink.per_arc) {
-                if constexpr (K <= (int)kInstrumentedMaxK)
-                    e = launch_mid<K, true>(n_roots, cap, low, dcap, window, compact_max, plan.split_min,
-                                            aux.help, warps, smem_for(warps), dag_off, dag_cols, mid_list, st,
-                                            queue, result, run.sink, work, ns, aux.budget, &this_grid, err,
-                                            s, num_sms);
-                else
-                    e = cudaErrorNotSupported;  // refused by citron_count_ex before any launch
-            } else
-                e = launch_mid<K, false>(n_roots, cap, low, dcap, window, compact_max, plan.split_min,
-                                         aux.help, warps, smem_for(warps), dag_off, dag_cols, mid_list, st,
-                                         queue, result, run.sink, work, ns, aux.budget, &this_grid, err, s,
-                                         num_sms);
+                if constexpr (K <= (int)kInstrumentedMaxK) e = launch(std::integral_constant<int, 1>());
+                else e = cudaErrorNotSupported;  // refused by citron_count_ex before any launch
+            } else if (teams > 1) {
+                if constexpr (K <= 6) e = launch(std::integral_constant<int, 2>());
+            } else {
+                e = launch(std::integral_constant<int, 0>());
+            }
             if (e) return e;
             if (!grid) grid = this_grid;
         }
