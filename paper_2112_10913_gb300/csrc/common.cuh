@@ -233,15 +233,16 @@ struct RootSink {
     __device__ __forceinline__ bool wants_root_total() const { return per_root || group_counts; }
 };
 
-// A heavy root whose units (its edge tasks, i.e. the rows of its local subgraph) any block may
-// take: the block that took the root from the queue publishes it here; blocks that find the root
-// queue empty rebuild its local subgraph and take units from the same cursors.
+// A heavy root whose units any block may take: its wide rows (taken by groups of warps), and for the
+// others the edge tasks or, in rows of more than 128 members, the edge sub-tasks (u, a_t, b).  The block
+// that took the root from the queue publishes it here; blocks that find the root queue empty rebuild
+// its local subgraph and take units from the same cursors.
 struct HeavySlot {
     uint32_t u;            // the root
-    uint32_t units;        // bit 31 once u is published; its rows by class: 10 bits of wide rows
-                           // for large groups, 10 of those for two warps, 11 of the others
-    uint32_t wide_cursor;  // next wide row to take of the first (low half) and second class, and ...
-    uint32_t cursor;       // ... next other row (all may run past the end)
+    uint32_t units;        // bit 31 once u is published; 10 bits of wide rows, 21 of other units
+    uint32_t wide_cursor;  // next wide row: of those for large groups (low half) and of those for two
+                           // warps; either runs to kCursorEnd, and by the blocks that meet its end past it
+    uint32_t cursor;       // next other unit (may run past the end)
 };
 
 struct HelpTable {

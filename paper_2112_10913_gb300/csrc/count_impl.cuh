@@ -997,6 +997,9 @@ constexpr int kMidMaxWarps = 32;
 constexpr uint32_t kMidStaticSmem = 2048;  // room left for the kernel's static shared memory
 constexpr uint32_t kNoHelpSlot = 0xffffffffu;
 constexpr uint32_t kHelpSlots = 8192;    // heavy roots that can take help, per launch
+constexpr uint32_t kUnitMask = (1u << 21) - 1;  // units of a heavy root besides its wide rows (HeavySlot)
+constexpr uint32_t kCursorEnd = 32768;   // where either wide cursor of a heavy root ends (HeavySlot)
+constexpr uint32_t kSplitMembers = 128;  // heavy roots: rows above this many members are cut by member
 constexpr uint32_t kMaxGroups = 15;      // pairs of warps that can head a group (named barriers 1..15)
 
 // Words of the complement rows of a wide set of s members.
@@ -1031,9 +1034,10 @@ __device__ __forceinline__ uint32_t pick_help_slot(const HelpTable &ht, int lane
             const uint32_t un = units.load(cuda::memory_order_acquire);
             const uint32_t cw = *(volatile uint32_t *)&ht.slots[sl].wide_cursor;
             const uint32_t cn = *(volatile uint32_t *)&ht.slots[sl].cursor;
-            const uint32_t big = (un >> 21) & 1023u, mid = (un >> 11) & 1023u, narrow = un & 2047u;
-            const uint32_t cb = cw & 0xffffu, cm = cw >> 16;
-            rem = (cb < big ? big - cb : 0u) + (cm < mid ? mid - cm : 0u) + (cn < narrow ? narrow - cn : 0u);
+            const uint32_t cb = cw & 0xffffu, cm = cw >> 16, other = un & kUnitMask;
+            if (un)
+                rem = (cb < kCursorEnd ? kCursorEnd - cb : 0u) + (cm < kCursorEnd ? kCursorEnd - cm : 0u) +
+                      (cn < other ? other - cn : 0u);
         }
         uint32_t bsl = sl;
 #pragma unroll
@@ -1210,10 +1214,13 @@ __device__ __forceinline__ void wide_row(const WarpCtx &x, const Group &g, uint3
 //       as the root's widest row needs for the rows that two warps cannot hold, then two warps each;
 //       the other rows by one warp each.
 //   D < split_min: the rows are taken from counters in shared memory.
-//   D >= split_min (heavy roots, K >= 6): the rows are taken from cursors in a global table.
-//       Blocks that find the root queue empty pick the published heavy root with the most rows
-//       left, rebuild its rows and take from the same cursors (work stealing across blocks);
-//       every block adds its own part of the root's count.
+//   D >= split_min (heavy roots, K >= 6): the wide rows and the units of the others are taken from
+//       cursors in a global table; a unit is an edge task or, in a row of more than kSplitMembers
+//       members that is not wide (general DAGs, no re-encoding), the sub-task (u, a_t, b) of one
+//       member b: the (K-3)-cliques of row_t ∧ row_b.  Blocks that find the root queue empty pick the
+//       published heavy root with the most units left, rebuild its rows and take from the same
+//       cursors (work stealing across blocks); every block adds its own part of the root's count.
+//       (One root of 800, k = 6, ids kept: 49 ms when whole rows were its units, 14 ms by member.)
 // block_ns (optional): each block's start and end on the global timer.
 // TEAMED: the block is `team_count` teams instead of one (an instance of its own: the plain kernel has no
 // registers to spare).
@@ -1239,7 +1246,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     uint32_t *sL = smem + (size_t)team * team_words;
     uint32_t *rows = sL + dcap;
     __shared__ uint32_t s_idx[kMaxTeams], s_task[kMaxTeams], s_tri[kMaxTeams], s_slot[kMaxTeams], s_u[kMaxTeams],
-        s_unsorted[kMaxTeams];
+        s_unsorted[kMaxTeams], s_units[kMaxTeams];
     // (roots with wide rows are not counted by teams)
     __shared__ uint32_t s_wide[2], s_most;
     __shared__ uint32_t s_cls[2][kBitmapCap / 32];  // wide rows of either class, one bit each
@@ -1249,8 +1256,8 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     uint32_t *wscr = lists + (size_t)w * warp_list_words(dcap, compact_max);
     const uint32_t buf_words = warp_buf_words(dcap, compact_max, K >= 8);
     uint32_t *bufs = lists + (size_t)nw * warp_list_words(dcap, compact_max);
-    // order of a root's rows, wide ones first: it reuses sL, which is dead once the rows are built
-    uint16_t *s_order = reinterpret_cast<uint16_t *>(sL);
+    // units before each of a heavy root's rows: it reuses sL, which is dead once the rows are built
+    uint32_t *s_upre = sL;
     WarpCtx x;
     x.rows = rows;
     x.cbuf = wscr;
@@ -1396,10 +1403,9 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             x.RS = RS;
             x.W = W;
             x.tri = s_tri[team] != 0;
-            // Wide rows come first in the order of the rows: those that need more than two warps'
-            // buffers, the other ones, then the rows of one warp.  A root of at most 129
-            // out-neighbours has no wide row.
-            uint32_t nbig = 0, nmid = 0, narrow = D;
+            // Wide rows: those that need more than two warps' buffers, then the other ones.  A root of
+            // at most 129 out-neighbours has none.
+            uint32_t nbig = 0, nmid = 0, units = D;
             const uint32_t most_gw = 1u << (31 - __clz(nw));  // warps of the largest group
             if constexpr (K >= 5) {
                 if (x.tri && compact_max && D > kNarrow + 1) {
@@ -1425,40 +1431,45 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                             nbig += __popc(s_cls[0][q]);
                             nmid += __popc(s_cls[1][q]);
                         }
-                        for (uint32_t q = w; q < W; q += nw) {
-                            uint32_t rb = 0, rm = 0;
-                            for (uint32_t v = 0; v < q; v++) {
-                                rb += __popc(s_cls[0][v]);
-                                rm += __popc(s_cls[1][v]);
-                            }
-                            const uint32_t t = q * 32 + lane, bb = s_cls[0][q], mb = s_cls[1][q];
-                            rb += __popc(bb & lanemask_lt());
-                            rm += __popc(mb & lanemask_lt());
-                            const uint32_t at = (bb >> lane) & 1u   ? rb
-                                                : (mb >> lane) & 1u ? nbig + rm
-                                                                    : nbig + nmid + (t - rb - rm);
-                            if (t < D) s_order[at] = (uint16_t)t;
-                        }
-                        sync();
                     }
                 }
-                narrow = D - nbig - nmid;
             }
             const uint32_t nwide = nbig + nmid;
+            auto is_wide = [&](uint32_t t) { return ((s_cls[0][t >> 5] | s_cls[1][t >> 5]) >> (t & 31u)) & 1u; };
             if (heavy) {
+                for (uint32_t t = w; t < D; t += nw) {
+                    const uint32_t c = lane < W ? rows[t * RS + lane] : 0u;
+                    const uint32_t m = __reduce_add_sync(kFull, __popc(c));
+                    if (lane == 0)
+                        s_upre[t] = m < (uint32_t)(K - 2) || (nwide && is_wide(t)) ? 0u : m > kSplitMembers ? m : 1u;
+                }
+                sync();
+                if (w == 0) {
+                    uint32_t run = 0;
+                    for (uint32_t t0 = 0; t0 < D; t0 += 32) {
+                        const uint32_t v = t0 + lane < D ? s_upre[t0 + lane] : 0u;
+                        const uint32_t inc = warp_incl_scan(v);
+                        if (t0 + lane < D) s_upre[t0 + lane] = run + inc - v;
+                        run += __shfl_sync(kFull, inc, 31);
+                    }
+                    if (lane == 0) s_units[team] = run;
+                }
+                sync();
+                units = s_units[team];
                 if (tx == 0) {
-                    const uint32_t units = 0x80000000u | (nbig << 21) | (nmid << 11) | narrow;
+                    const uint32_t word = 0x80000000u | (nwide << 21) | units;
                     if (owner && ht.slots) {
                         const uint32_t sl = atomicAdd(ht.nslots, 1u);
                         if (sl < ht.cap) {
                             ht.slots[sl].u = u;
+                            ht.slots[sl].wide_cursor = (kCursorEnd - nmid) << 16 | (kCursorEnd - nbig);
                             cuda::atomic_ref<uint32_t, cuda::thread_scope_device> pub(ht.slots[sl].units);
-                            pub.store(units, cuda::memory_order_release);
+                            pub.store(word, cuda::memory_order_release);
                             s_slot[team] = sl;
                         }
-                    } else if (!owner && ht.slots[s_slot[team]].units != units) {
+                    } else if (!owner && ht.slots[s_slot[team]].units != word) {
                         set_error(err, kDevBadInput);  // the rebuilt root differs from the published one
-                        s_task[team] = narrow;               // take nothing
+                        s_task[team] = units;          // take nothing
                         s_wide[0] = nbig;
                         s_wide[1] = nmid;
                         s_slot[team] = kNoHelpSlot;
@@ -1466,15 +1477,15 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                 }
                 sync();
             }
-            // the rows of a published heavy root are taken from its slot's cursors in global
+            // the units of a published heavy root are taken from its slot's cursors in global
             // memory, the others from the block's counters in shared memory
             HeavySlot *slot = s_slot[team] != kNoHelpSlot ? &ht.slots[s_slot[team]] : nullptr;
             if constexpr (K >= 5) {
-                // Rows s_order[first .. first + count) of class cls by groups of gw warps.  A group is
-                // named by its first warp (barrier and shared state), so that a warp can go on to
-                // the next class while other groups are still at this one: every warp of the new
-                // group has left its old group, whose last barrier it shared with the rest.
-                auto run_wide = [&](int cls, uint32_t first, uint32_t count, uint32_t gw) {
+                // The `count` wide rows of class cls by groups of gw warps.  A group is named by its first
+                // warp (barrier and shared state), so that a warp can go on to the next class while
+                // other groups are still at this one: every warp of the new group has left its old
+                // group, whose last barrier it shared with the rest.
+                auto run_wide = [&](int cls, uint32_t count, uint32_t gw) {
                     const uint32_t w0 = (uint32_t)w & ~(gw - 1);
                     if (w0 + gw > (uint32_t)nw || w0 >= 2 * kMaxGroups) return;
                     Group g;
@@ -1489,15 +1500,17 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                             uint32_t v = count;
                             if (!(heavy && budget.over(err))) {
                                 if (!slot) v = atomicAdd(&s_wide[cls], 1u);
-                                else v = cls == 0 ? atomicAdd(&slot->wide_cursor, 1u) & 0xffffu
-                                                  : atomicAdd(&slot->wide_cursor, 0x10000u) >> 16;
+                                else
+                                    v = (cls == 0 ? atomicAdd(&slot->wide_cursor, 1u) & 0xffffu
+                                                  : atomicAdd(&slot->wide_cursor, 0x10000u) >> 16) -
+                                        (kCursorEnd - count);
                             }
                             *g.sh = {0, v, 0, 0, 0, 0, 0};
                         }
                         g.sync();
                         const uint32_t i = g.sh->unit;
                         if (i >= count) break;
-                        const uint32_t t = s_order[first + i];
+                        const uint32_t t = select_member(lane < W ? s_cls[cls][lane] : 0u, i);
                         const uint32_t c = lane < W ? rows[t * RS + lane] : 0u;
                         wide_row<K - 2, WORK>(x, g, c, lane, acc, work);
                         if (WORK && sink.per_arc) {
@@ -1519,7 +1532,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                     }
 #pragma unroll 1
                     for (int cls = nbig ? 0 : 1; cls < 2; cls++)
-                        run_wide(cls, cls ? nbig : 0u, cls ? nmid : nbig, cls ? 2u : gw);
+                        run_wide(cls, cls ? nmid : nbig, cls ? 2u : gw);
                 }
             }
             // k = 4, upper-triangular rows: the triangles of the local subgraph are the arcs (t, b)'s
@@ -1562,26 +1575,50 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                         acc += s2;
                         __syncwarp();
                     }
-                    narrow = 0;
+                    units = 0;
                 }
             }
-            // a warp claims its next row before it works on the current one, so that the
+            // a warp claims its next unit before it works on the current one, so that the
             // atomic's round trip (global memory for a published heavy root) overlaps the work
             auto claim = [&]() -> uint32_t {
                 uint32_t v = 0;
                 if (lane == 0)
-                    v = heavy && budget.over(err) ? narrow : (slot ? atomicAdd(&slot->cursor, 1u) : atomicAdd(&s_task[team], 1u));
+                    v = heavy && budget.over(err) ? units : (slot ? atomicAdd(&slot->cursor, 1u) : atomicAdd(&s_task[team], 1u));
                 return v;
             };
             uint32_t next_i = claim();
             for (;;) {
                 const uint32_t i = __shfl_sync(kFull, next_i, 0);
-                if (i >= narrow) break;
+                if (i >= units) break;
                 next_i = claim();
-                const uint32_t t = nwide ? s_order[nwide + i] : i;
+                uint32_t t = i, j = 0;
+                bool whole = true;
+                if (heavy) {
+                    // the row of unit i: the last t with s_upre[t] <= i
+                    uint32_t lo = 0, hi = D - 1;
+                    while (lo < hi) {
+                        const uint32_t mid = (lo + hi + 1) >> 1;
+                        if (s_upre[mid] <= i) lo = mid;
+                        else hi = mid - 1;
+                    }
+                    t = lo;
+                    j = i - s_upre[t];
+                    whole = (t + 1 < D ? s_upre[t + 1] : units) - s_upre[t] == 1u;
+                } else if (nwide && is_wide(t)) {
+                    continue;
+                }
                 const uint32_t c = lane < W ? rows[t * RS + lane] : 0u;
-                const uint32_t cnt = __reduce_add_sync(kFull, __popc(c));
-                if (cnt >= K - 2) warp_dfs<K - 2, WORK>(x, c, lane, acc, work);
+                if (whole) {
+                    const uint32_t cnt = __reduce_add_sync(kFull, __popc(c));
+                    if (cnt >= K - 2) warp_dfs<K - 2, WORK>(x, c, lane, acc, work);
+                } else if constexpr (K >= 6) {
+                    // the j-th member b of row t: the sub-task (u, a_t, b)
+                    const uint32_t b = select_member(c, j);
+                    const uint32_t c2 = lane < W ? (c & rows[b * RS + lane]) : 0u;
+                    if (WORK && lane < (int)W) work += 1;
+                    const uint32_t cnt = __reduce_add_sync(kFull, __popc(c2));
+                    if (cnt >= K - 3) warp_dfs<K - 3, WORK>(x, c2, lane, acc, work);
+                }
                 if (WORK && sink.per_arc) {
                     // debug output (instrumented kernel only): acc holds this unit's part of edge
                     // task t alone (it restarts from zero after every unit; the warp's running

@@ -48,3 +48,26 @@ def test_one_dense_set(gpu, oracle_lib, s, p, hubs, k):
     if k <= 6 and s <= 200:
         total, per_arc = G.count_per_arc(k)
         assert total == want and int(per_arc.sum()) == want
+
+
+@pytest.mark.parametrize("s,p", [(140, 0.6), (260, 0.4), (700, 0.15)])
+@pytest.mark.parametrize("k", [6, 7])
+@pytest.mark.parametrize("plan", [dict(relabel=False), dict(compact_max=1), dict(warps_per_cta=2)])
+def test_heavy_roots_cut_by_member(gpu, oracle_lib, s, p, k, plan):
+    """Heavy roots whose rows of more than 128 members are not re-encoded: a DAG that keeps ids, no
+    re-encoding, and rows too wide for the buffers of a block of two warps; split and whole."""
+    import paper_2112_10913_gb300 as cg
+
+    if k == 7 and s == 140:
+        s = 132  # (a shorter oracle run)
+    g = one_set(s, p, s + k)
+    relabel = plan.get("relabel", True)
+    tuned = {a: b for a, b in plan.items() if a != "relabel"}
+    rank = np.arange(g.n, dtype=np.uint32)
+    G = cg.DeviceGraph(g, rank=rank) if relabel else cg.DeviceGraph(g, relabel=False)
+    off, cols = G.dag_numpy()
+    want = oracle_lib.count(off, cols, g.n, k)
+    for split in (33, 129, 0, 1):
+        assert G.count(k, split_min=split, **tuned) == want
+    total, per_arc = G.count_per_arc(k, split_min=33, **tuned)
+    assert total == want and int(per_arc.sum()) == want
