@@ -404,6 +404,7 @@ citron_status citron_count_batch(uint32_t n, const uint64_t *d_dag_off, const ui
         if (!((kmask >> k) & 1)) continue;
         CountRun run;
         run.plan = plan;
+        run.keeps_ids = !d_rank;
         run.filter.group_of_row = gor;
         run.filter.group_k = d_group_k;
         run.filter.ngroups = ngroups;

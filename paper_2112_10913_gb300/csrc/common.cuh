@@ -302,6 +302,7 @@ struct CountRun {
     citron::RootFilter filter;                               // roots of this pass
     bool count_work = false;                 // instrumented launch: count word operations
     bool time_kernels = false;               // record device time of the counting kernels
+    bool keeps_ids = false;                  // the DAG is known to keep vertex ids (run_count finds out)
     bool balance = false;                    // record when each bitmap-path block starts and ends
     unsigned long long budget_ns = 0;        // device time the count may take (0: no limit)
     unsigned long long work = 0;             // out: word operations (AND + POPC of 32-bit words)

@@ -33,7 +33,9 @@ namespace citron {
 
 // counted: the largest out-degree that the launches after this one can count (a caller's bound on
 // the rows may be too small); a root above it is an error.
-__global__ void k_classify(uint32_t n, const uint64_t *__restrict__ dag_off, uint32_t need,
+// dag_cols (optional): look whether the DAG keeps vertex ids (st->down).
+__global__ void k_classify(uint32_t n, const uint64_t *__restrict__ dag_off,
+                           const uint32_t *__restrict__ dag_cols, uint32_t need,
                            uint32_t small_max, uint32_t bitmap_max, uint32_t *small_list,
                            uint32_t *big_list, uint32_t *mid_hist, CountStats *st,
                            unsigned long long *per_root, unsigned long long *per_arc,
@@ -56,6 +58,7 @@ __global__ void k_classify(uint32_t n, const uint64_t *__restrict__ dag_off, uin
         if (D >= need && filter.takes(u)) {
             cls = D <= small_max ? 0 : (D <= bitmap_max ? 2 : 1);
             if (D > counted) set_error(err, kDevBadInput);
+            if (dag_cols && cls == 2 && dag_cols[dag_off[u]] < u) st->down = 1;
         }
     }
     uint32_t off_in_warp[2] = {0, 0}, warp_base[2] = {0, 0};
@@ -86,9 +89,11 @@ __global__ void k_classify(uint32_t n, const uint64_t *__restrict__ dag_off, uin
     if (cls == 1) big_list[s_base[1] + warp_base[1] + off_in_warp[1]] = u;
 }
 
-// Bin starts for the mid roots in DESCENDING out-degree: cursor[d] = #roots with degree > d.
+// Bin starts for the mid roots in DESCENDING out-degree: cursor[d] = #roots with degree > d.  The roots
+// of at most `low` out-neighbours, the end of the queue, are left to the launch of small blocks if there
+// are at least min_low of them, and, in a DAG found to keep vertex ids, only without roots above.
 __global__ __launch_bounds__(1024) void k_mid_bins(const uint32_t *hist, uint32_t bins, uint32_t low,
-                                                    uint32_t *cursor, CountStats *st)
+                                                    uint32_t min_low, uint32_t *cursor, CountStats *st)
 {
     __shared__ uint32_t scratch[33];
     // reversed index: position i holds degree bins-1-i
@@ -101,10 +106,13 @@ __global__ __launch_bounds__(1024) void k_mid_bins(const uint32_t *hist, uint32_
     for (uint32_t i = lo; i < hi; i++) {
         const uint32_t d = bins - 1 - i;
         cursor[d] = run;
-        if (d == low) st->n_high = run;  // (zero when no degree above it has a bin)
+        if (d == low) st->n_high = total - run >= min_low && !(run && st->down) ? run : total;
         run += hist[d];
     }
-    if (threadIdx.x == 0) st->n_mid = total;
+    if (threadIdx.x == 0) {
+        st->n_mid = total;
+        if (low >= bins) st->n_high = total >= min_low ? 0u : total;  // no degree above the line has a bin
+    }
 }
 
 __global__ void k_mid_scatter(uint32_t n, const uint64_t *__restrict__ dag_off, uint32_t need,
@@ -230,6 +238,13 @@ size_t count_ws_bytes(uint32_t n, uint32_t max_outdeg, int num_sms)
     return s.used;
 }
 
+// Roots of at most low_max out-neighbours from which on they get a launch of small blocks.
+static uint32_t min_low_roots(uint32_t k, const CountPlan &plan, int num_sms)
+{
+    if (k == 6 && plan.compact_max == 0) return 0xffffffffu;
+    return (uint32_t)num_sms * kLowSlotsPerSm * kLowPerSlot;
+}
+
 // Runs the count for k >= 3.  Returns a CUDA error, or cudaErrorMemoryAllocation when the
 // workspace is too small.  The host value lands in *h_result.
 cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_cols, uint32_t k,
@@ -267,10 +282,11 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
     const uint32_t need = k - 1;
     const uint32_t blocks = (n + 255) / 256;
     if (n) {
-        k_classify<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max,
+        k_classify<<<blocks, 256, 0, s>>>(n, dag_off, k == 6 ? dag_cols : nullptr, need, plan.small_max, plan.bitmap_max,
                                           small_list, big_list, hist, st, run.sink.per_root,
                                           run.sink.per_arc, run.filter, 0xffffffffu, err);
-        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, low_max(k), cursor, st);
+        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, low_max(k),
+                                        min_low_roots(k, plan, num_sms), cursor, st);
         k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max,
                                              cursor, mid_list, run.filter);
         note_launches(3);
@@ -278,6 +294,7 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
     CountStats hs;
     if ((e = cudaMemcpyAsync(&hs, st, sizeof(hs), cudaMemcpyDeviceToHost, s))) return e;
     if ((e = cudaStreamSynchronize(s))) return e;
+    hs.n_low = hs.n_mid - hs.n_high;
 #define CITRON_CASE(KK)                                                                           \
     case KK:                                                                                      \
         e = launch_count_##KK(run, dag_off, dag_cols, hs, st, small_list, mid_list, big_list,     \
@@ -353,22 +370,27 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     uint32_t counted = plan.small_max;
     if (max_outdeg > plan.bitmap_max) counted = 0xffffffffu;
     else if (max_outdeg > plan.small_max) counted = min((max_outdeg + 31) & ~31u, plan.bitmap_max);
-    k_classify<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max, small_list,
+    k_classify<<<blocks, 256, 0, s>>>(n, dag_off, nullptr, need, plan.small_max, plan.bitmap_max, small_list,
                                       big_list, hist, st, nullptr, nullptr, run.filter, counted, err);
     note_launches(1);
+    // With no row above the line one launch is enough: of small blocks unless there are too few vertices.
+    const uint32_t max_mid = max_outdeg < plan.bitmap_max ? max_outdeg : plan.bitmap_max;
+    uint32_t min_low = min_low_roots(k, plan, num_sms);
+    if (n < min_low || (k == 6 && run.keeps_ids && max_mid > low_max(k))) min_low = 0xffffffffu;
+    else if (max_mid <= low_max(k)) min_low = 0u;
     if (max_outdeg > plan.small_max) {  // else no row is on the bitmap path
-        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, low_max(k), cursor, st);
+        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, low_max(k), min_low, cursor, st);
         k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max, cursor,
                                              mid_list, run.filter);
         note_launches(2);
     }
     CountStats hs = {};
     hs.n_small = max_outdeg >= need ? n : 0;
-    hs.max_mid = max_outdeg < plan.bitmap_max ? max_outdeg : plan.bitmap_max;
+    hs.max_mid = max_mid;
     hs.n_mid = hs.max_mid > plan.small_max ? n : 0;
     // upper bounds of both parts of the queue: the kernels read the real ones on the device
-    hs.n_high = hs.max_mid > low_max(k) ? n : 0;
-    hs.bound = 1;
+    hs.n_high = min_low ? n : 0;
+    hs.n_low = min_low == 0xffffffffu ? 0 : n;
     hs.max_big = max_outdeg;
     hs.n_big = max_outdeg > plan.bitmap_max ? n : 0;
     run.time_kernels = false;

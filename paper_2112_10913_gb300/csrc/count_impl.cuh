@@ -21,8 +21,9 @@ constexpr uint32_t kMidWindow = 32768;  // ids in a block's membership bitmap (k
 struct CountStats {
     uint32_t n_small, n_mid, n_big;
     uint32_t max_mid, max_big, max_all;
-    uint32_t n_high;  // bitmap-path roots above low_max, the first n_high of the queue
-    uint32_t bound;   // host copy only: the numbers are upper bounds (each part may hold n_mid roots)
+    uint32_t n_high;  // bitmap-path roots of the launch of large blocks, the first n_high of the queue
+    uint32_t n_low;   // host copy only: the others, or an upper bound of them
+    uint32_t down;    // k = 6: some row reaches below its own id (a DAG that keeps vertex ids)
 };
 
 // Bitmap-path roots of at most low_max(k) out-neighbours run in a launch of their own, in blocks of 8
@@ -32,6 +33,15 @@ struct CountStats {
 // (R-MAT 15, k = 8: 69 ms in one launch, 129 in two at 128), so only the smallest roots, which the
 // warp-register path leaves to this one there, go in small blocks.
 constexpr uint32_t kLowWarps = 8;
+// That launch needs kLowPerSlot such roots for every block of 8 warps that the chip holds: with fewer a
+// root is left to 8 warps while others idle, and what is a short launch of its own comes after the
+// tail of the other one.  40 roots of 99, k = 6,
+// ids kept: 2.4 ms in small blocks, 1.4 in large ones; R-MAT 15, k = 4: 0.22 ms against 0.31.
+// At k = 6 sets that are enumerated (a DAG that keeps ids, no re-encoding) outweigh their rows' build as
+// they do from k = 7 on, and the queue is not cut in two: R-MAT 15, ids kept, 13.9 ms in two launches,
+// 10.9 in one.  (Without roots above the line one launch of small blocks is still better: 200,000
+// vertices of degree 50, 1.8 ms against 3.5.)
+constexpr uint32_t kLowSlotsPerSm = 4, kLowPerSlot = 4;
 // Under a cap on the blocks, that launch's blocks hold up to kMaxTeams teams of 8 warps, each with roots
 // of its own: as many blocks of 8 warps as the cap's warps are spread over all SMs, and no block of
 // 32 warps of another stream finds an empty one.  114 blocks, 180,000 roots of at most 119, k = 4..6,
@@ -1890,7 +1900,7 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
             return e;
         uint32_t grid = 0;
         for (int low = 0; low < 2; low++) {
-            const uint32_t n_roots = !low ? hs.n_high : hs.bound ? hs.n_mid : hs.n_mid - hs.n_high;
+            const uint32_t n_roots = low ? hs.n_low : hs.n_high;
             if (!n_roots) continue;
             const uint32_t dmax = low && hs.max_mid > low_max(K) ? low_max(K) : hs.max_mid;
             const uint32_t dcap = (dmax + 31) & ~31u, rs = (dcap / 32) | 1;
