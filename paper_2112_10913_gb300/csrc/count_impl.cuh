@@ -277,7 +277,8 @@ struct WarpCtx {
     uint32_t *lbuf;
     uint32_t *mv;    // compress masks: 5 per candidate word, then the member prefix per word
     uint32_t *mbuf;  // compact rows, 4 words each (16-byte aligned); aliases lbuf
-    uint32_t compact_max;  // largest candidate set re-encoded compactly by one warp (0 or 128)
+    uint32_t compact_max;  // largest candidate set re-encoded compactly by one warp (0 or 128) ...
+    uint32_t compact3_max;  // ... and at R = 3 (as many members as its buffer holds packed rows of, up to 192)
     uint32_t pair_cap;     // uint16 entries of elem
     uint32_t *err;
 };
@@ -381,12 +382,33 @@ __device__ __forceinline__ uint32_t tri_rounds(const WarpCtx &x, const uint32_t 
 // ---- Compact re-encoding of a candidate set ------------------------------------------------
 // A candidate set with s members (listed in elem) is re-encoded as the s x s adjacency of its
 // induced subgraph: bit j of row i is member j, so that the remaining levels work on ceil(s/32)
-// words per set instead of the root-wide span.  What is stored is the COMPLEMENT, symmetric (the
-// members j that are not adjacent to member i): dense sets are counted on it (dense.cuh); a set
-// with more than half of its pairs missing is turned back into upper-triangular adjacency rows
-// and enumerated (cdfs below).  Sets of at most 128 members are handled by one warp (one 16-byte
-// load per row), wider ones by a group of warps (wide_row).
+// words per set instead of the root-wide span.  Dense sets are counted on the symmetric COMPLEMENT
+// (dense.cuh), the others enumerated on upper-triangular adjacency rows (cdfs below).  Sets of at
+// most 128 members are handled by one warp, one uint4 per row.  Wider edge tasks that are dense are
+// counted by a group of warps (wide_row); at R = 3 the others of up to 192 members take packed rows of 5
+// or 6 words (below), and the rest stays on the root-wide bitmap.
 //
+// The line between the sides, in 64ths of a set's pairs that may be missing.  Where the sides cross
+// (G(n, p), every set on either side): sets of one warp at p = 0.55 (k = 6: 183 us on either side at
+// 0.5, 240 against 254 at 0.6; for k = 5 they stay within 5 % from 0.5 to 0.8), small sets of deep walks
+// later, because a 4-clique form costs a few hundred instructions however small its set is (k = 8, 40
+// copies of G(100, 0.5): 0.65 ms with the line at one half, 0.47 now).  Wide sets pay for the groups and
+// barriers: at k = 5 packed rows are better to p = 0.77 (G(400, 0.7) 0.50 -> 0.31 ms), root-wide ones to
+// 0.65; at k = 6 0.57 (G(400, 0.5) 0.77 -> 0.41); from k = 7 on, where the set's own members are walked
+// first, 0.73 (G(700, 0.5) 72 -> 29 ms, G(400, 0.7) 82 -> 42).
+__host__ __device__ constexpr uint32_t dense_line(int R, uint32_t s)
+{
+    if (s <= kNarrow) return R == 3 ? 28 : R >= 6 && s <= 32 ? 20 : 28;
+    return R == 3 ? (s <= 192 ? 14 : 22) : R == 4 ? 28 : 17;
+}
+// Whether a set of s members of which `missing` of `pairs` pairs (all, or a sample) are not adjacent is
+// counted on its complement.
+template <int R>
+__device__ __forceinline__ bool is_dense(uint32_t s, uint32_t missing, uint32_t pairs)
+{
+    return 64 * missing <= dense_line(R, s) * pairs;
+}
+
 // Compress masks and member prefix of every candidate word (lane w: word w), for the builders.
 __device__ __forceinline__ void prepare_masks(const WarpCtx &x, int clo, int chi, int lane)
 {
@@ -442,7 +464,69 @@ __device__ __forceinline__ uint32_t complement_round(const WarpCtx &x, uint32_t 
     return bits;
 }
 
-// Complement rows of the s <= 128 members of a set by one warp, one uint4 per row in mbuf.
+// Upper-triangular adjacency rows of the s <= 128 members of a set (words in cbuf, members in elem;
+// triangular layout) by one warp, one uint4 per row in mbuf.  Returns this lane's arcs.
+__device__ __forceinline__ uint32_t build_rows(const WarpCtx &x, uint32_t s, int clo, int chi, int lane)
+{
+    prepare_masks(x, clo, chi, lane);
+    uint4 *M = reinterpret_cast<uint4 *>(x.mbuf);
+    uint32_t arcs = 0;
+    for (uint32_t i0 = 0; i0 < s; i0 += 32) {
+        const uint32_t i = i0 + lane;
+        const uint32_t *row = x.rows + (uint32_t)x.elem[i < s ? i : i0] * x.RS;
+        uint32_t o[4] = {0, 0, 0, 0};
+        // rows hold bits above their own member only: start at the word of the first member
+        int w = (int)(x.elem[i0] >> 5);
+        uint32_t ow = x.mv[160 + w] >> 5, sh = x.mv[160 + w] & 31u, cur = 0;
+        // (the member prefix is the same on every lane: the words fill and leave at uniform places)
+        auto leave = [&]() {
+            if (ow == 0) o[0] = cur;
+            else if (ow == 1) o[1] = cur;
+            else if (ow == 2) o[2] = cur;
+            else o[3] = cur;
+        };
+        for (; w < chi; w++) {
+            const uint32_t m = x.cbuf[w];
+            if (!m) continue;
+            const uint32_t piece = member_bits(x, row[w], m, w);
+            cur |= piece << sh;
+            const uint32_t end = sh + __popc(m);
+            if (end >= 32) {
+                leave();
+                ow++;
+                cur = sh ? piece >> (32 - sh) : 0u;
+            }
+            sh = end & 31u;
+        }
+        if (sh) leave();
+        if (i < s) {
+            M[i] = make_uint4(o[0], o[1], o[2], o[3]);
+            arcs += __popc(o[0]) + __popc(o[1]) + __popc(o[2]) + __popc(o[3]);
+        }
+    }
+    __syncwarp();
+    return arcs;
+}
+
+// mbuf from upper-triangular adjacency rows to complement rows of the s <= 128 members (a word of a
+// row is read before its mirror image is written by the same lane: block rows in order).
+__device__ __forceinline__ void rows_to_complement(const WarpCtx &x, uint32_t s, int lane)
+{
+    const uint4 *M = reinterpret_cast<const uint4 *>(x.mbuf);
+    const uint32_t nblk = (s + 31) >> 5;
+    for (uint32_t a = 0; a < nblk; a++) {
+        const uint32_t i = (a << 5) + lane;
+        const uint4 r = M[i < s ? i : s - 1];
+        const uint32_t g[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (uint32_t ow = 0; ow < 4; ow++)
+            if (ow >= a && ow < nblk) put_block(x.mbuf, 0, s, a, ow, g[ow], lane);
+        __syncwarp();
+    }
+}
+
+// Complement rows of the s <= 128 members of a set by one warp, one uint4 per row in mbuf.  Returns
+// the complement's bits written by this lane (over all lanes, twice its edges).
 __device__ __forceinline__ uint32_t build_complement(const WarpCtx &x, uint32_t s, int clo, int chi, int lane)
 {
     prepare_masks(x, clo, chi, lane);
@@ -480,6 +564,128 @@ __device__ __forceinline__ void drop_top(uint32_t (&Y)[CW])
             Y[q] &= ~(0x80000000u >> __clz(Y[q]));
             done = true;
         }
+    }
+}
+
+// o[q] |= lo, o[q + 1] |= hi for a warp-uniform q (the member prefix of a candidate word is the
+// same on every lane): a uniform branch instead of a select per output word.
+template <int NW>
+__device__ __forceinline__ void place_piece(uint32_t (&o)[NW], uint32_t q, uint32_t lo, uint32_t hi)
+{
+#pragma unroll
+    for (int t = 0; t < NW; t++) {
+        if (q == (uint32_t)t) {
+            o[t] |= lo;
+            if (t + 1 < NW) o[t + 1] |= hi;
+        }
+    }
+}
+
+// Packed triangular compact rows for R = 3 sets of 129..192 members (CW = 5 or 6 words): the row
+// of member i holds only its words q = i/32 .. CW-1 (the words below are zero in an
+// upper-triangular sub-DAG), so 192 rows take 672 words instead of 1152 and fit the warp's
+// scratch.  Rows of the members of word q start at packed_base(q) and are (CW - q) words long.
+template <int CW>
+__host__ __device__ constexpr uint32_t packed_base(int q)
+{
+    return q <= 0 ? 0u : packed_base<CW>(q - 1) + 32u * (uint32_t)(CW - (q - 1));
+}
+
+__host__ __device__ constexpr uint32_t packed_words(int cw) { return 16u * (uint32_t)(cw * (cw + 1)); }
+
+template <int CW>
+__device__ __forceinline__ void build_packed(const WarpCtx &x, uint32_t s, int clo, int chi, int lane)
+{
+    prepare_masks(x, clo, chi, lane);
+#pragma unroll
+    for (int q = 0; q < CW; q++) {
+        const uint32_t i0 = (uint32_t)q * 32;
+        if (i0 >= s) break;
+        const uint32_t i = i0 + lane;
+        const bool act = i < s;
+        const uint32_t ei = act ? x.elem[i] : x.elem[i0];
+        const uint32_t *row = x.rows + ei * x.RS;
+        uint32_t o[CW];
+#pragma unroll
+        for (int t = 0; t < CW; t++) o[t] = 0;
+        for (int w = (int)(x.elem[i0] >> 5); w < chi; w++) {
+            const uint32_t m = x.cbuf[w];
+            if (!m) continue;
+            uint32_t mv[5];
+#pragma unroll
+            for (int t = 0; t < 5; t++) mv[t] = x.mv[t * 32 + w];
+            const uint32_t pre = x.mv[160 + w];
+            const uint32_t piece = compress_with(row[w], m, mv);
+            const uint32_t qq = pre >> 5, sh = pre & 31;
+            const uint32_t lo = piece << sh, hi = sh ? (piece >> (32 - sh)) : 0u;
+            place_piece<CW>(o, qq, lo, hi);
+        }
+        if (act) {
+            uint32_t *dst = x.mbuf + packed_base<CW>(q) + (uint32_t)lane * (CW - q);
+#pragma unroll
+            for (int t = q; t < CW; t++) dst[t - q] = o[t];
+        }
+    }
+    __syncwarp();
+}
+
+// Arcs inside the lane's set D (CW words; zero below word Q2) on packed rows; Y = the members
+// to visit (D without its highest member).
+template <int CW, bool WORK, int Q2>
+__device__ __forceinline__ void packed_leaf(const uint32_t *P, const uint32_t (&D)[CW],
+                                            const uint32_t (&Y)[CW], uint32_t &ones, uint32_t &s,
+                                            unsigned long long &work)
+{
+    if constexpr (Q2 < CW) {
+        uint32_t y = Y[Q2];
+        if (WORK) work += (unsigned long long)__popc(y) * (CW - Q2);
+        // two members per step (the highest and the lowest), their words paired in the adder
+        while (y & (y - 1u)) {
+            const uint32_t j1 = 31u - __clz(y);
+            const uint32_t lb = y & (0u - y);
+            const uint32_t j2 = 31u - __clz(lb);
+            y ^= (1u << j1) | lb;
+            const uint32_t *r1 = P + packed_base<CW>(Q2) + j1 * (CW - Q2);
+            const uint32_t *r2 = P + packed_base<CW>(Q2) + j2 * (CW - Q2);
+#pragma unroll
+            for (int w = Q2; w < CW; w++) csa_add(ones, D[w] & r1[w - Q2], D[w] & r2[w - Q2], s);
+        }
+        if (y) {
+            const uint32_t *rj = P + packed_base<CW>(Q2) + (31u - __clz(y)) * (CW - Q2);
+#pragma unroll
+            for (int w = Q2; w + 1 < CW; w += 2) csa_add(ones, D[w] & rj[w - Q2], D[w + 1] & rj[w + 1 - Q2], s);
+            if ((CW - Q2) & 1) s += __popc(D[CW - 1] & rj[CW - 1 - Q2]);
+        }
+        packed_leaf<CW, WORK, Q2 + 1>(P, D, Y, ones, s, work);
+    }
+}
+
+// Triangles of a dense compact set of s members (members 0..s-1) on packed rows: lane l takes
+// member 32q + l of each word q, forms D = C ∧ row and adds the arcs inside D.
+template <int CW, bool WORK, int Q>
+__device__ __forceinline__ void packed_r3(const uint32_t *P, uint32_t s_members, int lane,
+                                          uint32_t &s, unsigned long long &work)
+{
+    if constexpr (Q < CW) {
+        const uint32_t m = (uint32_t)Q * 32 + lane;
+        if (m < s_members) {
+            const uint32_t *rm = P + packed_base<CW>(Q) + (uint32_t)lane * (CW - Q);
+            uint32_t D[CW];
+#pragma unroll
+            for (int w = 0; w < CW; w++) {
+                const uint32_t cw = (uint32_t)w * 32 >= s_members ? 0u
+                                    : (s_members >= (uint32_t)w * 32 + 32 ? kFull : ((1u << (s_members - w * 32)) - 1));
+                D[w] = w < Q ? 0u : (cw & rm[w - Q]);
+            }
+            uint32_t Y[CW];
+#pragma unroll
+            for (int w = 0; w < CW; w++) Y[w] = D[w];
+            drop_top<CW>(Y);
+            uint32_t ones = 0, t = 0;
+            packed_leaf<CW, WORK, Q>(P, D, Y, ones, t, work);
+            s += t + __popc(ones);
+        }
+        packed_r3<CW, WORK, Q + 1>(P, s_members, lane, s, work);
     }
 }
 
@@ -547,21 +753,20 @@ __device__ __forceinline__ void cdfs_word(const uint4 *M, const uint32_t (&C)[CW
 // every lane of a round holds a member (dealing by bit position would leave the lanes of the
 // absent members idle); lane r forms D = C ∧ row(m_r) and adds the arcs inside D.
 template <int CW, bool TRI, bool WORK>
-__device__ __forceinline__ void cdfs3_dealt(const WarpCtx &x, const uint32_t (&C)[CW], int lane,
+__device__ __forceinline__ void cdfs3_dealt(const uint4 *M, uint16_t *elem, const uint32_t (&C)[CW], int lane,
                                             unsigned long long &acc, unsigned long long &work)
 {
-    const uint4 *M = reinterpret_cast<const uint4 *>(x.mbuf);
     uint32_t total = 0;
 #pragma unroll
     for (int q = 0; q < CW; q++) {
-        if ((C[q] >> lane) & 1) x.elem[total + __popc(C[q] & lanemask_lt())] = (uint16_t)(q * 32 + lane);
+        if ((C[q] >> lane) & 1) elem[total + __popc(C[q] & lanemask_lt())] = (uint16_t)(q * 32 + lane);
         total += __popc(C[q]);
     }
     __syncwarp();
     uint32_t s = 0, ones = 0;
     for (uint32_t r0 = 0; r0 < total; r0 += 32) {
         if (r0 + lane < total) {
-            const uint32_t m = x.elem[r0 + lane];
+            const uint32_t m = elem[r0 + lane];
             const uint4 mi = M[m];
             uint32_t D[CW];
             D[0] = C[0] & mi.x;
@@ -584,12 +789,11 @@ __device__ __forceinline__ void cdfs3_dealt(const WarpCtx &x, const uint32_t (&C
     __syncwarp();
 }
 
-// R-cliques inside the compact set C (CW words, the same on every lane); rows in mbuf.
+// R-cliques inside the compact set C (CW words, the same on every lane) on rows M.
 template <int R, int CW, bool TRI, bool WORK>
-__device__ __forceinline__ void cdfs(const WarpCtx &x, const uint32_t (&C)[CW], int lane,
+__device__ __forceinline__ void cdfs(const uint4 *M, uint16_t *elem, const uint32_t (&C)[CW], int lane,
                                      unsigned long long &acc, unsigned long long &work)
 {
-    const uint4 *M = reinterpret_cast<const uint4 *>(x.mbuf);
     if constexpr (R == 1) {
         if (lane == 0) {
             uint32_t t = 0;
@@ -631,8 +835,8 @@ __device__ __forceinline__ void cdfs(const WarpCtx &x, const uint32_t (&C)[CW], 
             for (int t = 0; t < CW; t++) cnt += __popc(C2[t]);
             if (WORK && lane == 0) work += CW;
             if (cnt >= R - 1) {
-                if constexpr (R == 4) cdfs3_dealt<CW, TRI, WORK>(x, C2, lane, acc, work);
-                else cdfs<R - 1, CW, TRI, WORK>(x, C2, lane, acc, work);
+                if constexpr (R == 4) cdfs3_dealt<CW, TRI, WORK>(M, elem, C2, lane, acc, work);
+                else cdfs<R - 1, CW, TRI, WORK>(M, elem, C2, lane, acc, work);
             }
         }
     }
@@ -643,11 +847,9 @@ __device__ __forceinline__ void cdfs(const WarpCtx &x, const uint32_t (&C)[CW], 
 // p forming D = M[i] ∧ M[j] and adding the arcs inside D.  Dealing the members of each C ∧ M[i]
 // on its own leaves the lanes above |C ∧ M[i]| idle; pairs of many i fill every lane.
 template <int CW, bool WORK>
-__device__ __forceinline__ void cdfs4_pairs(const WarpCtx &x, uint32_t s, uint32_t cap, int lane,
+__device__ __forceinline__ void cdfs4_pairs(const uint4 *M, uint16_t *pairs, uint32_t s, uint32_t cap, int lane,
                                             unsigned long long &acc, unsigned long long &work)
 {
-    const uint4 *M = reinterpret_cast<const uint4 *>(x.mbuf);
-    uint16_t *pairs = x.elem;
     uint32_t sum = 0, ones = 0, n = 0;
     auto drain = [&]() {
         __syncwarp();
@@ -696,7 +898,7 @@ __device__ __forceinline__ void cdfs4_pairs(const WarpCtx &x, uint32_t s, uint32
 }
 
 template <int R, int CW, bool TRI, bool WORK>
-__device__ __forceinline__ void cdfs_all(const WarpCtx &x, uint32_t s, int lane,
+__device__ __forceinline__ void cdfs_all(const uint4 *M, uint16_t *elem, uint32_t cap, uint32_t s, int lane,
                                          unsigned long long &acc, unsigned long long &work)
 {
     uint32_t C[CW];
@@ -705,8 +907,8 @@ __device__ __forceinline__ void cdfs_all(const WarpCtx &x, uint32_t s, int lane,
         const uint32_t lo = q * 32;
         C[q] = s >= lo + 32 ? kFull : (s > lo ? ((1u << (s - lo)) - 1) : 0u);
     }
-    if constexpr (R == 4 && TRI) cdfs4_pairs<CW, WORK>(x, s, x.pair_cap, lane, acc, work);
-    else cdfs<R, CW, TRI, WORK>(x, C, lane, acc, work);
+    if constexpr (R == 4 && TRI) cdfs4_pairs<CW, WORK>(M, elem, s, cap, lane, acc, work);
+    else cdfs<R, CW, TRI, WORK>(M, elem, C, lane, acc, work);
 }
 
 // A compact set's complement rows (chunk-major, dense.cuh): S rows per chunk, nch chunks.
@@ -762,9 +964,9 @@ __device__ __forceinline__ void dense_dfs(const WarpCtx &x, const CompSet &cs, u
                     __syncwarp();
                     Bs[lane] = nc;
                     __syncwarp();
-                    const CompCount t = comp3_wide<false, WORK>(M, cs.S, cs.nch, Bs, m, ng, 0, 1, lane);
+                    const CompCount t = comp3_wide<WORK>(M, cs.S, cs.nch, Bs, m, ng, 0, 1, lane);
                     if (WORK) work += t.work;
-                    n += n3_finish(m, __reduce_add_sync(kFull, t.n), false);
+                    n += n3_finish(m, __reduce_add_sync(kFull, t.n));
                 }
             } else {
                 unsigned long long sl = o.sl;
@@ -816,7 +1018,7 @@ __device__ __noinline__ LaneSums packed_dfs(const WarpCtx x, uint32_t *m32, uint
     return o;
 }
 
-// C(s, R) for s <= 128 and R <= 11 (below 2^51).
+// C(s, R) for s <= 128 and R <= 10 (below 2^48).
 template <int R>
 __device__ __forceinline__ unsigned long long choose(uint32_t s)
 {
@@ -826,28 +1028,22 @@ __device__ __forceinline__ unsigned long long choose(uint32_t s)
     return v;
 }
 
-// A set with more than half of its pairs missing: its rows are turned back and enumerated.  Out of
-// line: sets of an edge task are seldom sparse, and the code would push the others' out of the
-// instruction cache.
+// A set that is not dense, on its rows in mbuf.  Out of line: the sets of a dense core's edge tasks are
+// seldom sparse, and the code would push the others' out of the instruction cache.
 template <int R, int CW, bool WORK>
-__device__ __noinline__ LaneSums sparse_count(const WarpCtx x, uint32_t s, int lane)
+__device__ __noinline__ LaneSums sparse_count(const uint4 *M, uint16_t *elem, uint32_t cap, uint32_t s, int lane)
 {
     LaneSums o = {0, 0};
-    complement_to_rows(x, s, lane);
-    cdfs_all<R, CW, true, WORK>(x, s, lane, o.acc, o.work);
+    cdfs_all<R, CW, true, WORK>(M, elem, cap, s, lane, o.acc, o.work);
     return o;
 }
 
 // Counts a set of s members with CW words: its complement rows are in mbuf.
 template <int R, int CW, bool WORK>
-__device__ __forceinline__ void compact_count(const WarpCtx &x, uint32_t s, bool dense, int lane,
-                                              unsigned long long &acc, unsigned long long &work)
+__device__ __forceinline__ void compact_count(const WarpCtx &x, uint32_t s, int lane, unsigned long long &acc,
+                                              unsigned long long &work)
 {
-    if (!dense) {
-        const LaneSums o = sparse_count<R, CW, WORK>(x, s, lane);
-        acc += o.acc;
-        if (WORK) work += o.work;
-    } else if constexpr (R == 3) {
+    if constexpr (R == 3) {
         x.cbuf[lane] = word_mask(s, lane);
         __syncwarp();
         const CompCount o = comp3<CW, WORK>(reinterpret_cast<const uint4 *>(x.mbuf), x.cbuf, s, lane);
@@ -859,24 +1055,66 @@ __device__ __forceinline__ void compact_count(const WarpCtx &x, uint32_t s, bool
     }
 }
 
-// Entry for a candidate set of at most compact_max members (lane word c), triangular layout.
-// The complement is worked when it has at most half of the pairs: its levels cost its edges, the
-// enumeration's cost the adjacent pairs.
-template <int R, bool WORK>
+// Triangles of a set of 129..192 members (lane word c) on packed rows.
+template <bool WORK>
+__device__ __forceinline__ LaneSums packed_count(const WarpCtx &x, uint32_t s, int clo, int chi, int lane)
+{
+    LaneSums o = {0, 0};
+    uint32_t t = 0;
+    if (s <= 160) {
+        build_packed<5>(x, s, clo, chi, lane);
+        packed_r3<5, WORK, 0>(x.mbuf, s, lane, t, o.work);
+    } else {
+        build_packed<6>(x, s, clo, chi, lane);
+        packed_r3<6, WORK, 0>(x.mbuf, s, lane, t, o.work);
+    }
+    o.acc = t;
+    return o;
+}
+
+// packed_count out of line, for the walks of k >= 6 (their kernels are short of registers).
+template <bool WORK>
+__device__ __noinline__ LaneSums packed_call(const WarpCtx x, uint32_t s, int clo, int chi, int lane)
+{
+    return packed_count<WORK>(x, s, clo, chi, lane);
+}
+
+// Entry for a candidate set of at most compact_max members (R = 3: compact3_max; lane word c),
+// triangular layout.  TASK: the set is an edge task's.
+template <int R, bool WORK, bool TASK>
 __device__ __forceinline__ void compact_entry(const WarpCtx &x, uint32_t c, int lane,
                                               unsigned long long &acc, unsigned long long &work)
 {
     int clo, chi;
     const uint32_t s = compact(x, c, lane, clo, chi);
-    if (s >= (uint32_t)R) {
-        const uint32_t twice = __reduce_add_sync(kFull, build_complement(x, s, clo, chi, lane));
-        if (twice == 0) {  // a clique
+    if (R == 3 && s > kNarrow) {
+        const LaneSums o = TASK ? packed_count<WORK>(x, s, clo, chi, lane) : packed_call<WORK>(x, s, clo, chi, lane);
+        acc += o.acc;
+        if (WORK) work += o.work;
+    } else if (s >= (uint32_t)R) {
+        // An edge task's own set at k = 5 is packed as it is and mirrored when it is dense; deeper
+        // walks pack the complement and turn it back when it is not.
+        constexpr bool kRowsFirst = R == 3 && TASK;
+        const uint32_t pairs = s * (s - 1) / 2;
+        const uint32_t missing =
+            kRowsFirst ? pairs - __reduce_add_sync(kFull, build_rows(x, s, clo, chi, lane))
+                       : __reduce_add_sync(kFull, build_complement(x, s, clo, chi, lane)) / 2;
+        if (!is_dense<R>(s, missing, pairs)) {
+            if (!kRowsFirst) complement_to_rows(x, s, lane);
+            const uint4 *M = reinterpret_cast<const uint4 *>(x.mbuf);
+            const LaneSums o = s <= 32   ? sparse_count<R, 1, WORK>(M, x.elem, x.pair_cap, s, lane)
+                               : s <= 64 ? sparse_count<R, 2, WORK>(M, x.elem, x.pair_cap, s, lane)
+                               : s <= 96 ? sparse_count<R, 3, WORK>(M, x.elem, x.pair_cap, s, lane)
+                                         : sparse_count<R, 4, WORK>(M, x.elem, x.pair_cap, s, lane);
+            acc += o.acc;
+            if (WORK) work += o.work;
+        } else if (missing == 0) {  // a clique
             if (lane == 0) add_acc(acc, choose<R>(s), x.err);
         } else {
-            const bool dense = 2 * twice <= s * (s - 1);
-            if (s <= 32) compact_count<R, 1, WORK>(x, s, dense, lane, acc, work);
-            else if (s <= 64) compact_count<R, 2, WORK>(x, s, dense, lane, acc, work);
-            else compact_count<R, 4, WORK>(x, s, dense, lane, acc, work);
+            if (kRowsFirst) rows_to_complement(x, s, lane);
+            if (s <= 32) compact_count<R, 1, WORK>(x, s, lane, acc, work);
+            else if (s <= 64) compact_count<R, 2, WORK>(x, s, lane, acc, work);
+            else compact_count<R, 4, WORK>(x, s, lane, acc, work);
         }
     }
     __syncwarp();
@@ -884,20 +1122,20 @@ __device__ __forceinline__ void compact_entry(const WarpCtx &x, uint32_t c, int 
 
 // Counts the R-cliques inside the candidate set whose word w sits in lane w (words >= W are
 // zero); adds lane-partial sums to acc.
-//   R >= 3, triangular layout, at most compact_max members: re-encoded compactly
-//           (compact_entry) and finished on the compact rows.
+//   R >= 3, triangular layout, at most compact_max (R = 3: compact3_max) members: re-encoded
+//           compactly (compact_entry) and finished on the compact rows.
 //   R >= 4: warp-uniform walk over the members a; the next candidate set c ∧ row_a is again
 //           spread over the lanes (one shared-memory load per lane).
 //   R == 3: members are compacted and dealt to lanes; each lane builds its own c ∧ row_a and
 //           sums its arcs (the last two levels run lane-parallel).
 //   R == 2: members dealt to lanes, each adds |c ∧ row_a|.
-template <int R, bool WORK>
+template <int R, bool WORK, bool TASK = false>
 __device__ __forceinline__ void warp_dfs(const WarpCtx &x, uint32_t c, int lane,
                                          unsigned long long &acc, unsigned long long &work)
 {
     if constexpr (R >= 3) {
-        if (x.tri && __reduce_add_sync(kFull, __popc(c)) <= x.compact_max) {
-            compact_entry<R, WORK>(x, c, lane, acc, work);
+        if (x.tri && __reduce_add_sync(kFull, __popc(c)) <= (R == 3 ? x.compact3_max : x.compact_max)) {
+            compact_entry<R, WORK, TASK>(x, c, lane, acc, work);
             return;
         }
     }
@@ -998,10 +1236,6 @@ __host__ __device__ __forceinline__ uint32_t warp_buf_words(uint32_t dcap, uint3
     const uint32_t m = compact_max ? compact_max * 4 + (deep ? 256 + 128 : 0) : 0u;
     return dcap > m ? dcap : m;
 }
-__host__ __device__ __forceinline__ uint32_t warp_scratch_words(uint32_t dcap, uint32_t compact_max, bool deep)
-{
-    return warp_list_words(dcap, compact_max) + warp_buf_words(dcap, compact_max, deep);
-}
 
 constexpr int kMidMaxWarps = 32;
 constexpr uint32_t kMidStaticSmem = 2048;  // room left for the kernel's static shared memory
@@ -1069,7 +1303,7 @@ __device__ __forceinline__ uint32_t pick_help_slot(const HelpTable &ht, int lane
 // Shared state of a group of warps on a wide row.
 struct GroupShared {
     unsigned long long sl;
-    uint32_t unit, mbar, sd, st, next, over;
+    uint32_t unit, sd, st, next, over;
 };
 
 // A group's place: gw warps (a power of two), this warp's index gi, its named barrier.
@@ -1097,7 +1331,7 @@ __device__ __forceinline__ uint32_t select_member(uint32_t c, uint32_t r)
     return (uint32_t)wl * 32 + select_bit(word, r - before);
 }
 
-// R-cliques (R >= 3) of a row c (lane word, more than 128 members; triangular layout), counted by
+// R-cliques (R >= 3) of a dense row c (lane word, more than 128 members; triangular layout), counted by
 // the warps of a group together: they build the complement rows (32 members per round), then R = 3
 // and R = 4 are one pass over (32 members, chunk of 128 codegrees) units, and for R >= 5 the warps
 // take the members one at a time and walk down from there.  Every warp of the group calls this.
@@ -1135,102 +1369,110 @@ __device__ __forceinline__ void wide_row(const WarpCtx &x, const Group &g, uint3
     g.sync();
     const CompSet cs = {g.buf, s, (s + 127) >> 7};
     const uint32_t nblk = (s + 31) >> 5;
-    uint32_t bits = 0;
     // rounds get shorter: dealt forth and back
     for (uint32_t a = 0; a < nblk; a++) {
         const uint32_t p = a & (g.gw - 1);
-        if ((a & g.gw ? g.gw - 1 - p : p) == g.gi) bits += complement_round(y, cs.m32, s, s, a, chi, lane);
+        if ((a & g.gw ? g.gw - 1 - p : p) == g.gi) complement_round(y, cs.m32, s, s, a, chi, lane);
     }
-    bits = __reduce_add_sync(kFull, bits);
-    if (lane == 0) atomicAdd(&g.sh->mbar, bits);
     g.sync();
     x.cbuf[lane] = word_mask(s, lane);
     __syncwarp();
-    const bool dense = 2 * g.sh->mbar <= s * (s - 1);
     const uint4 *M = reinterpret_cast<const uint4 *>(cs.m32);
     bool counted = false;
     if constexpr (R == 3) {
-        // either side of the pairs: the complement's triangles and Goodman's identity, or the set's
-        CompCount o = dense ? comp3_wide<false, WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, lane)
-                            : comp3_wide<true, WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, lane);
+        CompCount o = comp3_wide<WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, lane);
         if (WORK) work += o.work;
         o.n = __reduce_add_sync(kFull, o.n);
         if (lane == 0) atomicAdd(&g.sh->sd, o.n);
         g.sync();
-        if (g.gi == 0 && lane == 0) add_acc(acc, n3_finish(s, g.sh->sd, !dense), x.err);
+        if (g.gi == 0 && lane == 0) add_acc(acc, n3_finish(s, g.sh->sd), x.err);
         counted = true;
-    } else if (dense) {
-        if constexpr (R == 4) {
-            CompSums o = comp4_wide<WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, x.mv, lane);
-            if (WORK) work += o.work;
-            const bool over = __any_sync(kFull, o.over);
-            o.sd = __reduce_add_sync(kFull, o.sd);
-            o.st = __reduce_add_sync(kFull, o.st);
+    } else if constexpr (R == 4) {
+        CompSums o = comp4_wide<WORK>(M, s, cs.nch, x.cbuf, s, nblk, g.gi, g.gw, x.mv, lane);
+        if (WORK) work += o.work;
+        const bool over = __any_sync(kFull, o.over);
+        o.sd = __reduce_add_sync(kFull, o.sd);
+        o.st = __reduce_add_sync(kFull, o.st);
 #pragma unroll
-            for (int k = 16; k > 0; k >>= 1) o.sl += __shfl_xor_sync(kFull, o.sl, k);
-            if (lane == 0) {
-                if (over) atomicOr(&g.sh->over, 1u);
-                atomicAdd(&g.sh->sd, o.sd);
-                atomicAdd(&g.sh->st, o.st);
-                atomicAdd(&g.sh->sl, o.sl);
-            }
-            g.sync();
-            counted = !g.sh->over;
-            if (counted && g.gi == 0 && lane == 0)
-                add_acc(acc, n4_finish(s, g.sh->sd, g.sh->st, g.sh->sl), x.err);
+        for (int k = 16; k > 0; k >>= 1) o.sl += __shfl_xor_sync(kFull, o.sl, k);
+        if (lane == 0) {
+            if (over) atomicOr(&g.sh->over, 1u);
+            atomicAdd(&g.sh->sd, o.sd);
+            atomicAdd(&g.sh->st, o.st);
+            atomicAdd(&g.sh->sl, o.sl);
         }
+        g.sync();
+        counted = !g.sh->over;
+        if (counted && g.gi == 0 && lane == 0)
+            add_acc(acc, n4_finish(s, g.sh->sd, g.sh->st, g.sh->sl), x.err);
     }
-    if (!counted) {
-        // member by member: on the complement rows when they are sparse, else on the root's rows
-        for (;;) {
+    if constexpr (R >= 4) {
+        while (!counted) {  // member by member
             uint32_t r = 0;
             if (lane == 0) r = atomicAdd(&g.sh->next, 1u);
             r = __shfl_sync(kFull, r, 0);
             if (r >= s) break;
-            if (dense) {
-                if constexpr (R >= 4) {
-                    const uint32_t nc = adjacent_above(cs, word_mask(s, lane), r, lane);
-                    const uint32_t m = __reduce_add_sync(kFull, __popc(nc));
-                    if (m < R - 1) continue;
-                    if constexpr (R == 4) {
-                        __syncwarp();
-                        x.cbuf[lane] = nc;
-                        __syncwarp();
-                        const CompCount o = comp3_wide<false, WORK>(M, s, cs.nch, x.cbuf, m, nblk, 0, 1, lane);
-                        if (WORK) work += o.work;
-                        const uint32_t sum = __reduce_add_sync(kFull, o.n);
-                        if (lane == 0) add_acc(acc, n3_finish(m, sum, false), x.err);
-                    } else {
-                        dense_dfs<R - 1, 0, WORK>(x, cs, nc, m, lane, acc, work);
-                    }
-                }
+            const uint32_t nc = adjacent_above(cs, word_mask(s, lane), r, lane);
+            const uint32_t m = __reduce_add_sync(kFull, __popc(nc));
+            if (m < R - 1) continue;
+            if constexpr (R == 4) {
+                __syncwarp();
+                x.cbuf[lane] = nc;
+                __syncwarp();
+                const CompCount o = comp3_wide<WORK>(M, s, cs.nch, x.cbuf, m, nblk, 0, 1, lane);
+                if (WORK) work += o.work;
+                const uint32_t sum = __reduce_add_sync(kFull, o.n);
+                if (lane == 0) add_acc(acc, n3_finish(m, sum), x.err);
             } else {
-                const uint32_t b = select_member(c, r);
-                const uint32_t c2 = lane < (int)x.W ? (c & x.rows[b * x.RS + lane]) : 0u;
-                if (WORK && lane < (int)x.W) work += 1;
-                const uint32_t m = __reduce_add_sync(kFull, __popc(c2));
-                if (m >= R - 1) warp_dfs<R - 1, WORK>(x, c2, lane, acc, work);
+                dense_dfs<R - 1, 0, WORK>(x, cs, nc, m, lane, acc, work);
             }
         }
     }
+}
+
+// Whether the set of m > 128 members whose word w sits in lane w (triangular layout) is dense enough
+// for a group of warps: the arcs above 32 of its members, spread evenly, against the line.
+template <int R>
+__device__ __noinline__ bool wide_dense(const uint32_t *rows, uint32_t RS, uint32_t c, uint32_t m, int lane)
+{
+    // member r of the set in lane l: the word in which r falls (binary search over the lanes' prefix
+    // sums), then the bit
+    const uint32_t r = (uint32_t)lane * m >> 5, pc = __popc(c), excl = warp_incl_scan(pc) - pc;
+    uint32_t o = 0;
+#pragma unroll
+    for (uint32_t step = 16; step > 0; step >>= 1) {
+        const uint32_t e = __shfl_sync(kFull, excl, (o + step) & 31u);
+        if (e <= r) o += step;
+    }
+    // (empty words share their prefix with the next: the search ends at the last of them, which holds r)
+    const uint32_t word = __shfl_sync(kFull, c, o), before = __shfl_sync(kFull, excl, o);
+    const uint32_t *row = rows + (o * 32 + select_bit(word, r - before)) * RS;
+    uint32_t arcs = 0;
+    for (uint32_t nz = __ballot_sync(kFull, c != 0); nz; nz &= nz - 1) {
+        const int w = __ffs(nz) - 1;
+        arcs += __popc(__shfl_sync(kFull, c, w) & row[w]);
+    }
+    const uint32_t pairs = __reduce_add_sync(kFull, m - 1 - r);
+    return is_dense<R>(m, pairs - __reduce_add_sync(kFull, arcs), pairs);
 }
 
 // Bitmap path (small_max < D <= dcap): one block (or one of its `teams`) per root, roots taken largest-D first from the
 // queue.  The block builds the root's local subgraph as D x D bitmap rows in shared memory
 // (row i = V(g_u) ∩ N+(a_i), Algorithm GenSub-CITRON by sorted-list intersection) and its warps
 // count the (K-2)-cliques of every row: the edge tasks (u, a_t).
-//   K >= 5, triangular layout: rows of more than 128 members (wide rows) are counted first, each
+//   K >= 5, triangular layout: dense rows of more than 128 members (wide rows) are counted first, each
 //       by a group of warps whose scratch buffers together hold its complement rows: as many warps
 //       as the root's widest row needs for the rows that two warps cannot hold, then two warps each;
 //       the other rows by one warp each.
-//   D < split_min: the rows are taken from counters in shared memory.
+//   D < split_min: the rows are taken from counters in shared memory, and cut like a heavy root's where
+//       there are sparse ones of more than kSplitMembers members.
 //   D >= split_min (heavy roots, K >= 6): the wide rows and the units of the others are taken from
 //       cursors in a global table; a unit is an edge task or, in a row of more than kSplitMembers
-//       members that is not wide (general DAGs, no re-encoding), the sub-task (u, a_t, b) of one
+//       members that is not wide (sparse rows, general DAGs, no re-encoding), the sub-task (u, a_t, b) of one
 //       member b: the (K-3)-cliques of row_t ∧ row_b.  Blocks that find the root queue empty pick the
 //       published heavy root with the most units left, rebuild its rows and take from the same
 //       cursors (work stealing across blocks); every block adds its own part of the root's count.
-//       (One root of 800, k = 6, ids kept: 49 ms when whole rows were its units, 14 ms by member.)
+//       (One root of 800, k = 6, ids kept: 49 ms when whole rows were its units, 15 ms by member.)
 // block_ns (optional): each block's start and end on the global timer.
 // TEAMED: the block is `team_count` teams instead of one (an instance of its own: the plain kernel has no
 // registers to spare).
@@ -1238,7 +1480,7 @@ template <int K, bool WORK, bool TEAMED>
 __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     const uint64_t *__restrict__ dag_off, const uint32_t *__restrict__ dag_cols,
     const uint32_t *__restrict__ list, const CountStats *st, uint32_t *next, int low, int team_count, uint32_t dcap,
-    uint32_t team_words, uint32_t window, uint32_t compact_max, uint32_t split_min, HelpTable ht,
+    uint32_t team_words, uint32_t buf_words, uint32_t window, uint32_t compact_max, uint32_t split_min, HelpTable ht,
     unsigned long long *result, RootSink sink, unsigned long long *work_out, unsigned long long *block_ns, Budget budget,
     uint32_t *err)
 {
@@ -1258,13 +1500,12 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     __shared__ uint32_t s_idx[kMaxTeams], s_task[kMaxTeams], s_tri[kMaxTeams], s_slot[kMaxTeams], s_u[kMaxTeams],
         s_unsorted[kMaxTeams], s_units[kMaxTeams];
     // (roots with wide rows are not counted by teams)
-    __shared__ uint32_t s_wide[2], s_most;
+    __shared__ uint32_t s_wide[2], s_most, s_sparse, s_ask;
     __shared__ uint32_t s_cls[2][kBitmapCap / 32];  // wide rows of either class, one bit each
     __shared__ unsigned long long s_acc[32], s_arc[32];
     __shared__ GroupShared s_group[kMaxGroups];
     uint32_t *lists = K > 3 ? rows + (size_t)dcap * rs_cap : rows;  // k = 3 keeps no rows
     uint32_t *wscr = lists + (size_t)w * warp_list_words(dcap, compact_max);
-    const uint32_t buf_words = warp_buf_words(dcap, compact_max, K >= 8);
     uint32_t *bufs = lists + (size_t)nw * warp_list_words(dcap, compact_max);
     // units before each of a heavy root's rows: it reuses sL, which is dead once the rows are built
     uint32_t *s_upre = sL;
@@ -1276,6 +1517,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
     x.lbuf = bufs + (size_t)w * buf_words;
     x.mbuf = x.lbuf;
     x.compact_max = compact_max;
+    x.compact3_max = !compact_max ? 0u : buf_words >= packed_words(6) ? 192u : buf_words >= packed_words(5) ? 160u : 128u;
     x.pair_cap = dcap;
     x.err = err;
     // the membership window of the root being built lies over the warps' lists and buffers
@@ -1296,6 +1538,8 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             s_task[team] = 0;
             s_wide[0] = s_wide[1] = 0;
             s_most = 0;
+            s_sparse = 0;
+            s_ask = 0;
             s_tri[team] = 1;
             s_unsorted[team] = 0;
             s_slot[team] = kNoHelpSlot;
@@ -1424,19 +1668,31 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                         uint32_t m = 0;
                         if (t < D)
                             for (uint32_t v = q; v < W; v++) m += __popc(rows[t * RS + v]);
-                        // a row too wide for the block's buffers is left to one warp
-                        const bool wide = m > kNarrow && wide_words(m) <= buf_words * most_gw;
-                        const bool big = wide && wide_words(m) > buf_words * 2;
-                        const uint32_t bb = __ballot_sync(kFull, big), mb = __ballot_sync(kFull, wide && !big);
-                        const uint32_t most = __reduce_max_sync(kFull, wide ? m : 0u);
+                        // a row too wide for the block's buffers, or sparse, is left to one warp
+                        const bool fits = m > kNarrow && nw > 1 && wide_words(m) <= buf_words * most_gw;
+                        const uint32_t ask = __ballot_sync(kFull, fits);
                         if (lane == 0) {
-                            s_cls[0][q] = bb;
-                            s_cls[1][q] = mb;
-                            if (most) atomicMax(&s_most, most);
+                            s_cls[0][q] = ask;
+                            s_cls[1][q] = 0;
+                            if (ask) s_ask = 1;
                         }
                     }
                     sync();
-                    if (s_most) {
+                    if (s_ask) {
+                        for (uint32_t t = w; t < D; t += nw) {
+                            if (!((*(volatile uint32_t *)&s_cls[0][t >> 5] >> (t & 31u)) & 1u)) continue;
+                            const uint32_t c = lane < W ? rows[t * RS + lane] : 0u;
+                            const uint32_t m = __reduce_add_sync(kFull, __popc(c));
+                            const bool dense = wide_dense<K - 2>(rows, RS, c, m, lane);
+                            const bool big = wide_words(m) > buf_words * 2;
+                            if (lane == 0) {
+                                if (!dense || !big) atomicAnd(&s_cls[0][t >> 5], ~(1u << (t & 31u)));
+                                if (dense && !big) atomicOr(&s_cls[1][t >> 5], 1u << (t & 31u));
+                                if (dense) atomicMax(&s_most, m);
+                                else s_sparse = 1;
+                            }
+                        }
+                        sync();
                         for (uint32_t q = 0; q < W; q++) {
                             nbig += __popc(s_cls[0][q]);
                             nmid += __popc(s_cls[1][q]);
@@ -1446,7 +1702,8 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
             }
             const uint32_t nwide = nbig + nmid;
             auto is_wide = [&](uint32_t t) { return ((s_cls[0][t >> 5] | s_cls[1][t >> 5]) >> (t & 31u)) & 1u; };
-            if (heavy) {
+            const bool cut = heavy || (K >= 6 && !TEAMED && s_sparse);
+            if (cut) {
                 for (uint32_t t = w; t < D; t += nw) {
                     const uint32_t c = lane < W ? rows[t * RS + lane] : 0u;
                     const uint32_t m = __reduce_add_sync(kFull, __popc(c));
@@ -1466,6 +1723,8 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                 }
                 sync();
                 units = s_units[team];
+            }
+            if (heavy) {
                 if (tx == 0) {
                     const uint32_t word = 0x80000000u | (nwide << 21) | units;
                     if (owner && ht.slots) {
@@ -1515,7 +1774,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                                                   : atomicAdd(&slot->wide_cursor, 0x10000u) >> 16) -
                                         (kCursorEnd - count);
                             }
-                            *g.sh = {0, v, 0, 0, 0, 0, 0};
+                            *g.sh = {0, v, 0, 0, 0, 0};
                         }
                         g.sync();
                         const uint32_t i = g.sh->unit;
@@ -1603,7 +1862,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                 next_i = claim();
                 uint32_t t = i, j = 0;
                 bool whole = true;
-                if (heavy) {
+                if (cut) {
                     // the row of unit i: the last t with s_upre[t] <= i
                     uint32_t lo = 0, hi = D - 1;
                     while (lo < hi) {
@@ -1620,7 +1879,7 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
                 const uint32_t c = lane < W ? rows[t * RS + lane] : 0u;
                 if (whole) {
                     const uint32_t cnt = __reduce_add_sync(kFull, __popc(c));
-                    if (cnt >= K - 2) warp_dfs<K - 2, WORK>(x, c, lane, acc, work);
+                    if (cnt >= K - 2) warp_dfs<K - 2, WORK, true>(x, c, lane, acc, work);
                 } else if constexpr (K >= 6) {
                     // the j-th member b of row t: the sub-task (u, a_t, b)
                     const uint32_t b = select_member(c, j);
@@ -1837,7 +2096,8 @@ struct Timer {
 
 template <int K, bool WORK, bool TEAMED>
 static cudaError_t launch_mid(uint32_t grid_cap, uint32_t block_cap, int low, uint32_t teams, uint32_t dcap,
-                              uint32_t window, uint32_t compact_max, uint32_t split_min, const HelpTable &ht,
+                              uint32_t buf_words, uint32_t window, uint32_t compact_max, uint32_t split_min,
+                              const HelpTable &ht,
                               uint32_t warps, size_t team_smem, const uint64_t *dag_off,
                               const uint32_t *dag_cols, const uint32_t *mid_list,
                               const CountStats *st, uint32_t *next, unsigned long long *result,
@@ -1869,7 +2129,7 @@ static cudaError_t launch_mid(uint32_t grid_cap, uint32_t block_cap, int low, ui
     if (grid > (uint32_t)num_sms * kMidBlocksPerSmCap) grid = (uint32_t)num_sms * kMidBlocksPerSmCap;
     *grid_out = grid;
     k_count_mid<K, WORK, TEAMED><<<grid, warps * 32, smem, s>>>(dag_off, dag_cols, mid_list, st, next, low, (int)teams, dcap,
-                                                        (uint32_t)(team_smem / sizeof(uint32_t)), window, compact_max,
+                                                        (uint32_t)(team_smem / sizeof(uint32_t)), buf_words, window, compact_max,
                                                         split_min, ht, result, sink, work, block_ns, budget, err);
     note_launches(1);
     return cudaGetLastError();
@@ -1906,13 +2166,19 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
             const uint32_t dcap = (dmax + 31) & ~31u, rs = (dcap / 32) | 1;
             uint32_t warps = plan.warps_per_cta > (uint32_t)kMidMaxWarps ? kMidMaxWarps : plan.warps_per_cta;
             if (low && warps > kLowWarps) warps = kLowWarps;
+            uint32_t buf_words = warp_buf_words(dcap, compact_max, K >= 8);
             auto scratch = [&](uint32_t nw) {  // words for the warps' lists and buffers
-                return K > 3 ? (size_t)nw * warp_scratch_words(dcap, compact_max, K >= 8) : (size_t)kMidWindow / 32;
+                return K > 3 ? (size_t)nw * (warp_list_words(dcap, compact_max) + buf_words) : (size_t)kMidWindow / 32;
             };
             auto smem_for = [&](uint32_t nw) {
                 return ((size_t)dcap + (K > 3 ? (size_t)dcap * rs : 0) + scratch(nw)) * sizeof(uint32_t);
             };
             while (warps > 1 && smem_for(warps) > (size_t)smem_cap) warps--;
+            // room for the packed rows of 192 members where it costs no warp
+            if (const uint32_t was = buf_words; compact_max && dcap > kNarrow && was < packed_words(6)) {
+                buf_words = packed_words(6);
+                if (smem_for(warps) > (size_t)smem_cap) buf_words = was;
+            }
             // the window's bitmap and first places (k > 3) have to fit the scratch
             uint32_t window = kMidWindow;
             while ((size_t)window / 32 + (K > 3 ? window / 64 : 0) > scratch(warps)) window /= 2;
@@ -1928,7 +2194,7 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
             auto launch = [&](auto kind) {
                 constexpr int v = decltype(kind)::value;  // 0 plain, 1 instrumented, 2 in teams
                 return launch_mid<K, v == 1, v == 2>((n_roots + teams - 1) / teams, plan.max_blocks, low, teams, dcap,
-                                                     window, compact_max, plan.split_min, aux.help, warps,
+                                                     buf_words, window, compact_max, plan.split_min, aux.help, warps,
                                                      smem_for(warps), dag_off, dag_cols, mid_list, st, queue, result,
                                                      run.sink, work, ns, aux.budget, &this_grid, err, s, num_sms);
             };

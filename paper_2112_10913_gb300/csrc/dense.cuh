@@ -22,9 +22,8 @@
 //
 // What bounds it: instruction issue (and, for the 4-clique form, instruction fetch): listing a set,
 // packing its rows and the adders outweigh the word operations.  k_count_mid, k = 6 on R-MAT 20:
-// 683 ms enumerating the sets' arcs, 231 ms when this came in, 209 ms now; k = 8 on R-MAT 15: 577 ms,
-// 69 and 55.  The line between the sides is one half of the pairs: the cost of either is about
-// its edges.
+// 683 ms enumerating the sets' arcs, 231 ms when this came in, 207 ms now; k = 8 on R-MAT 15: 577 ms,
+// 69 and 57.  Where the line between the sides lies: dense_line (count_impl.cuh).
 //
 // All arithmetic is exact modulo 2^32 (sets of at most 128 members) or 2^64; the results are
 // below the modulus.
@@ -453,14 +452,13 @@ __device__ __noinline__ void pack_subset(const uint4 *M, uint32_t uw, uint32_t u
 
 // Adjacent pairs (x, y) inside D (CW words), x in D's word T (bits b): y in a later word into `once`,
 // y in the same word into `twice` (both orders).  Two members x per step, the highest and the
-// lowest.  INV: the rows hold the complement of the adjacency meant (x itself is then counted once
-// in `twice`; the caller takes that off).
+// lowest.
 struct PairSums {
     uint32_t ones, once, ones2, twice;
     __device__ __forceinline__ uint32_t both() const { return 2 * (once + __popc(ones)) + twice + __popc(ones2); }
 };
 
-template <int CW, int T, bool INV>
+template <int CW, int T>
 __device__ __forceinline__ void pair_word(const uint4 *M, const uint32_t (&D)[CW], uint32_t b, uint32_t base, PairSums &p)
 {
     while (b) {
@@ -472,7 +470,7 @@ __device__ __forceinline__ void pair_word(const uint4 *M, const uint32_t (&D)[CW
         load_row<CW>(M, base + b2, r2);
 #pragma unroll
         for (int w = T < 0 ? 0 : T; w < CW; w++) {
-            const uint32_t x1 = D[w] & (INV ? ~r1[w] : r1[w]), x2 = D[w] & (INV ? ~r2[w] : r2[w]) & two;
+            const uint32_t x1 = D[w] & r1[w], x2 = D[w] & r2[w] & two;
             if (w == T) csa_add(p.ones2, x1, x2, p.twice);
             else csa_add(p.ones, x1, x2, p.once);
         }
@@ -483,7 +481,7 @@ template <int CW, int T>
 __device__ __forceinline__ void pair_words(const uint4 *M, const uint32_t (&D)[CW], PairSums &p)
 {
     if constexpr (T < CW) {
-        pair_word<CW, T, false>(M, D, D[T], (uint32_t)T << 5, p);
+        pair_word<CW, T>(M, D, D[T], (uint32_t)T << 5, p);
         pair_words<CW, T + 1>(M, D, p);
     }
 }
@@ -787,9 +785,8 @@ __device__ __forceinline__ unsigned long long n4_finish(uint32_t s32, uint32_t s
     return (s * (s - 1) * (s - 2) * (s - 3) / 6 - 2 * m * (s - 2) * (s - 3) + 2 * m * (m - 1) - 4 * s * (st / 6) + sl) >> 2;
 }
 
-// As comp4_wide, for N3: lane-partial sum over the warp's share of d(s-1-d) + 2 t, or with INV, for a
-// set that is the sparse side itself, twice its triangles (n3_finish).
-template <bool INV, bool WORK>
+// As comp4_wide, for N3: lane-partial sum over the warp's share of d(s-1-d) + 2 t (n3_finish).
+template <bool WORK>
 __device__ __noinline__ CompCount comp3_wide(const uint4 *M, uint32_t S, uint32_t nch, const uint32_t *Bs,
                                              uint32_t s, uint32_t ngroups, uint32_t u0, uint32_t ustep, int lane)
 {
@@ -802,7 +799,7 @@ __device__ __noinline__ CompCount comp3_wide(const uint4 *M, uint32_t S, uint32_
         const uint32_t g = u / nch, q = u - g * nch;
         const uint32_t v = (g << 5) + lane;
         if ((Bs[g] >> lane) & 1u) {
-            if (!INV && (v >> 7) == q) {
+            if ((v >> 7) == q) {
                 uint32_t d = 0;
                 for (uint32_t c = 0; c < nch; c++) {
                     const uint4 h = M[c * S + v], b = B4[c];
@@ -816,7 +813,7 @@ __device__ __noinline__ CompCount comp3_wide(const uint4 *M, uint32_t S, uint32_
                 const uint4 a = M[c * S + v], b = B4[c];
                 const uint32_t x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-                for (int t = 0; t < 4; t++) h[t] = (INV ? ~x[t] : x[t]) & y[t] & above_word(v, (c << 2) + t);
+                for (int t = 0; t < 4; t++) h[t] = x[t] & y[t] & above_word(v, (c << 2) + t);
             };
             if (q >= (g >> 2)) {
                 const uint4 *Mq = M + q * S;
@@ -828,15 +825,14 @@ __device__ __noinline__ CompCount comp3_wide(const uint4 *M, uint32_t S, uint32_
                         later(c, h);
 #pragma unroll
                         for (int t = 0; t < 4; t++) {
-                            pair_word<4, -1, INV>(Mq, D, h[t], (c << 7) + (t << 5), p);
+                            pair_word<4, -1>(Mq, D, h[t], (c << 7) + (t << 5), p);
                             if (WORK) o.work += 4 * __popc(h[t]);
                         }
                     }
-                    pair_word<4, 0, INV>(Mq, D, D[0], (q << 7), p);
-                    pair_word<4, 1, INV>(Mq, D, D[1], (q << 7) + 32, p);
-                    pair_word<4, 2, INV>(Mq, D, D[2], (q << 7) + 64, p);
-                    pair_word<4, 3, INV>(Mq, D, D[3], (q << 7) + 96, p);
-                    if (INV) lin -= __popc(D[0]) + __popc(D[1]) + __popc(D[2]) + __popc(D[3]);
+                    pair_word<4, 0>(Mq, D, D[0], (q << 7), p);
+                    pair_word<4, 1>(Mq, D, D[1], (q << 7) + 32, p);
+                    pair_word<4, 2>(Mq, D, D[2], (q << 7) + 64, p);
+                    pair_word<4, 3>(Mq, D, D[3], (q << 7) + 96, p);
                     if (WORK) o.work += 3 * (__popc(D[0]) + __popc(D[1]) + __popc(D[2]) + __popc(D[3]));
                 }
             }
@@ -848,10 +844,10 @@ __device__ __noinline__ CompCount comp3_wide(const uint4 *M, uint32_t S, uint32_
 }
 
 // N3 of a set of s members from its sum.
-__device__ __forceinline__ unsigned long long n3_finish(uint32_t s32, uint32_t sum, bool inv)
+__device__ __forceinline__ unsigned long long n3_finish(uint32_t s32, uint32_t sum)
 {
     const unsigned long long s = s32;
-    return (inv ? sum : (uint32_t)(s * (s - 1) * (s - 2) / 3) - sum) >> 1;
+    return ((uint32_t)(s * (s - 1) * (s - 2) / 3) - sum) >> 1;
 }
 
 }  // namespace citron

@@ -71,3 +71,29 @@ def test_heavy_roots_cut_by_member(gpu, oracle_lib, s, p, k, plan):
         assert G.count(k, split_min=split, **tuned) == want
     total, per_arc = G.count_per_arc(k, split_min=33, **tuned)
     assert total == want and int(per_arc.sum()) == want
+
+
+# Sets around the line between the two sides: one warp's (k = 5, 6, 8), small ones of deep walks, wide
+# ones on packed rows of 5 and 6 words, on the root-wide bitmap and by groups
+LINE = [(s, p, k) for s in (31, 32, 33, 96, 97, 128) for p, k in ((0.56, 5), (0.56, 6), (0.56, 8), (0.69, 8))]
+LINE += [(s, p, 5) for s in (129, 160, 161, 192) for p in (0.45, 0.78)]
+LINE += [(s, p, 5) for s in (193, 400) for p in (0.5, 0.66)]
+LINE += [(s, p, 6) for s in (129, 300) for p in (0.4, 0.57)]
+LINE += [(s, p, 7) for s in (129, 170) for p in (0.5, 0.73)]
+
+
+@pytest.mark.parametrize("s,p,k", LINE)
+def test_sets_around_the_line(gpu, oracle_lib, s, p, k):
+    import paper_2112_10913_gb300 as cg
+
+    g = one_set(s, p, s * 11 + k)
+    rank = np.arange(g.n, dtype=np.uint32)
+    off, cols = oracle_lib.dag_by_rank(g.off, g.cols, g.n, rank, relabel=True)
+    want = oracle_lib.count(off, cols, g.n, k)
+    G = cg.DeviceGraph(g, rank=rank)
+    assert G.count(k) == want
+    assert G.count(k, warps_per_cta=3) == want
+    assert G.count(k, split_min=33) == want
+    if k <= 6:
+        total, per_arc = G.count_per_arc(k)
+        assert total == want and int(per_arc.sum()) == want
