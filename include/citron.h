@@ -188,8 +188,7 @@ citron_status citron_list(uint32_t n, const uint64_t *d_dag_off, const uint32_t 
                                         built for k <= 8: larger k returns CITRON_E_UNSUPPORTED) */
 #define CITRON_COUNT_BALANCE 4u      /* fill busy_ms (each bitmap-path block's start and end) */
 typedef struct {
-    uint32_t small_max;      /* in: warp-register path for out-degree <= small_max, 0..32
-                                (0: 32, for k >= 7 16) */
+    uint32_t small_max;      /* in: warp-register path for out-degree <= small_max, 0..32 (0: 32) */
     uint32_t bitmap_max;     /* in: shared-memory bitmap path up to this out-degree, <= 1024
                                 (0: 1024); larger roots take the sorted-list path */
     uint32_t warps_per_cta;  /* in: warps per bitmap-path block, 1..32 (0: 32); fewer are used

@@ -183,8 +183,7 @@ static bool plan_from_opts(const citron_count_opts *opts, CountPlan &plan)
     if (opts->compact_max) plan.compact_max = opts->compact_max == 1 ? 0 : opts->compact_max;
     if (opts->split_min) plan.split_min = opts->split_min == 1 ? 0xffffffffu : opts->split_min;
     plan.max_blocks = opts->max_blocks;
-    const uint32_t least = plan.small_max ? plan.small_max : 32;
-    if (plan.bitmap_max < least) plan.bitmap_max = least;
+    if (plan.bitmap_max < plan.small_max) plan.bitmap_max = plan.small_max;
     return true;
 }
 

@@ -279,14 +279,8 @@ namespace citron_host {
 // the deep recursion of k = 9..12 takes most of the build's time, and debug modes there are rare.
 constexpr uint32_t kInstrumentedMaxK = 8;
 
-// Default of small_max.  The warp-register path enumerates its 32-bit sets; for k >= 7 the larger
-// roots among them are better off on the bitmap path, which ends four levels earlier (dense.cuh):
-// R-MAT 15, k = 8: 13.1 ms of the warp-register path up to 32, 0.4 ms up to 16, the bitmap path
-// 69 ms either way.  At k = 6 the blocks' overhead on R-MAT 20 takes that back.
-inline uint32_t small_default(uint32_t k) { return k >= 7 ? 16 : 32; }
-
 struct CountPlan {
-    uint32_t small_max = 0;        // roots with out-degree <= this use the warp-register path (0: small_default)
+    uint32_t small_max = 32;       // roots with out-degree <= this use the warp-register path
     uint32_t bitmap_max = 1024;    // ... <= this use the shared-memory bitmap path
     uint32_t warps_per_cta = 32;   // warps per block of the bitmap path (fewer if shared memory is short)
     uint32_t compact_max = 128;    // candidate sets up to this size are re-encoded compactly (0: never)

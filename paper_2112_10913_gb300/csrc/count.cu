@@ -91,9 +91,10 @@ __global__ void k_classify(uint32_t n, const uint64_t *__restrict__ dag_off,
 
 // Bin starts for the mid roots in DESCENDING out-degree: cursor[d] = #roots with degree > d.  The roots
 // of at most `low` out-neighbours, the end of the queue, are left to the launch of small blocks if there
-// are at least min_low of them, and, in a DAG found to keep vertex ids, only without roots above.
+// are at least min_low of them, and, with `together` or in a DAG found to keep vertex ids, only without
+// roots above.
 __global__ __launch_bounds__(1024) void k_mid_bins(const uint32_t *hist, uint32_t bins, uint32_t low,
-                                                    uint32_t min_low, uint32_t *cursor, CountStats *st)
+                                                    uint32_t min_low, bool together, uint32_t *cursor, CountStats *st)
 {
     __shared__ uint32_t scratch[33];
     // reversed index: position i holds degree bins-1-i
@@ -106,7 +107,7 @@ __global__ __launch_bounds__(1024) void k_mid_bins(const uint32_t *hist, uint32_
     for (uint32_t i = lo; i < hi; i++) {
         const uint32_t d = bins - 1 - i;
         cursor[d] = run;
-        if (d == low) st->n_high = total - run >= min_low && !(run && st->down) ? run : total;
+        if (d == low) st->n_high = total - run >= min_low && !(run && (together || st->down)) ? run : total;
         run += hist[d];
     }
     if (threadIdx.x == 0) {
@@ -238,12 +239,10 @@ size_t count_ws_bytes(uint32_t n, uint32_t max_outdeg, int num_sms)
     return s.used;
 }
 
-// Roots of at most low_max out-neighbours from which on they get a launch of small blocks.
-static uint32_t min_low_roots(uint32_t k, const CountPlan &plan, int num_sms)
-{
-    if (k == 6 && plan.compact_max == 0) return 0xffffffffu;
-    return (uint32_t)num_sms * kLowSlotsPerSm * kLowPerSlot;
-}
+// Roots of at most kLowMax out-neighbours from which on they get a launch of small blocks.
+static uint32_t min_low_roots(int num_sms) { return (uint32_t)num_sms * kLowSlotsPerSm * kLowPerSlot; }
+// Whether the larger roots, if there are any, take them along (the end of the comment at kLowSlotsPerSm).
+static bool low_together(uint32_t k, const CountPlan &plan) { return k >= 7 || (k == 6 && plan.compact_max == 0); }
 
 // Runs the count for k >= 3.  Returns a CUDA error, or cudaErrorMemoryAllocation when the
 // workspace is too small.  The host value lands in *h_result.
@@ -272,7 +271,6 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
     uint32_t *list_scratch = (uint32_t *)(c.base + c.used);
     const size_t list_words = c.cap > c.used ? (c.cap - c.used) / sizeof(uint32_t) : 0;
     unsigned long long *work = result + 1;
-    if (!run.plan.small_max) run.plan.small_max = small_default(k);
     const CountPlan &plan = run.plan;
 
     cudaError_t e;
@@ -285,8 +283,8 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
         k_classify<<<blocks, 256, 0, s>>>(n, dag_off, k == 6 ? dag_cols : nullptr, need, plan.small_max, plan.bitmap_max,
                                           small_list, big_list, hist, st, run.sink.per_root,
                                           run.sink.per_arc, run.filter, 0xffffffffu, err);
-        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, low_max(k),
-                                        min_low_roots(k, plan, num_sms), cursor, st);
+        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, kLowMax, min_low_roots(num_sms),
+                                    low_together(k, plan), cursor, st);
         k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max,
                                              cursor, mid_list, run.filter);
         note_launches(3);
@@ -355,7 +353,6 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     uint32_t *list_scratch = (uint32_t *)(c.base + c.used);
     const size_t list_words = c.cap > c.used ? (c.cap - c.used) / sizeof(uint32_t) : 0;
     unsigned long long *work = result + 1;
-    if (!run.plan.small_max) run.plan.small_max = small_default(k);
     const CountPlan &plan = run.plan;
     cudaError_t e;
     if ((e = cudaMemsetAsync(st, 0, (char *)(hist + kBitmapCap + 2) - (char *)st, s))) return e;
@@ -375,11 +372,12 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     note_launches(1);
     // With no row above the line one launch is enough: of small blocks unless there are too few vertices.
     const uint32_t max_mid = max_outdeg < plan.bitmap_max ? max_outdeg : plan.bitmap_max;
-    uint32_t min_low = min_low_roots(k, plan, num_sms);
-    if (n < min_low || (k == 6 && run.keeps_ids && max_mid > low_max(k))) min_low = 0xffffffffu;
-    else if (max_mid <= low_max(k)) min_low = 0u;
+    uint32_t min_low = min_low_roots(num_sms);
+    const bool together = low_together(k, plan) || (k == 6 && run.keeps_ids);
+    if (n < min_low || (together && max_mid > kLowMax)) min_low = 0xffffffffu;
+    else if (max_mid <= kLowMax) min_low = 0u;
     if (max_outdeg > plan.small_max) {  // else no row is on the bitmap path
-        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, low_max(k), min_low, cursor, st);
+        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, kLowMax, min_low, together, cursor, st);
         k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max, cursor,
                                              mid_list, run.filter);
         note_launches(2);

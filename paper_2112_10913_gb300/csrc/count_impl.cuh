@@ -26,21 +26,20 @@ struct CountStats {
     uint32_t down;    // k = 6: some row reaches below its own id (a DAG that keeps vertex ids)
 };
 
-// Bitmap-path roots of at most low_max(k) out-neighbours run in a launch of their own, in blocks of 8
-// warps, several per SM: a block of 32 warps has a handful of rows per warp to build for them and
-// waits at its barriers instead.  R-MAT 15, k = 6: 0.70 ms in one launch, 0.64 in two (0.79 with 4
-// warps).  From k = 7 on a root's counting outweighs its build and two launches end in two tails
-// (R-MAT 15, k = 8: 69 ms in one launch, 129 in two at 128), so only the smallest roots, which the
-// warp-register path leaves to this one there, go in small blocks.
+// Bitmap-path roots of at most kLowMax out-neighbours run in a launch of their own, in blocks of 8 warps,
+// several per SM: a block of 32 warps has a handful of rows per warp to build for them and waits at
+// its barriers instead.  R-MAT 15, k = 6: 0.70 ms in one launch, 0.64 in two (0.79 with 4 warps).
+constexpr uint32_t kLowMax = 128;
 constexpr uint32_t kLowWarps = 8;
 // That launch needs kLowPerSlot such roots for every block of 8 warps that the chip holds: with fewer a
 // root is left to 8 warps while others idle, and what is a short launch of its own comes after the
 // tail of the other one.  40 roots of 99, k = 6,
 // ids kept: 2.4 ms in small blocks, 1.4 in large ones; R-MAT 15, k = 4: 0.22 ms against 0.31.
-// At k = 6 sets that are enumerated (a DAG that keeps ids, no re-encoding) outweigh their rows' build as
-// they do from k = 7 on, and the queue is not cut in two: R-MAT 15, ids kept, 13.9 ms in two launches,
-// 10.9 in one.  (Without roots above the line one launch of small blocks is still better: 200,000
-// vertices of degree 50, 1.8 ms against 3.5.)
+// Where the counting outweighs the rows' build, two launches end in two tails: from k = 7 on (R-MAT 15,
+// k = 8: 69 ms in one launch, 129 in two), and at k = 6 where sets are enumerated (a DAG that keeps ids, no
+// re-encoding; R-MAT 15, ids kept, 10.9 ms against 13.9).  There the small blocks are for graphs without
+// larger roots (200,000 vertices of degree 50, k = 6, ids kept: 1.8 ms against 3.5; k = 7: 1.7
+// against 3.3).
 constexpr uint32_t kLowSlotsPerSm = 4, kLowPerSlot = 4;
 // Under a cap on the blocks, that launch's blocks hold up to kMaxTeams teams of 8 warps, each with roots
 // of its own: as many blocks of 8 warps as the cap's warps are spread over all SMs, and no block of
@@ -49,7 +48,6 @@ constexpr uint32_t kLowSlotsPerSm = 4, kLowPerSlot = 4;
 // 0.25 to 1.6 ms beside teams.  (Blocks of 32 warps on one root each leave the SMs free too, but
 // k = 3 on R-MAT 18 takes 1.7 ms with them, 1.3 with teams.)
 constexpr int kMaxTeams = 4;
-__host__ __device__ constexpr uint32_t low_max(uint32_t k) { return k <= 6 ? 128 : 32; }
 
 // ------------------------------------------------------------------------------------------
 // Warp-register path (D <= 32).
@@ -116,144 +114,6 @@ struct Window {
         return first[p >> 5] + __popc(bits[p >> 5] & ((1u << (p & 31u)) - 1u));
     }
 };
-
-// One warp per root; the D (D - 1) / 2 pairs of its members are looked up (binary search of one
-// member in the other's list).  Scanning the members' whole lists instead costs their length:
-// R-MAT 20, roots of 9..32 out-neighbours: 3061 list entries per root on average, 116 pairs.
-template <int K>
-__global__ __launch_bounds__(kSmallWarps * 32) void k_count_small(
-    const uint64_t *__restrict__ dag_off, const uint32_t *__restrict__ dag_cols,
-    const uint32_t *__restrict__ list, const CountStats *st, unsigned long long *result,
-    RootSink sink, Budget budget, uint32_t *err)
-{
-    // per member: its id, its list and the list's first entry; its row as it fills
-    __shared__ uint64_t s_rb[kSmallWarps][32];
-    __shared__ uint32_t s_x[kSmallWarps][32], s_len[kSmallWarps][32], s_min[kSmallWarps][32], s_row[kSmallWarps][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t nlist = st->n_small;
-    const uint32_t gw = blockIdx.x * kSmallWarps + w, nwarps = gridDim.x * kSmallWarps;
-    unsigned long long total = 0;
-    for (uint32_t idx = gw; idx < nlist; idx += nwarps) {
-        int stop = 0;
-        if (lane == 0) stop = budget.over(err);
-        if (__shfl_sync(kFull, stop, 0)) break;
-        const uint32_t u = list[idx];
-        const uint64_t base = dag_off[u];
-        const uint32_t D = (uint32_t)(dag_off[u + 1] - base);
-        if (lane < D) {
-            const uint32_t x = dag_cols[base + lane];
-            const uint64_t rb = dag_off[x];
-            const uint32_t len = (uint32_t)(dag_off[x + 1] - rb);
-            s_x[w][lane] = x;
-            s_rb[w][lane] = rb;
-            s_len[w][lane] = len;
-            s_min[w][lane] = len ? dag_cols[rb] : 0xffffffffu;
-        }
-        s_row[w][lane] = 0;
-        __syncwarp();
-        // Where rows reach down to smaller ids (a DAG that keeps vertex ids) a pair takes two lookups:
-        // there, short lists (one load per lane) are scanned, every entry searched among the members.
-        // 20,000 vertices of degree 40, such a DAG, k = 3: 0.23 ms by pairs, 0.17 by lists; a relabelled
-        // DAG is better off with pairs (micro-batch of 64 graphs 3.01 ms by pairs, 3.07 by lists).
-        const bool down = lane < D && s_len[w][lane] && s_min[w][lane] < s_x[w][lane];
-        const bool lists = __any_sync(kFull, down) && __all_sync(kFull, lane >= D || s_len[w][lane] <= 32);
-        if (lists) {
-            for (uint32_t i = 0; i < D; i++) {
-                const uint32_t y = lane < s_len[w][i] ? dag_cols[s_rb[w][i] + lane] : 0xffffffffu;
-                const uint32_t j = lower_bound_smem(s_x[w], D, y);
-                const uint32_t bits = __reduce_or_sync(kFull, j < D && s_x[w][j] == y ? 1u << j : 0u);
-                if (lane == 0) s_row[w][i] = bits;
-            }
-        }
-        // Every pair of members once, two per lane and round: pair p is (c, c + r + 1 mod D) with
-        // r = p / D, c = p mod D.  An arc between them is in the row of one of the two: the one
-        // of lower index if rows only hold larger ids (a relabelled DAG), else either.
-        const uint32_t npairs = lists ? 0u : D * (D - 1) / 2;
-        const float inv = 1.0f / (float)D;
-        for (uint32_t p0 = 0; p0 < npairs; p0 += 64) {
-            uint32_t src[2], dst[2], lo[2], left[2];
-            const uint32_t *row[2];
-            uint32_t want[2];
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const uint32_t p = p0 + 32 * h + lane;
-                const uint32_t r = (uint32_t)(((float)p + 0.5f) * inv), c = p - r * D;
-                const uint32_t o = c + r + 1 >= D ? c + r + 1 - D : c + r + 1;
-                const bool in = p < npairs;
-                src[h] = in ? min(c, o) : 0u;
-                dst[h] = in ? max(c, o) : 0u;
-                lo[h] = 0;
-                left[h] = in ? s_len[w][src[h]] : 0u;
-                row[h] = dag_cols + s_rb[w][src[h]];
-                want[h] = s_x[w][dst[h]];
-            }
-            for (;;) {
-                // both searches step together, so that two loads are in flight
-                while (left[0] | left[1]) {
-                    uint32_t y[2];
-#pragma unroll
-                    for (int h = 0; h < 2; h++) y[h] = left[h] ? row[h][lo[h] + (left[h] >> 1)] : 0u;
-#pragma unroll
-                    for (int h = 0; h < 2; h++) {
-                        const uint32_t half = left[h] >> 1;
-                        if (left[h] && y[h] == want[h]) {
-                            atomicOr(&s_row[w][src[h]], 1u << dst[h]);
-                            left[h] = 0;
-                            dst[h] = src[h];  // found
-                        } else if (y[h] < want[h]) {
-                            lo[h] += left[h] ? half + 1 : 0u;
-                            left[h] -= left[h] ? half + 1 : 0u;
-                        } else {
-                            left[h] = half;
-                        }
-                    }
-                }
-                // the other direction, where the row's ids reach down to it
-                bool more = false;
-#pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    if (dst[h] > src[h] && s_min[w][dst[h]] <= s_x[w][src[h]]) {
-                        const uint32_t t = src[h];
-                        src[h] = dst[h];
-                        dst[h] = t;
-                        lo[h] = 0;
-                        left[h] = s_len[w][src[h]];
-                        row[h] = dag_cols + s_rb[w][src[h]];
-                        want[h] = s_x[w][t];
-                        more = true;
-                    }
-                }
-                if (!more) break;
-            }
-        }
-        __syncwarp();
-        const uint32_t myrow = s_row[w][lane];
-        unsigned long long acc = 0;
-        const uint32_t all = D == 32 ? kFull : ((1u << D) - 1);
-        if (sink.per_arc) {
-            // debug output: the root's edge tasks one at a time, each (K-2)-clique count of
-            // N+(u) ∩ N+(a) stored for its arc
-            for (uint32_t a = 0; a < D; a++) {
-                const uint32_t c2 = all & __shfl_sync(kFull, myrow, a);
-                unsigned long long t = 0;
-                if (__popc(c2) >= K - 2) small_dfs<K - 2>(c2, myrow, lane, t);
-                const unsigned long long tt = warp_sum_u64(t, err);
-                if (lane == 0) sink.per_arc[base + a] = tt;
-                acc += t;
-            }
-        } else {
-            small_dfs<K - 1>(all, myrow, lane, acc);
-        }
-        if (sink.wants_root_total()) {
-            const unsigned long long r = warp_sum_u64(acc, err);
-            if (lane == 0) sink.put(u, r, err);
-        }
-        total += acc;
-        __syncwarp();
-    }
-    total = warp_sum_u64(total, err);
-    if (lane == 0) add_checked(result, total, err);
-}
 
 // ------------------------------------------------------------------------------------------
 // Shared-memory bitmap path (small_max < D <= 1024).
@@ -1940,6 +1800,188 @@ __global__ __launch_bounds__(kMidMaxWarps * 32, 1) void k_count_mid(
 }
 
 // ------------------------------------------------------------------------------------------
+// Warp-register path: the kernel (its recursion, small_dfs, is above).
+
+template <int K>
+constexpr bool kSmallDense = K >= 7;  // below, enumerating at most 32 members is short
+constexpr uint32_t kSmallScratch = 32 + kMaskWords + kNbhdList + kNbhdWords;  // cbuf, then comp4's
+
+// Counts a root of D > 16 members on its complement if its rows (lane i: row i) are upper-triangular and
+// dense; else returns false.
+template <int K>
+__device__ __forceinline__ bool small_dense(uint32_t myrow, uint32_t D, int lane, bool compact, uint32_t *comp,
+                                            uint32_t *scr, uint32_t *err, unsigned long long &acc)
+{
+    if constexpr (kSmallDense<K>) {
+        if (!compact || D <= 16 || __any_sync(kFull, myrow & ~above_bit(lane))) return false;
+        const uint32_t pairs = D * (D - 1) / 2, missing = pairs - __reduce_add_sync(kFull, __popc(myrow));
+        if (!is_dense<K - 1>(D, missing, pairs)) return false;
+        if (missing == 0) {
+            if (lane == 0) add_acc(acc, choose<K - 1>(D), err);
+            return true;
+        }
+        put_block(comp, 0, D, 0, 0, myrow, lane);
+        __syncwarp();
+        WarpCtx x = {};
+        x.cbuf = scr;
+        x.mv = scr + 32;
+        x.err = err;
+        const CompSet cs = {comp, 0, 1};
+        unsigned long long work = 0;
+        dense_dfs<K - 1, 1, false>(x, cs, word_mask(D, lane), D, lane, acc, work);
+        __syncwarp();
+        return true;
+    } else {
+        return false;
+    }
+}
+
+// One warp per root; the D (D - 1) / 2 pairs of its members are looked up (binary search of one
+// member in the other's list).  Scanning the members' whole lists instead costs their length:
+// R-MAT 20, roots of 9..32 out-neighbours: 3061 list entries per root on average, 116 pairs.
+// From k = 7 on a root whose subgraph is dense, in a DAG relabelled to its order, is counted on the
+// complement (one word per row) like the bitmap path's sets; the others are enumerated.  Leaving all
+// roots of more than 16 to blocks instead: 20,000 vertices of degree 40, k = 7 0.15 -> 0.23 ms; enumerating
+// all of them: R-MAT 15, k = 8 13 ms in this kernel.
+template <int K>
+__global__ __launch_bounds__(kSmallWarps * 32) void k_count_small(
+    const uint64_t *__restrict__ dag_off, const uint32_t *__restrict__ dag_cols,
+    const uint32_t *__restrict__ list, const CountStats *st, unsigned long long *result,
+    RootSink sink, bool compact, Budget budget, uint32_t *err)
+{
+    // per member: its id, its list and the list's first entry; its row as it fills
+    __shared__ uint64_t s_rb[kSmallWarps][32];
+    __shared__ uint32_t s_x[kSmallWarps][32], s_len[kSmallWarps][32], s_min[kSmallWarps][32], s_row[kSmallWarps][32];
+    // the complement's rows (16 bytes each) and the lists of its walk
+    __shared__ __align__(16) uint32_t s_comp[kSmallDense<K> ? kSmallWarps : 1][kSmallDense<K> ? 128 : 4];
+    __shared__ __align__(16) uint32_t s_scr[kSmallDense<K> ? kSmallWarps : 1][kSmallDense<K> ? kSmallScratch : 4];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t nlist = st->n_small;
+    const uint32_t gw = blockIdx.x * kSmallWarps + w, nwarps = gridDim.x * kSmallWarps;
+    unsigned long long total = 0;
+    for (uint32_t idx = gw; idx < nlist; idx += nwarps) {
+        int stop = 0;
+        if (lane == 0) stop = budget.over(err);
+        if (__shfl_sync(kFull, stop, 0)) break;
+        const uint32_t u = list[idx];
+        const uint64_t base = dag_off[u];
+        const uint32_t D = (uint32_t)(dag_off[u + 1] - base);
+        if (lane < D) {
+            const uint32_t x = dag_cols[base + lane];
+            const uint64_t rb = dag_off[x];
+            const uint32_t len = (uint32_t)(dag_off[x + 1] - rb);
+            s_x[w][lane] = x;
+            s_rb[w][lane] = rb;
+            s_len[w][lane] = len;
+            s_min[w][lane] = len ? dag_cols[rb] : 0xffffffffu;
+        }
+        s_row[w][lane] = 0;
+        __syncwarp();
+        // Where rows reach down to smaller ids (a DAG that keeps vertex ids) a pair takes two lookups:
+        // there, short lists (one load per lane) are scanned, every entry searched among the members.
+        // 20,000 vertices of degree 40, such a DAG, k = 3: 0.23 ms by pairs, 0.17 by lists; a relabelled
+        // DAG is better off with pairs (micro-batch of 64 graphs 3.01 ms by pairs, 3.07 by lists).
+        const bool down = lane < D && s_len[w][lane] && s_min[w][lane] < s_x[w][lane];
+        const bool lists = __any_sync(kFull, down) && __all_sync(kFull, lane >= D || s_len[w][lane] <= 32);
+        if (lists) {
+            for (uint32_t i = 0; i < D; i++) {
+                const uint32_t y = lane < s_len[w][i] ? dag_cols[s_rb[w][i] + lane] : 0xffffffffu;
+                const uint32_t j = lower_bound_smem(s_x[w], D, y);
+                const uint32_t bits = __reduce_or_sync(kFull, j < D && s_x[w][j] == y ? 1u << j : 0u);
+                if (lane == 0) s_row[w][i] = bits;
+            }
+        }
+        // Every pair of members once, two per lane and round: pair p is (c, c + r + 1 mod D) with
+        // r = p / D, c = p mod D.  An arc between them is in the row of one of the two: the one
+        // of lower index if rows only hold larger ids (a relabelled DAG), else either.
+        const uint32_t npairs = lists ? 0u : D * (D - 1) / 2;
+        const float inv = 1.0f / (float)D;
+        for (uint32_t p0 = 0; p0 < npairs; p0 += 64) {
+            uint32_t src[2], dst[2], lo[2], left[2];
+            const uint32_t *row[2];
+            uint32_t want[2];
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const uint32_t p = p0 + 32 * h + lane;
+                const uint32_t r = (uint32_t)(((float)p + 0.5f) * inv), c = p - r * D;
+                const uint32_t o = c + r + 1 >= D ? c + r + 1 - D : c + r + 1;
+                const bool in = p < npairs;
+                src[h] = in ? min(c, o) : 0u;
+                dst[h] = in ? max(c, o) : 0u;
+                lo[h] = 0;
+                left[h] = in ? s_len[w][src[h]] : 0u;
+                row[h] = dag_cols + s_rb[w][src[h]];
+                want[h] = s_x[w][dst[h]];
+            }
+            for (;;) {
+                // both searches step together, so that two loads are in flight
+                while (left[0] | left[1]) {
+                    uint32_t y[2];
+#pragma unroll
+                    for (int h = 0; h < 2; h++) y[h] = left[h] ? row[h][lo[h] + (left[h] >> 1)] : 0u;
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const uint32_t half = left[h] >> 1;
+                        if (left[h] && y[h] == want[h]) {
+                            atomicOr(&s_row[w][src[h]], 1u << dst[h]);
+                            left[h] = 0;
+                            dst[h] = src[h];  // found
+                        } else if (y[h] < want[h]) {
+                            lo[h] += left[h] ? half + 1 : 0u;
+                            left[h] -= left[h] ? half + 1 : 0u;
+                        } else {
+                            left[h] = half;
+                        }
+                    }
+                }
+                // the other direction, where the row's ids reach down to it
+                bool more = false;
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    if (dst[h] > src[h] && s_min[w][dst[h]] <= s_x[w][src[h]]) {
+                        const uint32_t t = src[h];
+                        src[h] = dst[h];
+                        dst[h] = t;
+                        lo[h] = 0;
+                        left[h] = s_len[w][src[h]];
+                        row[h] = dag_cols + s_rb[w][src[h]];
+                        want[h] = s_x[w][t];
+                        more = true;
+                    }
+                }
+                if (!more) break;
+            }
+        }
+        __syncwarp();
+        const uint32_t myrow = s_row[w][lane];
+        unsigned long long acc = 0;
+        const uint32_t all = D == 32 ? kFull : ((1u << D) - 1);
+        if (sink.per_arc) {
+            // debug output: the root's edge tasks one at a time, each (K-2)-clique count of
+            // N+(u) ∩ N+(a) stored for its arc
+            for (uint32_t a = 0; a < D; a++) {
+                const uint32_t c2 = all & __shfl_sync(kFull, myrow, a);
+                unsigned long long t = 0;
+                if (__popc(c2) >= K - 2) small_dfs<K - 2>(c2, myrow, lane, t);
+                const unsigned long long tt = warp_sum_u64(t, err);
+                if (lane == 0) sink.per_arc[base + a] = tt;
+                acc += t;
+            }
+        } else if (!small_dense<K>(myrow, D, lane, compact, s_comp[kSmallDense<K> ? w : 0], s_scr[kSmallDense<K> ? w : 0], err, acc)) {
+            small_dfs<K - 1>(all, myrow, lane, acc);
+        }
+        if (sink.wants_root_total()) {
+            const unsigned long long r = warp_sum_u64(acc, err);
+            if (lane == 0) sink.put(u, r, err);
+        }
+        total += acc;
+        __syncwarp();
+    }
+    total = warp_sum_u64(total, err);
+    if (lane == 0) add_checked(result, total, err);
+}
+
+// ------------------------------------------------------------------------------------------
 // Sorted-list path (D > bitmap_max).
 
 // R-cliques inside the sorted candidate list C[0..len); buf holds one list per deeper level.
@@ -2162,7 +2204,7 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
         for (int low = 0; low < 2; low++) {
             const uint32_t n_roots = low ? hs.n_low : hs.n_high;
             if (!n_roots) continue;
-            const uint32_t dmax = low && hs.max_mid > low_max(K) ? low_max(K) : hs.max_mid;
+            const uint32_t dmax = low && hs.max_mid > kLowMax ? kLowMax : hs.max_mid;
             const uint32_t dcap = (dmax + 31) & ~31u, rs = (dcap / 32) | 1;
             uint32_t warps = plan.warps_per_cta > (uint32_t)kMidMaxWarps ? kMidMaxWarps : plan.warps_per_cta;
             if (low && warps > kLowWarps) warps = kLowWarps;
@@ -2238,8 +2280,8 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
         if (plan.max_blocks && cap > plan.max_blocks * 4) cap = plan.max_blocks * 4;
         if (grid > cap) grid = cap;
         Timer t(run.time_kernels, s);
-        k_count_small<K><<<grid, kSmallWarps * 32, 0, s>>>(dag_off, dag_cols, small_list, st, result,
-                                                           run.sink, aux.budget, err);
+        k_count_small<K><<<grid, kSmallWarps * 32, 0, s>>>(dag_off, dag_cols, small_list, st, result, run.sink,
+                                                           plan.compact_max != 0, aux.budget, err);
         note_launches(1);
         if ((e = cudaGetLastError())) return e;
         t.stop();
