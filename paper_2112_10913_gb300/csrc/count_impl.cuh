@@ -1877,17 +1877,28 @@ __global__ __launch_bounds__(kSmallWarps * 32) void k_count_small(
         }
         s_row[w][lane] = 0;
         __syncwarp();
-        // Where rows reach down to smaller ids (a DAG that keeps vertex ids) a pair takes two lookups:
-        // there, short lists (one load per lane) are scanned, every entry searched among the members.
-        // 20,000 vertices of degree 40, such a DAG, k = 3: 0.23 ms by pairs, 0.17 by lists; a relabelled
-        // DAG is better off with pairs (micro-batch of 64 graphs 3.01 ms by pairs, 3.07 by lists).
-        const bool down = lane < D && s_len[w][lane] && s_min[w][lane] < s_x[w][lane];
-        const bool lists = __any_sync(kFull, down) && __all_sync(kFull, lane >= D || s_len[w][lane] <= 32);
+        // The members' lists are scanned instead where that is less: a step of 32 entries (one load and a
+        // search among the members in shared memory) costs about two levels of 64 pairs' searches, of
+        // which a pair takes twice as many where rows reach down to smaller ids (a DAG that keeps
+        // vertex ids).  20,000 vertices of degree 40, ids kept, k = 3: 158 us by pairs, 149 so; Chung-Lu
+        // of 20,000, ids kept, k = 4: 150 and 123.  With the line twice and four times as high
+        // 1,000,000 vertices of degree 10 take 0.64 and 0.70 ms instead of 0.57.
+        const uint32_t len = lane < D ? s_len[w][lane] : 0u;
+        const bool down = __any_sync(kFull, len && s_min[w][lane] < s_x[w][lane]);
+        const uint32_t steps = __reduce_add_sync(kFull, (len + 31) >> 5), levels = 32 - __clz(__reduce_max_sync(kFull, len));
+        const bool lists = 2 * steps <= ((D * (D - 1) / 2 + 63) / 64) * levels * (down ? 2 : 1);
         if (lists) {
+            const uint32_t most = s_x[w][D - 1];
             for (uint32_t i = 0; i < D; i++) {
-                const uint32_t y = lane < s_len[w][i] ? dag_cols[s_rb[w][i] + lane] : 0xffffffffu;
-                const uint32_t j = lower_bound_smem(s_x[w], D, y);
-                const uint32_t bits = __reduce_or_sync(kFull, j < D && s_x[w][j] == y ? 1u << j : 0u);
+                const uint32_t n = s_len[w][i];
+                uint32_t bits = 0;
+                for (uint32_t q = 0; q < n; q += 32) {
+                    const uint32_t y = q + lane < n ? dag_cols[s_rb[w][i] + q + lane] : 0xffffffffu;
+                    if (__shfl_sync(kFull, y, 0) > most) break;
+                    const uint32_t j = lower_bound_smem(s_x[w], D, y);
+                    if (j < D && s_x[w][j] == y) bits |= 1u << j;
+                }
+                bits = __reduce_or_sync(kFull, bits);
                 if (lane == 0) s_row[w][i] = bits;
             }
         }
