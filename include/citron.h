@@ -209,9 +209,9 @@ typedef struct {
                                 Sec. VII-C): their edge tasks are taken from global cursors, which
                                 blocks that find the root queue empty join after rebuilding the
                                 root's subgraph.  0: default (384); 1: never; else the threshold */
-    float busy_ms[2];        /* out (CITRON_COUNT_BALANCE): bitmap kernel's span from the first
-                                block start to the last block end, and its tail from the first
-                                block end to the last */
+    float busy_ms[2];        /* out (CITRON_COUNT_BALANCE): the bitmap path's span from the first
+                                block start to the last block end, over its one or two launches,
+                                and the sum of their tails from the first block end to the last */
     uint32_t budget_ms;      /* in: device time the count may take (0: no limit); when it runs
                                 out, the blocks stop taking work and the call returns
                                 CITRON_E_BUDGET */

@@ -302,8 +302,8 @@ struct CountRun {
     unsigned long long work = 0;             // out: word operations (AND + POPC of 32-bit words)
     uint32_t dev_error = 0;                  // out: the device error word after the count
     float kernel_ms[3] = {0, 0, 0};          // out: warp-register, bitmap, sorted-list kernels
-    float busy_ms[2] = {0, 0};               // out: bitmap kernel's span (first start to last end)
-                                             // and tail (first block end to last block end)
+    float busy_ms[2] = {0, 0};               // out: the bitmap launches' span (first start to last end)
+                                             // and tails (first block end to last block end)
 };
 
 // Number of kernels this library has launched (all devices, all threads).

@@ -231,7 +231,7 @@ size_t count_ws_bytes(uint32_t n, uint32_t max_outdeg, int num_sms)
     s.take<uint32_t>(kBitmapCap + 2);         // mid histogram
     s.take<uint32_t>(kBitmapCap + 2);         // mid cursors
     s.take<HeavySlot>(kHelpSlots);            // help table of heavy roots
-    s.take<unsigned long long>(2 * (size_t)num_sms * kMidBlocksPerSmCap);  // block start/end
+    s.take<unsigned long long>(kMidLaunches * 2 * (size_t)num_sms * kMidBlocksPerSmCap);  // block start/end
     // sorted-list scratch: one (k-3)-level stack per warp, sized for the largest root, so that
     // every root can take the list path (tuned thresholds send any root there)
     const uint32_t list_warps = (uint32_t)num_sms * kListWarps;
@@ -263,7 +263,7 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
     aux.help.slots = c.take<HeavySlot>(kHelpSlots);
     aux.help.cap = kHelpSlots;
     aux.help.nslots = next + 2;
-    aux.block_ns = c.take<unsigned long long>(2 * (size_t)num_sms * kMidBlocksPerSmCap);
+    aux.block_ns = c.take<unsigned long long>(kMidLaunches * 2 * (size_t)num_sms * kMidBlocksPerSmCap);
     aux.budget.clock0 = result + 2;
     aux.budget.ns = run.budget_ns;
     if (!c.ok) return cudaErrorMemoryAllocation;
@@ -346,7 +346,7 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     aux.help.slots = c.take<HeavySlot>(kHelpSlots);
     aux.help.cap = kHelpSlots;
     aux.help.nslots = next + 2;
-    aux.block_ns = c.take<unsigned long long>(2 * (size_t)num_sms * kMidBlocksPerSmCap);
+    aux.block_ns = c.take<unsigned long long>(kMidLaunches * 2 * (size_t)num_sms * kMidBlocksPerSmCap);
     aux.budget.clock0 = result + 2;
     aux.budget.ns = run.budget_ns;
     if (!c.ok) return cudaErrorMemoryAllocation;

@@ -2116,8 +2116,9 @@ namespace citron_host {
 using namespace citron;
 
 // Global-memory helpers of the bitmap kernel: the help table of heavy roots and the per-block
-// start/end times (2 words per block, kMidBlocksPerSmCap blocks per SM at most).
+// start/end times (2 words per block, kMidBlocksPerSmCap blocks per SM and launch at most).
 constexpr uint32_t kMidBlocksPerSmCap = 8;
+constexpr uint32_t kMidLaunches = 2;
 struct MidAux {
     HelpTable help;
     unsigned long long *block_ns = nullptr;
@@ -2209,9 +2210,9 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
         const uint32_t compact_max = K >= 5 ? plan.compact_max : 0u;
         Timer t(run.time_kernels, s);
         unsigned long long *block_ns = run.balance ? aux.block_ns : nullptr;
-        if (block_ns && (e = cudaMemsetAsync(block_ns, 0, 2 * sizeof(*block_ns) * kMidBlocksPerSmCap * num_sms, s)))
-            return e;
-        uint32_t grid = 0;
+        const size_t ns_words = 2 * (size_t)num_sms * kMidBlocksPerSmCap;  // of one launch
+        if (block_ns && (e = cudaMemsetAsync(block_ns, 0, kMidLaunches * ns_words * sizeof(*block_ns), s))) return e;
+        uint32_t grid[kMidLaunches] = {0, 0};
         for (int low = 0; low < 2; low++) {
             const uint32_t n_roots = low ? hs.n_low : hs.n_high;
             if (!n_roots) continue;
@@ -2235,8 +2236,7 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
             // the window's bitmap and first places (k > 3) have to fit the scratch
             uint32_t window = kMidWindow;
             while ((size_t)window / 32 + (K > 3 ? window / 64 : 0) > scratch(warps)) window /= 2;
-            unsigned long long *ns = grid ? nullptr : block_ns;  // timed: the first launch's blocks
-            uint32_t this_grid = 0;
+            unsigned long long *ns = block_ns ? block_ns + low * ns_words : nullptr;
             uint32_t *queue = next + (low ? 3 : 0);
             // under a cap: teams of kLowWarps in blocks as wide as the other launch's
             uint32_t teams = 1;
@@ -2249,7 +2249,7 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
                 return launch_mid<K, v == 1, v == 2>((n_roots + teams - 1) / teams, plan.max_blocks, low, teams, dcap,
                                                      buf_words, window, compact_max, plan.split_min, aux.help, warps,
                                                      smem_for(warps), dag_off, dag_cols, mid_list, st, queue, result,
-                                                     run.sink, work, ns, aux.budget, &this_grid, err, s, num_sms);
+                                                     run.sink, work, ns, aux.budget, &grid[low], err, s, num_sms);
             };
             // the instrumented kernel also serves the per-arc debug output (its code is compiled
             // out of the plain kernel)
@@ -2262,26 +2262,32 @@ static cudaError_t launch_count_k(CountRun &run, const uint64_t *dag_off, const 
                 e = launch(std::integral_constant<int, 0>());
             }
             if (e) return e;
-            if (!grid) grid = this_grid;
         }
         t.stop();
         run.kernel_ms[1] = t.ms();
-        if (block_ns && grid) {
-            // span = first block start .. last block end; tail = first block end .. last block end
-            unsigned long long h[2 * kMidBlocksPerSmCap * 256];
-            const size_t cnt = 2 * (size_t)grid;
-            if (cnt <= sizeof(h) / sizeof(h[0])) {
-                e = cudaMemcpyAsync(h, block_ns, cnt * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
+        if (block_ns) {
+            // span = first block start .. last block end, over both launches; tail = first block end ..
+            // last block end, of each launch
+            unsigned long long s0 = ~0ull, last = 0, tails = 0;
+            for (uint32_t l = 0; l < kMidLaunches; l++) {
+                unsigned long long h[2 * kMidBlocksPerSmCap * 256];
+                const size_t cnt = 2 * (size_t)grid[l];
+                if (!cnt || cnt > sizeof(h) / sizeof(h[0])) continue;
+                e = cudaMemcpyAsync(h, block_ns + l * ns_words, cnt * sizeof(h[0]), cudaMemcpyDeviceToHost, s);
                 if (!e) e = cudaStreamSynchronize(s);
                 if (e) return e;
-                unsigned long long s0 = ~0ull, e0 = ~0ull, e1 = 0;
-                for (uint32_t b = 0; b < grid; b++) {
+                unsigned long long e0 = ~0ull, e1 = 0;
+                for (uint32_t b = 0; b < grid[l]; b++) {
                     s0 = h[2 * b] < s0 ? h[2 * b] : s0;
                     e0 = h[2 * b + 1] < e0 ? h[2 * b + 1] : e0;
                     e1 = h[2 * b + 1] > e1 ? h[2 * b + 1] : e1;
                 }
-                run.busy_ms[0] = (float)((e1 - s0) * 1e-6);
-                run.busy_ms[1] = (float)((e1 - e0) * 1e-6);
+                last = e1 > last ? e1 : last;
+                tails += e1 - e0;
+            }
+            if (last) {
+                run.busy_ms[0] = (float)((last - s0) * 1e-6);
+                run.busy_ms[1] = (float)(tails * 1e-6);
             }
         }
     }

@@ -9,18 +9,18 @@ from paper_2112_10913_gb300 import graphgen as gg
 pytestmark = pytest.mark.gpu
 
 
-def _copies(size, copies, p, seed):
-    """`copies` disjoint random graphs of `size` vertices and one wider one beside them."""
+def _copies(size, copies, p, seed, wide=170, q=0.5):
+    """`copies` disjoint random graphs of `size` vertices and one of `wide` beside them."""
     rng = np.random.default_rng(seed)
     i, j = np.triu_indices(size, 1)
     shift = np.arange(copies)[:, None] * size
     keep = rng.random((copies, i.size)) < p
     base = size * copies
-    bi, bj = np.triu_indices(170, 1)
-    big = rng.random(bi.size) < 0.5
+    bi, bj = np.triu_indices(wide, 1)
+    big = rng.random(bi.size) < q
     src = np.concatenate([(i + shift)[keep], bi[big] + base])
     dst = np.concatenate([(j + shift)[keep], bj[big] + base])
-    return gg.csr_from_edges(base + 170, src, dst)
+    return gg.csr_from_edges(base + wide, src, dst)
 
 
 # about 35 roots a copy on the bitmap path: 70, 2,450 (around four per 8-warp block of 152 SMs) and 6,000
@@ -45,3 +45,14 @@ def test_one_launch_or_two(gpu, oracle_lib, copies, k, relabel):
                                G.ws, None, opts)
         gpu.citron_workspace_status(G.ws)
         assert int(counts.item()) == want
+
+
+def test_busy_time_covers_both_launches(gpu):
+    """busy_ms spans the launch of large blocks (few roots here) and the one of small blocks (12,000 roots)."""
+    g = _copies(72, 340, 0.93, 5, wide=260, q=0.7)
+    G = gpu.DeviceGraph(g)
+    for _ in range(2):  # (the first call pays for loading the kernels)
+        _, o = gpu.citron_count_ex(G.n, G.dag_off, G.dag_cols, 5, G.ws, G.max_outdeg, time_kernels=True, balance=True)
+    assert G.max_outdeg > 128 and o.kernel_ms[1] > 0.1
+    assert 0.7 * o.kernel_ms[1] < o.busy_ms[0] <= 1.05 * o.kernel_ms[1] + 0.02
+    assert 0 <= o.busy_ms[1] <= o.busy_ms[0]
