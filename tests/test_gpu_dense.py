@@ -97,3 +97,42 @@ def test_sets_around_the_line(gpu, oracle_lib, s, p, k):
     if k <= 6:
         total, per_arc = G.count_per_arc(k)
         assert total == want and int(per_arc.sum()) == want
+
+
+def test_nested_wide_set_beyond_the_planes(gpu):
+    """k = 7: subsets of a wide set with more than 128 members of complement degree above 128 (an
+    independent part of 135 at the end of the order), counted one level further down."""
+    from math import comb
+
+    import paper_2112_10913_gb300 as cg
+
+    clique, part = 137, 135
+    i, j = np.triu_indices(clique, 1)
+    src = np.concatenate([i, np.repeat(np.arange(clique), part)])
+    dst = np.concatenate([j, np.tile(np.arange(part) + clique, clique)])
+    g = gg.csr_from_edges(clique + part, src, dst)
+    G = cg.DeviceGraph(g, rank=np.arange(g.n, dtype=np.uint32))
+    want = comb(clique, 7) + part * comb(clique, 6)
+    assert G.count(7) == want
+    assert G.count(7, split_min=129) == want
+
+
+@pytest.mark.parametrize("parts,size,k", [(10, 7, 10), (11, 6, 11), (12, 6, 12)])
+def test_deep_walks_pack_their_subsets(gpu, parts, size, k):
+    """Two vertices joined to a complete multipartite graph of 66 to 72: sets of four words whose subsets
+    are packed to two and to one on the way down."""
+    from math import comb
+
+    import paper_2112_10913_gb300 as cg
+
+    n = parts * size
+    i, j = np.triu_indices(n, 1)
+    keep = i // size != j // size
+    src = np.concatenate([[0], np.zeros(n, int), np.ones(n, int), i[keep] + 2])
+    dst = np.concatenate([[1], np.arange(n) + 2, np.arange(n) + 2, j[keep] + 2])
+    g = gg.csr_from_edges(n + 2, src, dst)
+    G = cg.DeviceGraph(g, rank=np.arange(g.n, dtype=np.uint32))
+    e = [comb(parts, m) * size ** m for m in range(k + 1)]
+    want = e[k] + 2 * e[k - 1] + e[k - 2]
+    assert G.count(k) == want
+    assert G.count(k, small_max=1) == want
