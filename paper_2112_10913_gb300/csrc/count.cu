@@ -91,10 +91,11 @@ __global__ void k_classify(uint32_t n, const uint64_t *__restrict__ dag_off,
 
 // Bin starts for the mid roots in DESCENDING out-degree: cursor[d] = #roots with degree > d.  The roots
 // of at most `low` out-neighbours, the end of the queue, are left to the launch of small blocks if there
-// are at least min_low of them, and, with `together` or in a DAG found to keep vertex ids, only without
-// roots above.
+// are at least min_low of them (kLowIds times as many in a DAG found to keep vertex ids), and, with
+// `together`, only without roots above (at k = 6 in a DAG that keeps ids, too).
 __global__ __launch_bounds__(1024) void k_mid_bins(const uint32_t *hist, uint32_t bins, uint32_t low,
-                                                    uint32_t min_low, bool together, uint32_t *cursor, CountStats *st)
+                                                    uint32_t min_low, bool together, bool together_ids, uint32_t *cursor,
+                                                    CountStats *st)
 {
     __shared__ uint32_t scratch[33];
     // reversed index: position i holds degree bins-1-i
@@ -104,10 +105,14 @@ __global__ __launch_bounds__(1024) void k_mid_bins(const uint32_t *hist, uint32_
     for (uint32_t i = lo; i < hi; i++) s += hist[bins - 1 - i];
     uint32_t total;
     uint32_t run = block_excl_scan(s, scratch, total);
+    if (st->down) {
+        min_low *= kLowIds;
+        together |= together_ids;
+    }
     for (uint32_t i = lo; i < hi; i++) {
         const uint32_t d = bins - 1 - i;
         cursor[d] = run;
-        if (d == low) st->n_high = total - run >= min_low && !(run && (together || st->down)) ? run : total;
+        if (d == low) st->n_high = total - run >= min_low && !(run && together) ? run : total;
         run += hist[d];
     }
     if (threadIdx.x == 0) {
@@ -240,7 +245,7 @@ size_t count_ws_bytes(uint32_t n, uint32_t max_outdeg, int num_sms)
 }
 
 // Roots of at most kLowMax out-neighbours from which on they get a launch of small blocks.
-static uint32_t min_low_roots(int num_sms) { return (uint32_t)num_sms * kLowSlotsPerSm * kLowPerSlot; }
+static uint32_t min_low_roots(uint32_t k, int num_sms) { return k <= 4 ? 0u : (uint32_t)num_sms * kLowSlotsPerSm; }
 // Whether the larger roots, if there are any, take them along (the end of the comment at kLowSlotsPerSm).
 static bool low_together(uint32_t k, const CountPlan &plan) { return k >= 7 || (k == 6 && plan.compact_max == 0); }
 
@@ -280,11 +285,11 @@ cudaError_t run_count(uint32_t n, const uint64_t *dag_off, const uint32_t *dag_c
     const uint32_t need = k - 1;
     const uint32_t blocks = (n + 255) / 256;
     if (n) {
-        k_classify<<<blocks, 256, 0, s>>>(n, dag_off, k == 6 ? dag_cols : nullptr, need, plan.small_max, plan.bitmap_max,
+        k_classify<<<blocks, 256, 0, s>>>(n, dag_off, k >= 5 ? dag_cols : nullptr, need, plan.small_max, plan.bitmap_max,
                                           small_list, big_list, hist, st, run.sink.per_root,
                                           run.sink.per_arc, run.filter, 0xffffffffu, err);
-        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, kLowMax, min_low_roots(num_sms),
-                                    low_together(k, plan), cursor, st);
+        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, kLowMax, min_low_roots(k, num_sms),
+                                    low_together(k, plan), k == 6, cursor, st);
         k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max,
                                              cursor, mid_list, run.filter);
         note_launches(3);
@@ -372,12 +377,12 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     note_launches(1);
     // With no row above the line one launch is enough: of small blocks unless there are too few vertices.
     const uint32_t max_mid = max_outdeg < plan.bitmap_max ? max_outdeg : plan.bitmap_max;
-    uint32_t min_low = min_low_roots(num_sms);
+    uint32_t min_low = min_low_roots(k, num_sms) * (run.keeps_ids ? kLowIds : 1u);
     const bool together = low_together(k, plan) || (k == 6 && run.keeps_ids);
     if (n < min_low || (together && max_mid > kLowMax)) min_low = 0xffffffffu;
     else if (max_mid <= kLowMax) min_low = 0u;
     if (max_outdeg > plan.small_max) {  // else no row is on the bitmap path
-        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, kLowMax, min_low, together, cursor, st);
+        k_mid_bins<<<1, 1024, 0, s>>>(hist, plan.bitmap_max + 1, kLowMax, min_low, together, false, cursor, st);
         k_mid_scatter<<<blocks, 256, 0, s>>>(n, dag_off, need, plan.small_max, plan.bitmap_max, cursor,
                                              mid_list, run.filter);
         note_launches(2);
@@ -387,7 +392,7 @@ cudaError_t run_count_async(uint32_t n, const uint64_t *dag_off, const uint32_t 
     hs.max_mid = max_mid;
     hs.n_mid = hs.max_mid > plan.small_max ? n : 0;
     // upper bounds of both parts of the queue: the kernels read the real ones on the device
-    hs.n_high = min_low ? n : 0;
+    hs.n_high = min_low || max_mid > kLowMax ? n : 0;
     hs.n_low = min_low == 0xffffffffu ? 0 : n;
     hs.max_big = max_outdeg;
     hs.n_big = max_outdeg > plan.bitmap_max ? n : 0;

@@ -23,7 +23,7 @@ struct CountStats {
     uint32_t max_mid, max_big, max_all;
     uint32_t n_high;  // bitmap-path roots of the launch of large blocks, the first n_high of the queue
     uint32_t n_low;   // host copy only: the others, or an upper bound of them
-    uint32_t down;    // k = 6: some row reaches below its own id (a DAG that keeps vertex ids)
+    uint32_t down;    // k >= 5: some row reaches below its own id (a DAG that keeps vertex ids)
 };
 
 // Bitmap-path roots of at most kLowMax out-neighbours run in a launch of their own, in blocks of 8 warps,
@@ -31,16 +31,18 @@ struct CountStats {
 // its barriers instead.  R-MAT 15, k = 6: 0.70 ms in one launch, 0.64 in two (0.79 with 4 warps).
 constexpr uint32_t kLowMax = 128;
 constexpr uint32_t kLowWarps = 8;
-// That launch needs kLowPerSlot such roots for every block of 8 warps that the chip holds: with fewer a
-// root is left to 8 warps while others idle, and what is a short launch of its own comes after the
-// tail of the other one.  40 roots of 99, k = 6,
-// ids kept: 2.4 ms in small blocks, 1.4 in large ones; R-MAT 15, k = 4: 0.22 ms against 0.31.
+// From k = 5 on that launch needs a root for every block of 8 warps that the chip holds, kLowIds times as
+// many in a DAG that keeps ids, whose sets are enumerated: with fewer a root is left to 8 warps while
+// others idle, and what is a short launch of its own comes after the tail of the other one.  40 roots of
+// 99, k = 6, ids kept: 2.4 ms in small blocks, 1.4 in large ones; 2,000 roots in rank order (R-MAT 14,
+// factor 8), k = 6: 0.41 against 0.43.  At k = 3 and 4 the build is most of the work and small blocks are
+// better with any number (R-MAT 12, k = 3: 99 us against 113).
 // Where the counting outweighs the rows' build, two launches end in two tails: from k = 7 on (R-MAT 15,
 // k = 8: 69 ms in one launch, 129 in two), and at k = 6 where sets are enumerated (a DAG that keeps ids, no
 // re-encoding; R-MAT 15, ids kept, 10.9 ms against 13.9).  There the small blocks are for graphs without
 // larger roots (200,000 vertices of degree 50, k = 6, ids kept: 1.8 ms against 3.5; k = 7: 1.7
 // against 3.3).
-constexpr uint32_t kLowSlotsPerSm = 4, kLowPerSlot = 4;
+constexpr uint32_t kLowSlotsPerSm = 4, kLowIds = 4;
 // Under a cap on the blocks, that launch's blocks hold up to kMaxTeams teams of 8 warps, each with roots
 // of its own: as many blocks of 8 warps as the cap's warps are spread over all SMs, and no block of
 // 32 warps of another stream finds an empty one.  114 blocks, 180,000 roots of at most 119, k = 4..6,
