@@ -6,7 +6,8 @@
 // (Sec. II, Sec. IV) in rank space, where every local subgraph of the counting phase is
 // upper-triangular.
 //
-// Six launches; no block waits on another, and only the scan waits on earlier tiles:
+// Eight launches (k_tile_rows of order.cu first, k_rl_fill_mid twice); no block waits on another, and only
+// the scan waits on earlier tiles:
 //   k_rl_prologue : rowlen[r] = 0 and perm[rank[u]] = u (the vertex of each rank);
 //   k_rl_keep     : one pass over the arcs, one chunk of 512 arcs per warp and no block-wide
 //                   barrier.  Per arc u->v the keep-test rank[v] > rank[u] (the 16 rank gathers
